@@ -19,7 +19,8 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
               "--expt-relaxed-constexpr", "-DNDEBUG"]
 SOURCES = ["rf_api.cu", "rf_kernels.cu", "rf_pattern.cu", "rf_tc.cu", "rf_fft.cu", "rf_batch.cu",
-           "rf_mlp.cu", "rf_persist.cu", "rf_fftwarp.cu"]
+           "rf_mlp.cu", "rf_persist.cu", "rf_fftwarp.cu", "rf_team.cu", "rf_team_elastic.cu",
+           "rf_team_plastic.cu", "rf_team_any.cu"]
 
 
 def _nvcc() -> str:

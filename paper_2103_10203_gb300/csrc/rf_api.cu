@@ -45,6 +45,7 @@ void init_attributes(int dev) {
   init_attributes_fft();
   init_attributes_persist();
   init_attributes_fftwarp();
+  init_attributes_team();
   g_attr_done[dev] = true;
 }
 
@@ -255,6 +256,7 @@ void free_pattern(rf_ctx* c) {
     ax->M = ax->K = ax->nMT = ax->nKC = 0;
   }
   c->fft_colmode = kColSeparate;
+  c->team_on = false;
   c->have_pattern = false;
   c->fields_valid = false;
 }
@@ -288,6 +290,7 @@ void release_pattern_buffers(rf_ctx* c) {
   dfree(c->d_jn);
   dfree(c->d_hk);
   dfree(c->d_bar);
+  dfree(c->d_fin);
   dfree(c->d_ptrace);
   c->pcap.clear();
 }
@@ -370,23 +373,45 @@ int init_status(rf_ctx* c, const double* macro, const int32_t* control = nullptr
   s.last_r = 0.0;
   s.rmin = HUGE_VAL;
   for (int i = 0; i < 6; ++i) s.ebar[i] = macro[i];
+  return RF_OK;
+}
+
+int upload_status(rf_ctx* c) {
   return ck(cudaMemcpyAsync(c->d_status, c->h_status, sizeof(Status), cudaMemcpyHostToDevice,
                             c->stream), "upload status");
 }
 
+bool team_solve(const rf_ctx* c) { return c->fft_colmode == kColPersistent && c->team_on; }
+
+// The status and the start coefficients of a solve on the device: a plain start (add = 0), or N v
+// added at the zero frequency (add = 1).
+int begin_solve(rf_ctx* c, const double* v, int add) {
+  if (team_solve(c)) return launch_team_begin(c, v, add);
+  if (int e = upload_status(c)) return e;
+  return launch_reset_er(c, v, add);
+}
+
 // Persistent 2D solve: one cooperative launch runs the updates; traced solves record the phase
 // stamps of every update (row phase, column phase, each up to its grid barrier).
-int run_persistent(rf_ctx* c) {
+// On the team kernels an untraced solve is followed at once by its final pass (which does nothing
+// after a solve that failed) and one wait for both.
+int run_persistent(rf_ctx* c, int commit) {
   const int cap = c->tracing ? std::min(c->opt.max_iter, 8192) : 0;
   if (cap > 0)
     if (int e = palloc(c, &c->d_ptrace, 3 * (size_t)cap, "trace")) return e;
   unsigned long long* tr = cap > 0 ? c->d_ptrace : nullptr;
+  const bool team = team_solve(c);
   if (int e = c->fft_colmode == kColPersistW ? launch_persist_warp(c, tr, cap)
+              : team                         ? launch_team_solve(c, tr, cap)
                                              : launch_persist_solve(c, tr, cap))
     return e;
-  if (int e = ck(cudaMemcpyAsync(c->h_status, c->d_status, sizeof(Status), cudaMemcpyDeviceToHost,
-                                 c->stream), "read status"))
+  if (team && !c->tracing) {
+    if (int e = launch_final(c, commit)) return e;   // leaves h_status and h_sbar
+    c->final_queued = true;
+  } else if (int e = ck(cudaMemcpyAsync(c->h_status, c->d_status, sizeof(Status),
+                                        cudaMemcpyDeviceToHost, c->stream), "read status")) {
     return e;
+  }
   if (int e = ck(cudaStreamSynchronize(c->stream), "persistent solve")) return e;
   c->launched_iters = c->h_status->iters;
   if (cap > 0) {
@@ -407,7 +432,8 @@ int run_persistent(rf_ctx* c) {
   return RF_OK;
 }
 
-int run_iterations(rf_ctx* c) {
+int run_iterations(rf_ctx* c, int commit) {
+  c->final_queued = false;
   const int maxchunk = c->opt.check_every > 0 ? c->opt.check_every : 32;
   int chunk = std::min(4, maxchunk);
   const bool persistent = c->fft_colmode == kColPersistent || c->fft_colmode == kColPersistW;
@@ -423,7 +449,7 @@ int run_iterations(rf_ctx* c) {
   }
   if (!persistent && !c->tracing) get_while_graph(c);
   if (persistent) {
-    if (int e = run_persistent(c)) return e;
+    if (int e = run_persistent(c, commit)) return e;
   } else if (!c->tracing && c->while_exec) {
     if (int e = ck(cudaGraphLaunch(c->while_exec, c->stream), "graph launch")) return e;
     if (int e = ck(cudaMemcpyAsync(c->h_status, c->d_status, sizeof(Status),
@@ -468,11 +494,14 @@ int run_iterations(rf_ctx* c) {
 }
 
 int finish(rf_ctx* c, int commit, double* sbar) {
-  if (int e = launch_final(c, commit)) return e;
-  if (int e = ck(cudaMemcpyAsync(c->h_sbar, c->d_sbar, 8 * sizeof(double),
-                                 cudaMemcpyDeviceToHost, c->stream), "read sbar"))
-    return e;
-  if (int e = ck(cudaStreamSynchronize(c->stream), "final pass")) return e;
+  if (!c->final_queued) {
+    if (int e = launch_final(c, commit)) return e;
+    if (int e = ck(cudaMemcpyAsync(c->h_sbar, c->d_sbar, 8 * sizeof(double),
+                                   cudaMemcpyDeviceToHost, c->stream), "read sbar"))
+      return e;
+    if (int e = ck(cudaStreamSynchronize(c->stream), "final pass")) return e;
+  }
+  c->final_queued = false;
   trace_collect(c, 0);
   c->fields_valid = true;
   if (commit) c->last_viol = c->h_sbar[6];
@@ -620,7 +649,7 @@ int rf_create(rf_ctx** out, const rf_grid* grid, int32_t n_phases, const rf_phas
     d.lam = (float)phases[p].lambda;
     d.mu = (float)phases[p].mu;
     d.plastic = phases[p].plastic ? 1 : 0;
-    d.sy = d.plastic ? (float)phases[p].sigma_y0 : 0.f;
+    d.sy = d.plastic ? (float)phases[p].sigma_y0 : 3.0e38f;   // no yield
     d.H = d.plastic ? (float)phases[p].hardening : 0.f;
     d.r3muH = d.plastic ? (float)(1.0 / (3.0 * phases[p].mu + phases[p].hardening)) : 0.f;
     any_plastic = any_plastic || d.plastic;
@@ -883,6 +912,7 @@ int rf_set_pattern(rf_ctx* c, const int32_t* freqs, int64_t K) {
     // half-pattern entries grouped by kx index (counting sort) for the fused column phase
     std::vector<int> jptr(c->Kx + 1, 0), jlist(std::max<long long>(c->Kh, 1));
     for (long long h = 0; h < c->Kh; ++h) ++jptr[c->h_hidx[h].j + 1];
+    c->h_jcount.assign(jptr.begin() + 1, jptr.end());
     for (int j = 0; j < c->Kx; ++j) jptr[j + 1] += jptr[j];
     std::vector<int> fill(jptr.begin(), jptr.end() - 1);
     for (long long h = 0; h < c->Kh; ++h) jlist[fill[c->h_hidx[h].j]++] = (int)h;
@@ -966,12 +996,13 @@ int rf_solve(rf_ctx* c, const double macro[6], const float* warm, double hom_str
     if (int e = ck(cudaMemsetAsync(c->d_ER, 0, sizeof(float2) * c->rect, c->stream), "memset"))
       return e;
     if (int e = launch_warm_project(c, c->d_warm, macro)) return e;
+    if (int e = team_solve(c) ? launch_team_begin(c, macro, 2) : upload_status(c)) return e;
     // the staging vector must outlive the copy
     if (int e = ck(cudaStreamSynchronize(c->stream), "warm")) return e;
   } else {
-    if (int e = launch_reset_er(c, macro, 0.0)) return e;
+    if (int e = begin_solve(c, macro, 0)) return e;
   }
-  int st = run_iterations(c);
+  int st = run_iterations(c, 0);
   if (st < 0) return st;
   if (int e = finish(c, 0, hom_stress)) return e;
   for (int i = 0; i < 6; ++i) {
@@ -1008,11 +1039,12 @@ int rf_solve_mixed(rf_ctx* c, const int32_t control[6], const double target[6], 
     if (int e = ck(cudaMemsetAsync(c->d_ER, 0, sizeof(float2) * c->rect, c->stream), "memset"))
       return e;
     if (int e = launch_warm_project(c, c->d_warm, E0)) return e;
+    if (int e = team_solve(c) ? launch_team_begin(c, E0, 2) : upload_status(c)) return e;
     if (int e = ck(cudaStreamSynchronize(c->stream), "warm")) return e;
   } else {
-    if (int e = launch_reset_er(c, E0, 0.0)) return e;
+    if (int e = begin_solve(c, E0, 0)) return e;
   }
-  int st = run_iterations(c);
+  int st = run_iterations(c, 0);
   if (st < 0) return st;
   double E[6];
   for (int i = 0; i < 6; ++i) E[i] = c->h_status->ebar[i];
@@ -1048,8 +1080,8 @@ int rf_solve_path_mixed(rf_ctx* c, const int32_t control[6], int32_t n_steps, co
     mixed_start(c, control, incr, d);
     mixed_start(c, control, t, E0);
     if (int e = init_status(c, E0, control, t)) return e;
-    if (int e = launch_reset_er(c, d, 1.0)) return e;
-    int st = run_iterations(c);
+    if (int e = begin_solve(c, d, 1)) return e;
+    int st = run_iterations(c, 1);
     if (st < 0) return st;
     double E[6];
     for (int i = 0; i < 6; ++i) E[i] = c->h_status->ebar[i];
@@ -1082,8 +1114,8 @@ int rf_solve_path(rf_ctx* c, int32_t n_steps, const double* path, double* hom_st
     double d[6];
     for (int i = 0; i < 6; ++i) d[i] = m[i] - c->prev_macro[i];
     if (int e = init_status(c, m)) return e;
-    if (int e = launch_reset_er(c, d, 1.0)) return e;
-    int st = run_iterations(c);
+    if (int e = begin_solve(c, d, 1)) return e;
+    int st = run_iterations(c, 1);
     if (st < 0) return st;
     if (int e = finish(c, 1, hom_stress ? hom_stress + 6 * n : nullptr)) return e;
     for (int i = 0; i < 6; ++i) {
@@ -1256,6 +1288,11 @@ int rf_get_info(const rf_ctx* c, rf_info* info) {
     info->fft_row_blocks = c->persist_G;
     info->fft_row_threads = c->persist_threads;
     info->fft_rows = (c->rows + c->persist_G - 1) / c->persist_G;
+    if (c->team_on) {
+      info->fft_row_blocks = c->team_G;
+      info->fft_row_threads = c->team_threads;
+      info->fft_rows = 2 * ((c->rows / 2 + c->team_G - 1) / c->team_G);
+    }
   }
   info->fft_row_warps = fft && c->fft_colmode != kColPersistent ? c->fft_row_warps : 0;
   info->reserved = 0;
@@ -1374,7 +1411,8 @@ int rf_compat(rf_ctx* c, double hom_stress[6]) {
     return e;
   if (int e = launch_scatter_full(c, f)) return e;
   if (int e = init_status(f, c->prev_macro)) return e;
-  const int st = run_iterations(f);
+  if (int e = team_solve(f) ? launch_team_begin(f, c->prev_macro, 2) : upload_status(f)) return e;
+  const int st = run_iterations(f, 0);
   if (st < 0) return st;
   double sbar[6];
   if (int e = finish(f, 0, sbar)) return e;

@@ -993,7 +993,8 @@ int fft_autotune(rf_ctx* c) {
       !colw_shape)
     return RF_OK;
   rf_ctx::Tuned& tu = c->tuned;
-  if (tu.valid && tu.Kx == c->Kx && tu.Ky == c->Ky && tu.Kz == c->Kz) {
+  if (tu.valid && tu.Kx == c->Kx && tu.Ky == c->Ky && tu.Kz == c->Kz &&
+      !(persist_auto && tu.team_on && !team_geometry(c, tu.team_cluster))) {
     // same transform shapes as the last tuning on this context: same choice
     if (!rows_pinned) {
       if (tu.row_blocks_balanced) set_rows_balanced(c, tu.row_blocks_balanced);
@@ -1014,7 +1015,10 @@ int fft_autotune(rf_ctx* c) {
       }
     }
     if (colw_shape) c->fft_colw_M = tu.colw_M;
-    if (persist_auto && tu.persist_per_sm > 0 &&
+    c->team_on = persist_auto && tu.team_on;
+    if (c->team_on && c->opt.fft_fuse == 0 && tu.colmode == kColPersistent)
+      c->fft_colmode = kColPersistent;
+    if (!c->team_on && persist_auto && tu.persist_per_sm > 0 &&
         persist_geometry(c, tu.persist_threads, tu.persist_per_sm)) {
       if (c->opt.fft_fuse == 0 && tu.colmode == kColPersistent) c->fft_colmode = kColPersistent;
     }
@@ -1258,9 +1262,32 @@ int fft_autotune(rf_ctx* c) {
     hs.mu0 = c->mu0;
     float best = 1e30f;
     int bestT = 0, bestK = 0;
+    // the team kernels where they take the sides (a co-resident grid, or one cluster of 8 or 16
+    // blocks), the general persistent kernel otherwise
+    int bestCl = -1;
+    c->team_on = true;
+    for (int cl : {0, 8, 16}) {
+      if (err || !team_geometry(c, cl)) continue;
+      float ms = 1e30f;
+      const int e = time_it([&] {
+        if (int e2 = launch_team_begin(c, hs.ebar, 2)) return e2;
+        return launch_team_solve(c, nullptr, 0);
+      }, &ms);
+      if (e) {
+        cudaGetLastError();
+        set_error("");
+        continue;
+      }
+      ms /= 3.f * kUpd;
+      if (ms < best) {
+        best = ms;
+        bestCl = cl;
+      }
+    }
+    c->team_on = bestCl >= 0 && team_geometry(c, bestCl);
     const int cand[4][2] = {{512, 2}, {256, 2}, {512, 1}, {256, 1}};
     for (const auto& cd : cand) {
-      if (err || !persist_geometry(c, cd[0], cd[1])) continue;
+      if (err || c->team_on || !persist_geometry(c, cd[0], cd[1])) continue;
       float ms = 1e30f;
       const int e = time_it([&] {
         if (int e2 = tck(cudaMemcpyAsync(c->d_status, c->h_status, sizeof(Status),
@@ -1280,8 +1307,8 @@ int fft_autotune(rf_ctx* c) {
         bestK = cd[1];
       }
     }
-    if (bestT > 0) {
-      persist_geometry(c, bestT, bestK);
+    if (bestT > 0 || c->team_on) {
+      if (!c->team_on) persist_geometry(c, bestT, bestK);
       if (c->opt.fft_fuse == 3 || best < t_np) c->fft_colmode = kColPersistent;
       else c->fft_colmode = mode_np;
     } else if (c->opt.fft_fuse == 3) {
@@ -1358,6 +1385,8 @@ int fft_autotune(rf_ctx* c) {
     tu.colmode = c->fft_colmode;
     tu.persist_per_sm = c->persist_per_sm;
     tu.persist_threads = c->persist_threads;
+    tu.team_on = c->team_on;
+    tu.team_cluster = c->team_cluster;
     tu.row_warps = c->fft_row_warps;
     tu.colw_M = c->fft_colw_M;
   }

@@ -27,6 +27,7 @@ namespace rfk {
 constexpr int kMaxPhases = 16;
 constexpr int kGammaBlock = 128;   // threads per Green-operator block (one frequency each)
 
+// sy: initial yield stress; beyond any stress for an elastic phase
 struct DevPhase {
   float lam, mu, sy, H;
   int plastic;
@@ -220,6 +221,13 @@ struct rf_ctx {
   // grid-barrier words, per-update phase stamps of traced solves
   int persist_G = 0, persist_threads = 512, persist_per_sm = 0;
   size_t persist_smem = 0;
+  // the persistent solve on team FFTs (rf_team.cu), used by kColPersistent where it is faster:
+  // blocks, and the same number when they form one cluster (0: a co-resident grid)
+  bool team_on = false;
+  int team_G = 0, team_cluster = 0, team_threads = 0;
+  bool final_queued = false;            // the final pass went out behind the solve (rf_team.cu)
+  double* d_fin = nullptr;              // [blocks][8] partials of the team solve's final pass
+  std::vector<int> h_jcount;            // pattern entries of each kx index
   unsigned* d_bar = nullptr;
   unsigned long long* d_ptrace = nullptr;
   int* d_jptr = nullptr;                // [Kx + 1] offsets of each kx's entries in d_jlist
@@ -234,6 +242,8 @@ struct rf_ctx {
     int row_blocks_balanced = 0;
     int colmode = 0;
     int persist_per_sm = 0, persist_threads = 0;
+    bool team_on = false;
+    int team_cluster = 0;
     int row_warps = 0, colw_M = 1;
   } tuned;
 
@@ -444,6 +454,13 @@ int launch_persist_solve(rf_ctx* c, unsigned long long* trace, int trace_cap);
 int launch_persist_final(rf_ctx* c, int commit);
 void init_attributes_persist();
 int persist_setup(rf_ctx* c);
+// rf_team.cu
+bool team_ok(const rf_ctx* c);
+bool team_geometry(rf_ctx* c, int cluster);
+void init_attributes_team();
+int launch_team_solve(rf_ctx* c, unsigned long long* trace, int trace_cap);
+int launch_team_begin(rf_ctx* c, const double* macro, int mode);
+int launch_team_final(rf_ctx* c, int commit);
 int launch_gamma_finalize(rf_ctx* c, int splits, const int* done);
 void trace_begin(rf_ctx* c, long long idx);
 void trace_stage(rf_ctx* c, int stage);

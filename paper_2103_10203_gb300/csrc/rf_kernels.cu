@@ -376,23 +376,39 @@ __global__ __launch_bounds__(kGammaBlock) void k_gamma(GammaArgs a, double Nd) {
   }
 }
 
-__global__ void k_reduce_sbar(const double* part, const double* vpart, int nb, double invN,
-                              double* out) {
-  __shared__ double sh[256];
-  for (int c = 0; c < 7; ++c) {
-    double s = 0.0;
-    for (int i = threadIdx.x; i < nb; i += 256)
-      s = (c < 6) ? s + part[i * 6 + c] : fmax(s, vpart[i]);
-    sh[threadIdx.x] = s;
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-      if (threadIdx.x < w)
-        sh[threadIdx.x] = (c < 6) ? sh[threadIdx.x] + sh[threadIdx.x + w]
-                                  : fmax(sh[threadIdx.x], sh[threadIdx.x + w]);
-      __syncthreads();
+// Sums of the six stress components' block partials and the largest violation, in a fixed order:
+// thread 8 r + c takes component c of the rows r, r + 128, ... (neighbouring threads read
+// neighbouring words, four loads in flight), then a tree over the rows. One block: the chain of
+// dependent loads bounds it, so all components go at once (seven passes of 256 threads over the
+// 128 partials of a 256^2 cell took longer than the launch).
+constexpr int kReduceThreads = 1024;
+
+__global__ __launch_bounds__(kReduceThreads) void k_reduce_sbar(const double* part,
+                                                                const double* vpart, int nb,
+                                                                double invN, double* out) {
+  __shared__ double sh[32][8];
+  const int c = threadIdx.x & 7, r = threadIdx.x >> 3;
+  constexpr int kRows = kReduceThreads / 8;
+  auto add = [&](double x, double y) { return c < 6 ? x + y : fmax(x, y); };
+  double s = 0.0;
+  for (int i0 = r; i0 < nb; i0 += 4 * kRows) {
+    double v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int i = i0 + u * kRows;
+      v[u] = (i < nb && c < 7) ? (c < 6 ? part[(long long)i * 6 + c] : vpart[i]) : 0.0;
     }
-    if (threadIdx.x == 0) out[c] = (c < 6) ? sh[0] * invN : sh[0];
-    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < 4; ++u) s = add(s, v[u]);
+  }
+  s = add(s, __shfl_down_sync(0xffffffffu, s, 16));
+  s = add(s, __shfl_down_sync(0xffffffffu, s, 8));
+  if ((threadIdx.x & 31) < 8) sh[threadIdx.x >> 5][c] = s;
+  __syncthreads();
+  if (threadIdx.x < 7) {
+    double t = sh[0][c];
+    for (int w = 1; w < kReduceThreads / 32; ++w) t = add(t, sh[w][c]);
+    out[c] = c < 6 ? t * invN : t;
   }
 }
 
@@ -904,11 +920,15 @@ int launch_final(rf_ctx* c, int commit) {
   c->tracing = false;   // the whole final pass is one stage
   if (c->opt.transform == RF_TRANSFORM_FFT && c->fft_colmode == kColPersistent) {
     // the persistent solve leaves the strain lines of the final coefficients in its layout
-    const int ie = launch_persist_final(c, commit);
+    const int ie = c->team_on ? launch_team_final(c, commit) : launch_persist_final(c, commit);
     c->tracing = tr;
     if (ie) return ie;
-    k_reduce_sbar<<<1, 256, 0, c->stream>>>(c->d_sbar_part, c->d_viol_part, c->persist_G,
-                                            1.0 / (double)c->N, c->d_sbar);
+    if (c->team_on) {   // its last block leaves the sums
+      trace_end(c);
+      return RF_OK;
+    }
+    k_reduce_sbar<<<1, kReduceThreads, 0, c->stream>>>(c->d_sbar_part, c->d_viol_part, c->persist_G,
+                                                       1.0 / (double)c->N, c->d_sbar);
     int e = launch_check(c, "reduce_sbar");
     trace_end(c);
     return e;
@@ -918,8 +938,8 @@ int launch_final(rf_ctx* c, int commit) {
     if (!ie) ie = launch_fft_row(c, nullptr, true, commit);
     c->tracing = tr;
     if (ie) return ie;
-    k_reduce_sbar<<<1, 256, 0, c->stream>>>(c->d_sbar_part, c->d_viol_part, c->fft_blocks,
-                                            1.0 / (double)c->N, c->d_sbar);
+    k_reduce_sbar<<<1, kReduceThreads, 0, c->stream>>>(c->d_sbar_part, c->d_viol_part,
+                                                       c->fft_blocks, 1.0 / (double)c->N, c->d_sbar);
     int e = launch_check(c, "reduce_sbar");
     trace_end(c);
     return e;
@@ -935,8 +955,8 @@ int launch_final(rf_ctx* c, int commit) {
   ra.viol_part = c->d_viol_part;
   ra.commit = commit;
   if (int e = row_dispatch(c, ra, true)) return e;
-  k_reduce_sbar<<<1, 256, 0, c->stream>>>(c->d_sbar_part, c->d_viol_part, c->row_blocks,
-                                          1.0 / (double)c->N, c->d_sbar);
+  k_reduce_sbar<<<1, kReduceThreads, 0, c->stream>>>(c->d_sbar_part, c->d_viol_part, c->row_blocks,
+                                                     1.0 / (double)c->N, c->d_sbar);
   int e = launch_check(c, "reduce_sbar");
   trace_end(c);
   return e;

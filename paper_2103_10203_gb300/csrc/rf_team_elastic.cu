@@ -1,0 +1,18 @@
+// The persistent 2D solve on team FFTs (rf_team.cuh) for square cells, elastic phases.
+#include "rf_team.cuh"
+
+namespace rfk {
+namespace team {
+
+Kernel kernel_elastic(int side) {
+  switch (side) {
+#define X(L, R, M) \
+  case L: return k_team2d<L, false>;
+    RF_TEAM_SIDES(X)
+#undef X
+  }
+  return nullptr;
+}
+
+}  // namespace team
+}  // namespace rfk
