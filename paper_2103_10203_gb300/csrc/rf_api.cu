@@ -46,6 +46,7 @@ void init_attributes(int dev) {
   init_attributes_persist();
   init_attributes_fftwarp();
   init_attributes_team();
+  init_attributes_fft3();
   g_attr_done[dev] = true;
 }
 
@@ -291,6 +292,8 @@ void release_pattern_buffers(rf_ctx* c) {
   dfree(c->d_hk);
   dfree(c->d_bar);
   dfree(c->d_fin);
+  dfree(c->d_zrange);
+  dfree(c->d_ymap);
   dfree(c->d_ptrace);
   c->pcap.clear();
 }
@@ -442,8 +445,12 @@ int run_iterations(rf_ctx* c, int commit) {
     // first one needs the line transforms of the start coefficients
     const bool tr = c->tracing;
     c->tracing = false;
-    const int e = c->fft_colmode == kColWarp ? launch_fft_coly_init_warp(c)
-                                             : fft_inverse_stages(c, nullptr);
+    int e = RF_OK;
+    if (c->fft_colmode == kColZ) {   // their updates begin with the inverse along y
+      e = launch_fft3_z(c, false, nullptr);
+    } else {
+      e = c->fft_colmode == kColWarp ? launch_fft_coly_init_warp(c) : fft_inverse_stages(c, nullptr);
+    }
     c->tracing = tr;
     if (e) return e;
   }
@@ -905,7 +912,8 @@ int rf_set_pattern(rf_ctx* c, const int32_t* freqs, int64_t K) {
   if (!err)
     err = palloc(c, &c->d_part,
                  (size_t)std::max<long long>((c->Kh + kGammaBlock - 1) / kGammaBlock,
-                                             (long long)c->nc * c->Kx),
+                                             (long long)std::max(c->nc, c->dim == 3 ? c->Ky : 1) *
+                                                 c->Kx),
                  "partials");
   const bool fuse_ok = c->opt.transform == RF_TRANSFORM_FFT && c->dim == 2 && c->opt.fft_fuse >= 0;
   if (!err && fuse_ok) {
@@ -950,6 +958,7 @@ int rf_set_pattern(rf_ctx* c, const int32_t* freqs, int64_t K) {
     if (pe && c->opt.fft_fuse == 3) err = pe;
     else if (pe) set_error("");
   }
+  if (!err && c->opt.transform == RF_TRANSFORM_FFT) err = fft3_setup(c, kym.data());
   if (!err && c->opt.precision != RF_PREC_FP32) err = tc_setup(c);
   if (!err) err = ck(cudaMemsetAsync(c->d_OUT, 0, sizeof(float2) * splits * c->rect, c->stream), "memset");
   if (!err && c->opt.transform == RF_TRANSFORM_FFT) err = fft_autotune(c);
@@ -1278,7 +1287,7 @@ int rf_get_info(const rf_ctx* c, rf_info* info) {
   info->fft_row_threads = fft ? c->fft_row_threads : 0;
   info->fft_cols = fft ? c->fft_C : 0;
   info->fft_col_threads = fft ? c->fft_col_threads : 0;
-  info->fft_fused = c->fft_colmode;
+  info->fft_fused = c->fft_colmode == kColZ ? kColSeparate : c->fft_colmode;   // 2D modes
   info->fft_fuse_kx = c->fft_colmode == kColFused ? c->fft_M
                       : (c->fft_colmode == kColWarp || c->fft_colmode == kColPersistW)
                           ? c->fft_colw_M : 0;

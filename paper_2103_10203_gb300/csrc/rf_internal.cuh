@@ -214,7 +214,8 @@ struct rf_ctx {
   // (kColGreenInv); 4 as 1 with a warp per line column, the transforms in registers and the
   // line coefficients in kx slabs (kColWarp, 1024 x 1024, warp-FFT row kernel); 5 the
   // persistent solve on the same passes (kColPersistW). Modes 1, 2 and 4 start a solve with one
-  // inverse y of the start coefficients (3 and 5 inside their launch).
+  // inverse y of the start coefficients (3 and 5 inside their launch). 3D: 0, or 6 the updates on
+  // team FFTs (kColZ), which start with the inverse along z.
   int fft_colmode = 0;
   int fft_M = 1, fft_M_threads = 256;   // kx columns and threads per fused block
   // persistent 2D solve (column mode kColPersistent): grid, block size, dynamic shared memory,
@@ -228,6 +229,8 @@ struct rf_ctx {
   bool final_queued = false;            // the final pass went out behind the solve (rf_team.cu)
   double* d_fin = nullptr;              // [blocks][8] partials of the team solve's final pass
   std::vector<int> h_jcount;            // pattern entries of each kx index
+  int2* d_zrange = nullptr;             // 3D on team FFTs: entries of each (ky, kx) ...
+  short* d_ymap = nullptr;              // ... and the rectangle row of each position along y
   unsigned* d_bar = nullptr;
   unsigned long long* d_ptrace = nullptr;
   int* d_jptr = nullptr;                // [Kx + 1] offsets of each kx's entries in d_jlist
@@ -447,13 +450,20 @@ int launch_tc_axis(rf_ctx* c, const TcAxis& ax, const float2* in, int in_splits,
 int launch_fft_green_inv(rf_ctx* c, const int* done);
 int launch_gather_jentries(rf_ctx* c);
 constexpr int kColSeparate = 0, kColFused = 1, kColGreenInv = 2, kColPersistent = 3,
-              kColWarp = 4, kColPersistW = 5;
+              kColWarp = 4, kColPersistW = 5, kColZ = 6;
 // rf_persist.cu
 bool persist_geometry(rf_ctx* c, int threads, int per_sm);
 int launch_persist_solve(rf_ctx* c, unsigned long long* trace, int trace_cap);
 int launch_persist_final(rf_ctx* c, int commit);
 void init_attributes_persist();
 int persist_setup(rf_ctx* c);
+// rf_fft3.cu: 3D updates on team FFTs (column mode kColZ)
+bool fft3_ok(const rf_ctx* c);
+int fft3_setup(rf_ctx* c, const int* kym);
+void init_attributes_fft3();
+int launch_fft3_row(rf_ctx* c, const int* done, bool final_pass, int commit, int* blocks);
+int launch_fft3_y(rf_ctx* c, int sign, const int* done);
+int launch_fft3_z(rf_ctx* c, bool full, const int* done);
 // rf_team.cu
 bool team_ok(const rf_ctx* c);
 bool team_geometry(rf_ctx* c, int cluster);

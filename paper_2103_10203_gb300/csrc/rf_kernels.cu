@@ -834,6 +834,18 @@ int launch_iteration(rf_ctx* c) {
     if (int e = launch_fft_row(c, done, false, 0)) return e;
     return launch_fft_colphase_warp(c, done);
   }
+  if (fftm && c->fft_colmode == kColZ) {
+    trace_stage(c, 1);
+    if (int e = launch_fft3_y(c, +1, done)) return e;
+    trace_stage(c, 2);
+    if (int e = launch_fft3_row(c, done, false, 0, nullptr)) return e;
+    trace_stage(c, 3);
+    if (int e = launch_fft3_y(c, -1, done)) return e;
+    trace_stage(c, 6);
+    const int e = launch_fft3_z(c, true, done);
+    trace_end(c);
+    return e;
+  }
   if (fftm && c->fft_colmode == kColGreenInv) {
     // row pass, forward y, then the Green operator + decision inside the inverse y kernel
     trace_stage(c, 2);
@@ -928,6 +940,19 @@ int launch_final(rf_ctx* c, int commit) {
       return RF_OK;
     }
     k_reduce_sbar<<<1, kReduceThreads, 0, c->stream>>>(c->d_sbar_part, c->d_viol_part, c->persist_G,
+                                                       1.0 / (double)c->N, c->d_sbar);
+    int e = launch_check(c, "reduce_sbar");
+    trace_end(c);
+    return e;
+  }
+  if (c->opt.transform == RF_TRANSFORM_FFT && c->fft_colmode == kColZ) {
+    // the last z phase left the final coefficients transformed along z
+    int blocks = 0;
+    int ie = launch_fft3_y(c, +1, nullptr);
+    if (!ie) ie = launch_fft3_row(c, nullptr, true, commit, &blocks);
+    c->tracing = tr;
+    if (ie) return ie;
+    k_reduce_sbar<<<1, kReduceThreads, 0, c->stream>>>(c->d_sbar_part, c->d_viol_part, blocks,
                                                        1.0 / (double)c->N, c->d_sbar);
     int e = launch_check(c, "reduce_sbar");
     trace_end(c);

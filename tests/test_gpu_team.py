@@ -1,5 +1,5 @@
 """The kernels on team FFTs (several threads per transform, sizes fixed at compile time): the
-persistent 2D solve, at every side it takes, against the oracle.
+persistent 2D solve and the 3D updates, at every side they take, against the oracle.
 
 Tolerances as in test_gpu_parity.py: relative L2 error of fields and coefficients 1e-5 (FP32
 transforms of at most 512 points: some ten roundings of 2^-24 per pass, three passes per
@@ -104,3 +104,49 @@ def test_persistent_solve_continues_after_divergence(lib):
     with pytest.raises(lib.RFError):
         s.rf_get_fields()
     s.close()
+
+
+def check3(lib, pm, phases, pat, macro, n=3, **opts):
+    """The 3D updates (stage "column_phase" is theirs alone in 3D), traced and untraced."""
+    check(lib, pm, phases, pat, macro, n, **opts)
+    s = lib.Solver(pm, phases, pattern=pat, tol=0.0, max_iter=n, transform="fft", **opts)
+    s.rf_set_tracing(True)
+    s.rf_solve(macro)
+    ran = s.rf_get_stage_times()["column_phase"][1]
+    s.close()
+    return ran == n
+
+
+SIDES3 = [(32, 48, 64), (48, 96, 32), (96, 64, 48), (64, 32, 96), (32, 32, 128), (32, 128, 32),
+          (128, 32, 32), (192, 32, 32), (32, 192, 32), (32, 32, 192), (256, 32, 32), (32, 256, 32),
+          (32, 32, 256), (384, 32, 32), (32, 384, 32), (32, 32, 384), (512, 32, 32), (32, 512, 32),
+          (32, 32, 512)]
+
+
+@pytest.mark.parametrize("shape", SIDES3)
+def test_3d_updates_sides(lib, shape):
+    """Every side along every axis; ragged groups of kx and rows included."""
+    pm = blocks(shape, sum(shape))
+    pat = O.pattern_adapted(pm, 1, k_target(0.03, pm.size))
+    check3(lib, pm, elastic_phases(), pat, np.array([0.01, -0.004, 0.002, 0.001, 0.003, -0.002]))
+
+
+@pytest.mark.parametrize("shape", [(32, 48, 64), (64, 64, 64), (96, 32, 32)])
+def test_3d_updates_plastic(lib, shape):
+    pm = blocks(shape, 11)
+    pat = O.pattern_adapted(pm, 1, k_target(0.03, pm.size))
+    check3(lib, pm, j2_phases(), pat, np.array([0.015, -0.004, 0.002, 0.001, 0.003, -0.002]))
+
+
+def test_3d_updates_full_set(lib):
+    pm = blocks((32, 48, 32), 2)
+    check3(lib, pm, elastic_phases(), full_pattern(pm.shape), np.array([0.01, 0, 0, 0, 0.002, 0]))
+
+
+def test_3d_updates_are_the_ones_that_run(lib):
+    """At a size where their advantage is large the tuner takes them; pinned modes do not."""
+    pm = random_discs(64, (6.0, 10.0), 0.3, 5)[None].repeat(64, 0)
+    pat = O.pattern_adapted(pm, 1, k_target(0.02, pm.size))
+    macro = np.array([0.01, 0, 0, 0.002, 0, 0])
+    assert check3(lib, pm, elastic_phases(), pat, macro)
+    assert not check3(lib, pm, elastic_phases(), pat, macro, fft_fuse=-1)
