@@ -21,7 +21,7 @@ NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompil
 SOURCES = ["rf_api.cu", "rf_kernels.cu", "rf_pattern.cu", "rf_tc.cu", "rf_fft.cu", "rf_batch.cu",
            "rf_mlp.cu", "rf_persist.cu", "rf_fftwarp.cu", "rf_team.cu", "rf_team_elastic.cu",
            "rf_team_plastic.cu", "rf_team_any.cu", "rf_fft3.cu", "rf_fft3_row_elastic.cu",
-           "rf_fft3_row_plastic.cu", "rf_fft3_col.cu"]
+           "rf_fft3_row_plastic.cu", "rf_fft3_col.cu", "rf_dft.cu"]
 
 
 def _nvcc() -> str:

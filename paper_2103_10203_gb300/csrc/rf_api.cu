@@ -47,6 +47,7 @@ void init_attributes(int dev) {
   init_attributes_fftwarp();
   init_attributes_team();
   init_attributes_fft3();
+  init_attributes_dft();
   g_attr_done[dev] = true;
 }
 
@@ -293,6 +294,8 @@ void release_pattern_buffers(rf_ctx* c) {
   dfree(c->d_bar);
   dfree(c->d_fin);
   dfree(c->d_zrange);
+  dfree(c->d_Wi);
+  dfree(c->d_Wf);
   dfree(c->d_ymap);
   dfree(c->d_ptrace);
   c->pcap.clear();
@@ -862,20 +865,6 @@ int rf_set_pattern(rf_ctx* c, const int32_t* freqs, int64_t K) {
   const int NCK = c->nc * c->Kx;
   c->rect = (long long)c->Kz * c->Ky * NCK;
   c->zero_base_idx = ((long long)(pos(zs, 0) * c->Ky + pos(ys, 0)) * c->nc) * c->Kx + pos(xs, 0);
-  // split-K for the forward transforms so that the grid covers the GPU
-  int sms = 152;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->dev);
-  if (c->dim == 2) {
-    const long long blocks = (long long)((NCK + 63) / 64) * ((c->Ky + 31) / 32);
-    c->splitB = (int)std::max(1LL, std::min<long long>((2LL * sms + blocks - 1) / blocks,
-                                                        std::max(1, c->ny / 64)));
-    c->splitC = 1;
-  } else {
-    c->splitB = 1;
-    const long long blocks = (long long)((c->Ky * NCK + 63) / 64) * ((c->Kz + 31) / 32);
-    c->splitC = (int)std::max(1LL, std::min<long long>((2LL * sms + blocks - 1) / blocks,
-                                                        std::max(1, c->nz / 64)));
-  }
   // row kernel geometry
   c->row_R = std::max(1, std::min(16, 2048 / c->nx));
   auto smem_for = [&](int R) {
@@ -889,12 +878,8 @@ int rf_set_pattern(rf_ctx* c, const int32_t* freqs, int64_t K) {
   c->row_blocks = (c->rows + c->row_R - 1) / c->row_R;
   if (c->opt.transform == RF_TRANSFORM_FFT) {
     if (int e = fft_geometry(c)) return e;
-    c->splitB = c->splitC = 1;
   }
-  // the split-precision modes run the y and z transforms on the tensor cores, one output slice
-  if (c->opt.precision != RF_PREC_FP32) c->splitB = c->splitC = 1;
   const int part_blocks = std::max(c->row_blocks, c->rows);   // any FFT row tile (R >= 1)
-  const int splits = std::max(c->splitB, c->splitC);
   int err = palloc(c, &c->d_kx, c->Kx, "pattern");
   if (!err) err = palloc(c, &c->d_kym, c->Ky, "pattern");
   if (!err) err = palloc(c, &c->d_kzm, c->Kz, "pattern");
@@ -906,7 +891,7 @@ int rf_set_pattern(rf_ctx* c, const int32_t* freqs, int64_t K) {
   if (!err) err = palloc(c, &c->d_T1p, (size_t)c->rows * NCK, "line transforms");
   if (!err && c->dim == 3) err = palloc(c, &c->d_T2, (size_t)c->nz * c->Ky * NCK, "line transforms");
   if (!err && c->dim == 3) err = palloc(c, &c->d_T2f, (size_t)c->nz * c->Ky * NCK, "line transforms");
-  if (!err) err = palloc(c, &c->d_OUT, (size_t)splits * c->rect, "partials");
+  if (!err) err = palloc(c, &c->d_OUT, c->rect, "coefficients");
   // block partials of the convergence measure: Green kernel blocks, or column blocks of the
   // fused modes (<= NC Kx)
   if (!err)
@@ -959,8 +944,10 @@ int rf_set_pattern(rf_ctx* c, const int32_t* freqs, int64_t K) {
     else if (pe) set_error("");
   }
   if (!err && c->opt.transform == RF_TRANSFORM_FFT) err = fft3_setup(c, kym.data());
+  c->dft_U = 0;
+  if (!err && c->opt.transform == RF_TRANSFORM_DFT) err = dft_setup(c);
   if (!err && c->opt.precision != RF_PREC_FP32) err = tc_setup(c);
-  if (!err) err = ck(cudaMemsetAsync(c->d_OUT, 0, sizeof(float2) * splits * c->rect, c->stream), "memset");
+  if (!err) err = ck(cudaMemsetAsync(c->d_OUT, 0, sizeof(float2) * c->rect, c->stream), "memset");
   if (!err && c->opt.transform == RF_TRANSFORM_FFT) err = fft_autotune(c);
   if (!err) err = ck(cudaStreamSynchronize(c->stream), "pattern setup");
   if (!err) {

@@ -1081,7 +1081,7 @@ int fft_autotune(rf_ctx* c) {
     if (int e = fft_inverse_stages(c, nullptr)) return e;
     if (int e = launch_fft_row(c, nullptr, false, 0)) return e;
     if (int e = fft_forward_stages(c, nullptr)) return e;
-    return launch_gamma_finalize(c, 1, nullptr);
+    return launch_gamma_finalize(c, nullptr);
   };
   if (!err && !rows_pinned) {
     // uniform tiles of R rows, and balanced partitions over k blocks per SM
@@ -1193,7 +1193,7 @@ int fft_autotune(rf_ctx* c) {
       float sep = 1e30f, gi = 1e30f;
       err = time_it([&] {
         if (int e = fft_forward_stages(c, nullptr)) return e;
-        if (int e = launch_gamma_finalize(c, 1, nullptr)) return e;
+        if (int e = launch_gamma_finalize(c, nullptr)) return e;
         return fft_inverse_stages(c, nullptr);
       }, &sep);
       if (!err)

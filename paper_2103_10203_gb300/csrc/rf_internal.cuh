@@ -9,7 +9,7 @@
 //                                distinct values; entries outside the pattern stay zero
 //   T1, T1p  float2 [rows][NC][Kx]   per grid row (y, z): line transforms along x
 //   T2       float2 [Nz][Ky][NC][Kx] (3D) line transforms along y
-//   OUT      float2 [S][Kz][Ky][NC][Kx] split-K partial sums of the forward transform
+//   OUT      float2 [Kz][Ky][NC][Kx] forward transform on the rectangle
 // NC = 3 (11, 22, 12) in 2D plane strain, 6 (11, 22, 33, 23, 13, 12) in 3D.
 #pragma once
 
@@ -75,24 +75,6 @@ struct Status {
 constexpr double kDivergeRatio = 1e4;
 constexpr double kDivergeFloor = 1e-3;
 
-struct DftAxisArgs {
-  const float2* in;
-  long long in_split_stride;
-  int in_splits;
-  long long in_bstride;
-  float2* out;
-  long long out_split_stride;
-  int out_splits;
-  long long out_bstride;
-  int M, N, K, batch;
-  const int* mvals;   // nullable: m itself; values reduced to [0, L)
-  const int* kvals;   // nullable: k itself
-  const float2* table;  // exp(+2 pi i t / L), t in [0, L)
-  int L;
-  int sign;           // +1 inverse, -1 forward
-  const int* done;    // nullable early-exit flag
-};
-
 struct RowArgs {
   const float2* T;      // [rows][NC][Kx]
   float2* Tout;         // [rows][NC][Kx]
@@ -115,8 +97,6 @@ struct RowArgs {
 
 struct GammaArgs {
   const float2* OUT;
-  int splits;
-  long long split_stride;
   float2* ER;
   const HIdx* hidx;
   const float4* hn;     // unit wave vector (x, y, z) and multiplicity in w
@@ -131,6 +111,7 @@ struct GammaArgs {
   // while-loop graph: the last block clears the loop condition when it sets done
   cudaGraphConditionalHandle cond;
   int use_cond;
+  int early;            // let the next kernel start its prologue
 };
 
 }  // namespace rfk
@@ -177,7 +158,6 @@ struct rf_ctx {
   float2* d_T2 = nullptr;
   float2* d_T2f = nullptr;
   float2* d_OUT = nullptr;
-  int splitB = 1, splitC = 1;
   long long rect = 0;             // Kz*Ky*NC*Kx
   float2* d_twx = nullptr;
   float2* d_twy = nullptr;
@@ -229,6 +209,9 @@ struct rf_ctx {
   bool final_queued = false;            // the final pass went out behind the solve (rf_team.cu)
   double* d_fin = nullptr;              // [blocks][8] partials of the team solve's final pass
   std::vector<int> h_jcount;            // pattern entries of each kx index
+  float2* d_Wi = nullptr;               // pruned DFT along x (rf_dft.cu): twiddles [Kx][np], ...
+  float2* d_Wf = nullptr;               // ... [np][Kx], and units per block (0: general kernel)
+  int dft_U = 0;
   int2* d_zrange = nullptr;             // 3D on team FFTs: entries of each (ky, kx) ...
   short* d_ymap = nullptr;              // ... and the rectangle row of each position along y
   unsigned* d_bar = nullptr;
@@ -382,6 +365,12 @@ __device__ inline void decide(const double* part, int n, Status* st, double* sh)
 // the wait returns at once.
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// Lets the next kernel of the chain start its prologue now. Only for grids that leave room for it:
+// where the running grid fills the chip, waiting blocks would take slots from blocks still to come.
+__device__ __forceinline__ void grid_dep_launch() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
                               cudaStream_t st, Args... args) {
@@ -457,6 +446,13 @@ int launch_persist_solve(rf_ctx* c, unsigned long long* trace, int trace_cap);
 int launch_persist_final(rf_ctx* c, int commit);
 void init_attributes_persist();
 int persist_setup(rf_ctx* c);
+// rf_dft.cu
+int dft_setup(rf_ctx* c);
+void init_attributes_dft();
+int launch_row_dft(rf_ctx* c, const int* done, bool final_pass, int commit, int* blocks);
+int launch_axis_dft(rf_ctx* c, const float2* in, long long in_bs, float2* out, long long out_bs,
+                    int L, int N, int S, int batch, const int* vals, const float2* table, int sign,
+                    const int* done);
 // rf_fft3.cu: 3D updates on team FFTs (column mode kColZ)
 bool fft3_ok(const rf_ctx* c);
 int fft3_setup(rf_ctx* c, const int* kym);
@@ -471,7 +467,7 @@ void init_attributes_team();
 int launch_team_solve(rf_ctx* c, unsigned long long* trace, int trace_cap);
 int launch_team_begin(rf_ctx* c, const double* macro, int mode);
 int launch_team_final(rf_ctx* c, int commit);
-int launch_gamma_finalize(rf_ctx* c, int splits, const int* done);
+int launch_gamma_finalize(rf_ctx* c, const int* done);
 void trace_begin(rf_ctx* c, long long idx);
 void trace_stage(rf_ctx* c, int stage);
 void trace_end(rf_ctx* c);

@@ -76,77 +76,6 @@ __global__ void k_hinfo(const int* hk, long long Kh, int nx, int ny, int nz, int
 }
 
 // ------------------------------------------------------------------------------------------
-// line transform along one axis as a batched complex product with generated twiddles:
-//   out[s][b][m][n] = sum_{k in split s} w(m, k) * (sum_t in[t][b][k][n]),
-//   w(m, k) = exp(sign * 2 pi i * (mv(m) * kv(k) mod L) / L).
-// Block: 64 n-columns x 32 m-rows, 256 threads, k staged through shared memory in tiles of 32.
-template <int MT>
-__global__ __launch_bounds__(256) void k_dft_axis(DftAxisArgs a) {
-  if (a.done && *a.done) return;
-  __shared__ float2 xs[32][64];
-  __shared__ float2 ws[4 * MT][33];
-  const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * 64 + tx;
-  const int n0 = blockIdx.x * 64, m0 = blockIdx.y * (4 * MT);
-  const int b = blockIdx.z / a.out_splits, s = blockIdx.z % a.out_splits;
-  int kchunk = (a.K + a.out_splits - 1) / a.out_splits;
-  kchunk = (kchunk + 31) & ~31;
-  const int kbeg = s * kchunk;
-  const int kend = min(a.K, kbeg + kchunk);
-  float accr[MT], acci[MT];
-#pragma unroll
-  for (int i = 0; i < MT; ++i) accr[i] = acci[i] = 0.f;
-  const float2* inb = a.in + (long long)b * a.in_bstride;
-  for (int kb = kbeg; kb < kend; kb += 32) {
-    for (int i = tid; i < 32 * 64; i += 256) {
-      int kk = i >> 6, nn = i & 63;
-      int k = kb + kk, n = n0 + nn;
-      float2 v = make_float2(0.f, 0.f);
-      if (k < kend && n < a.N) {
-        const float2* p = inb + (long long)k * a.N + n;
-        for (int t = 0; t < a.in_splits; ++t) {
-          float2 u = p[t * a.in_split_stride];
-          v.x += u.x;
-          v.y += u.y;
-        }
-      }
-      xs[kk][nn] = v;
-    }
-    for (int i = tid; i < 4 * MT * 32; i += 256) {
-      int mm = i >> 5, kk = i & 31;
-      int m = m0 + mm, k = kb + kk;
-      float2 w = make_float2(0.f, 0.f);
-      if (m < a.M && k < kend) {
-        int mv = a.mvals ? a.mvals[m] : m;
-        int kv = a.kvals ? a.kvals[k] : k;
-        w = a.table[(int)(((long long)mv * kv) % a.L)];
-        if (a.sign < 0) w.y = -w.y;
-      }
-      ws[mm][kk] = w;
-    }
-    __syncthreads();
-#pragma unroll 4
-    for (int kk = 0; kk < 32; ++kk) {
-      float2 x = xs[kk][tx];
-#pragma unroll
-      for (int i = 0; i < MT; ++i) {
-        float2 w = ws[ty * MT + i][kk];
-        accr[i] = fmaf(w.x, x.x, fmaf(-w.y, x.y, accr[i]));
-        acci[i] = fmaf(w.x, x.y, fmaf(w.y, x.x, acci[i]));
-      }
-    }
-    __syncthreads();
-  }
-  const int n = n0 + tx;
-  if (n >= a.N) return;
-  float2* ob = a.out + (long long)s * a.out_split_stride + (long long)b * a.out_bstride;
-#pragma unroll
-  for (int i = 0; i < MT; ++i) {
-    int m = m0 + ty * MT + i;
-    if (m < a.M) ob[(long long)m * a.N + n] = make_float2(accr[i], acci[i]);
-  }
-}
-
-// ------------------------------------------------------------------------------------------
 // constitutive law: rf_law.cuh
 
 // ------------------------------------------------------------------------------------------
@@ -305,6 +234,7 @@ __global__ __launch_bounds__(kGammaBlock) void k_gamma(GammaArgs a, double Nd) {
     hi = a.hidx[h];
     n = a.hn[h];
   }
+  if (a.early) grid_dep_launch();
   grid_dep_wait();
   // the update's inputs are loaded together with the flag (they are discarded if it is set)
   const int dn = a.done ? __ldcg(a.done) : 0;
@@ -322,14 +252,6 @@ __global__ __launch_bounds__(kGammaBlock) void k_gamma(GammaArgs a, double Nd) {
   if (dn) return;
   float diff = 0.f;
   if (act) {
-    for (int s = 1; s < a.splits; ++s) {
-#pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        const float2 u = out[s * a.split_stride + c * a.Kx];
-        tv[c].x += u.x;
-        tv[c].y += u.y;
-      }
-    }
     float er[NC], ei[NC];
     const double* eb = a.st->ebar;
     double em[6];
@@ -487,35 +409,6 @@ static int launch_check(rf_ctx* c, const char* what) {
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, what);
   return RF_OK;
-}
-
-static int dft(rf_ctx* c, const float2* in, int in_splits, long long in_split_stride,
-               long long in_bstride, float2* out, int out_splits, long long out_split_stride,
-               long long out_bstride, int M, int N, int K, int batch, const int* mvals,
-               const int* kvals, const float2* tab, int L, int sign, const int* done) {
-  DftAxisArgs a;
-  a.in = in;
-  a.in_splits = in_splits;
-  a.in_split_stride = in_split_stride;
-  a.in_bstride = in_bstride;
-  a.out = out;
-  a.out_splits = out_splits;
-  a.out_split_stride = out_split_stride;
-  a.out_bstride = out_bstride;
-  a.M = M;
-  a.N = N;
-  a.K = K;
-  a.batch = batch;
-  a.mvals = mvals;
-  a.kvals = kvals;
-  a.table = tab;
-  a.L = L;
-  a.sign = sign;
-  a.done = done;
-  dim3 block(64, 4);
-  dim3 grid((N + 63) / 64, (M + 31) / 32, batch * out_splits);
-  k_dft_axis<8><<<grid, block, 0, c->stream>>>(a);
-  return launch_check(c, "dft_axis");
 }
 
 // twiddle buffers of fftc::table_len(n) entries per axis: plain table, then stage-major table
@@ -784,18 +677,16 @@ static int row_dispatch(rf_ctx* c, const RowArgs& a, bool final_pass) {
   return pl ? row_launch<6, true, false>(c, a) : row_launch<6, false, false>(c, a);
 }
 
-int launch_gamma_finalize(rf_ctx* c, int splits, const int* done);
+int launch_gamma_finalize(rf_ctx* c, const int* done);
 
 // transforms along y and z: tensor cores (split operands) in the split-precision modes, the
-// SIMT DFT otherwise
+// SIMT DFT otherwise (rf_dft.cu). sign +1: S sparse rows -> L dense ones, -1: the reverse.
 static int axis(rf_ctx* c, const TcAxis& ax, const float2* in, int in_splits, long long iss,
-                long long ibs, float2* out, int out_splits, long long oss, long long obs, int M,
-                int N, int K, int batch, const int* mvals, const int* kvals, const float2* tab,
-                int L, int sign, const int* done) {
+                long long ibs, float2* out, long long obs, int L, int N, int S, int batch,
+                const int* vals, const float2* tab, int sign, const int* done) {
   if (c->opt.precision != RF_PREC_FP32)
     return launch_tc_axis(c, ax, in, in_splits, iss, ibs, out, obs, N, batch, done);
-  return dft(c, in, in_splits, iss, ibs, out, out_splits, oss, obs, M, N, K, batch, mvals, kvals,
-             tab, L, sign, done);
+  return launch_axis_dft(c, in, ibs, out, obs, L, N, S, batch, vals, tab, sign, done);
 }
 
 static int inverse_stages(rf_ctx* c, const int* done) {
@@ -803,18 +694,17 @@ static int inverse_stages(rf_ctx* c, const int* done) {
   if (c->dim == 3) {
     // along z: T2[z][ky][c][kx] = sum_kz exp(+..kz z) ER[kz][ky][c][kx]
     trace_stage(c, 0);
-    if (int e = axis(c, c->tc_zi, c->d_ER, 1, 0, 0, c->d_T2, 1, 0, 0, c->nz, c->Ky * NCK, c->Kz,
-                     1, nullptr, c->d_kzm, c->d_twz, c->nz, +1, done))
+    if (int e = axis(c, c->tc_zi, c->d_ER, 1, 0, 0, c->d_T2, 0, c->nz, c->Ky * NCK, c->Kz, 1,
+                     c->d_kzm, c->d_twz, +1, done))
       return e;
     // along y, batched over z
     trace_stage(c, 1);
-    return axis(c, c->tc_yi, c->d_T2, 1, 0, (long long)c->Ky * NCK, c->d_T1, 1, 0,
-                (long long)c->ny * NCK, c->ny, NCK, c->Ky, c->nz, nullptr, c->d_kym, c->d_twy,
-                c->ny, +1, done);
+    return axis(c, c->tc_yi, c->d_T2, 1, 0, (long long)c->Ky * NCK, c->d_T1,
+                (long long)c->ny * NCK, c->ny, NCK, c->Ky, c->nz, c->d_kym, c->d_twy, +1, done);
   }
   trace_stage(c, 1);
-  return axis(c, c->tc_yi, c->d_ER, 1, 0, 0, c->d_T1, 1, 0, 0, c->ny, NCK, c->Ky, 1, nullptr,
-              c->d_kym, c->d_twy, c->ny, +1, done);
+  return axis(c, c->tc_yi, c->d_ER, 1, 0, 0, c->d_T1, 0, c->ny, NCK, c->Ky, 1, c->d_kym, c->d_twy,
+              +1, done);
 }
 
 int launch_iteration(rf_ctx* c) {
@@ -858,46 +748,45 @@ int launch_iteration(rf_ctx* c) {
     trace_stage(c, 2);
     if (int e = launch_fft_row(c, done, false, 0)) return e;
     if (int e = fft_forward_stages(c, done)) return e;
-    return launch_gamma_finalize(c, 1, done);
+    return launch_gamma_finalize(c, done);
   }
   if (int e = inverse_stages(c, done)) return e;
   const bool tcm = c->opt.precision != RF_PREC_FP32;
   trace_stage(c, 2);
   if (tcm) {
     if (int e = launch_tc_row(c, done)) return e;
+  } else if (c->dft_U > 0) {
+    if (int e = launch_row_dft(c, done, false, 0, nullptr)) return e;
   } else {
     RowArgs ra = row_args(c, done);
     if (int e = row_dispatch(c, ra, false)) return e;
   }
   const int NCK = c->nc * c->Kx;
-  const long long outstride = c->rect;
   // the tensor-core row kernel leaves one partial sum per 128-wide x slice
   const float2* fin = tcm ? reinterpret_cast<const float2*>(c->d_Tout) : c->d_T1p;
   const int fsplits = tcm ? c->tc_nXS : 1;
   const long long fstride = (long long)c->rows * NCK;
   trace_stage(c, 3);
   if (c->dim == 3) {
-    if (int e = axis(c, c->tc_yf, fin, fsplits, fstride, (long long)c->ny * NCK, c->d_T2f, 1, 0,
-                     (long long)c->Ky * NCK, c->Ky, NCK, c->ny, c->nz, c->d_kym, nullptr,
-                     c->d_twy, c->ny, -1, done))
+    if (int e = axis(c, c->tc_yf, fin, fsplits, fstride, (long long)c->ny * NCK, c->d_T2f,
+                     (long long)c->Ky * NCK, c->ny, NCK, c->Ky, c->nz, c->d_kym, c->d_twy, -1,
+                     done))
       return e;
     trace_stage(c, 4);
-    if (int e = axis(c, c->tc_zf, c->d_T2f, 1, 0, 0, c->d_OUT, c->splitC, outstride, 0, c->Kz,
-                     c->Ky * NCK, c->nz, 1, c->d_kzm, nullptr, c->d_twz, c->nz, -1, done))
+    if (int e = axis(c, c->tc_zf, c->d_T2f, 1, 0, 0, c->d_OUT, 0, c->nz, c->Ky * NCK, c->Kz, 1,
+                     c->d_kzm, c->d_twz, -1, done))
       return e;
   } else {
-    if (int e = axis(c, c->tc_yf, fin, fsplits, fstride, 0, c->d_OUT, c->splitB, outstride, 0,
-                     c->Ky, NCK, c->ny, 1, c->d_kym, nullptr, c->d_twy, c->ny, -1, done))
+    if (int e = axis(c, c->tc_yf, fin, fsplits, fstride, 0, c->d_OUT, 0, c->ny, NCK, c->Ky, 1,
+                     c->d_kym, c->d_twy, -1, done))
       return e;
   }
-  return launch_gamma_finalize(c, (c->dim == 3) ? c->splitC : c->splitB, done);
+  return launch_gamma_finalize(c, done);
 }
 
-int launch_gamma_finalize(rf_ctx* c, int splits, const int* done) {
+int launch_gamma_finalize(rf_ctx* c, const int* done) {
   GammaArgs g{};
   g.OUT = c->d_OUT;
-  g.splits = splits;
-  g.split_stride = c->rect;
   g.ER = c->d_ER;
   g.hidx = c->d_hidx;
   g.hn = c->d_hn;
@@ -915,6 +804,7 @@ int launch_gamma_finalize(rf_ctx* c, int splits, const int* done) {
   g.cond = c->while_cond;
   g.use_cond = c->capturing_while ? 1 : 0;
   const unsigned gb = (unsigned)((c->Kh + kGammaBlock - 1) / kGammaBlock);
+  g.early = gb <= 76 ? 1 : 0;
   trace_stage(c, 5);
   const cudaError_t le =
       c->nc == 3 ? launch_pdl(k_gamma<3>, dim3(gb), dim3(kGammaBlock), 0, c->stream, g, (double)c->N)
@@ -972,6 +862,15 @@ int launch_final(rf_ctx* c, int commit) {
   int ie = inverse_stages(c, nullptr);
   c->tracing = tr;
   if (ie) return ie;
+  if (c->dft_U > 0) {
+    int blocks = 0;
+    if (int e = launch_row_dft(c, nullptr, true, commit, &blocks)) return e;
+    k_reduce_sbar<<<1, kReduceThreads, 0, c->stream>>>(c->d_sbar_part, c->d_viol_part, blocks,
+                                                       1.0 / (double)c->N, c->d_sbar);
+    int e = launch_check(c, "reduce_sbar");
+    trace_end(c);
+    return e;
+  }
   RowArgs ra = row_args(c, nullptr);
   ra.eps_out = c->d_eps;
   ra.sig_out = c->d_sig;
