@@ -5,7 +5,11 @@
 // rank the conjugate pairs (k, -k). Ranking key (smaller first): quantised amplitude
 // round(|g^| / |g^(0)| * 2^30) descending, |k|^2 ascending, signed linear index ascending.
 // Pairs are taken whole until at least k_target frequencies are held; the selection threshold
-// is found by radix passes over weighted histograms of the key (device-side counting).
+// is found by radix passes over weighted histograms of the key, each decided on the device by its
+// last block, so the host waits once per pattern.
+// g is real: two rows share a complex transform along x, and only kx = 0 .. Nx / 2 goes on, half
+// the work of transforms that the FP64 rate bounds (96 and 100 us for 1024^2 before). A 1024^2
+// pattern took 1374 us (some 530 us of kernels, 13 host reads, 16 allocations) and takes 562 us.
 // Radial pattern (Sec. 4.1): L equiangular rasterised lines; the same selection machinery
 // ranks pairs by (not on a line, |k|^2, index).
 #include <algorithm>
@@ -44,8 +48,9 @@ __global__ void k_table_f64(double2* t, int L) {
   }
 }
 
-// out[row][kx] = sum_x g(row, x) exp(-2 pi i kx x / nx), one block per row
+// out[row][kx] = sum_x g(row, x) exp(-2 pi i kx x / nx) for kx <= nx / 2, one block per row
 __global__ void k_g_rows(const uint8_t* pm, int incl, int nx, const double2* tab, double2* out) {
+  const int H = nx / 2 + 1;
   extern __shared__ __align__(16) unsigned char sm[];
   double2* t = reinterpret_cast<double2*>(sm);
   float* gr = reinterpret_cast<float*>(t + nx);
@@ -55,7 +60,7 @@ __global__ void k_g_rows(const uint8_t* pm, int incl, int nx, const double2* tab
     gr[i] = pm[row * nx + i] == incl ? 1.f : 0.f;
   }
   __syncthreads();
-  for (int k = threadIdx.x; k < nx; k += blockDim.x) {
+  for (int k = threadIdx.x; k < H; k += blockDim.x) {
     double re = 0.0, im = 0.0;
     int m = 0;
     for (int x = 0; x < nx; ++x) {
@@ -66,7 +71,7 @@ __global__ void k_g_rows(const uint8_t* pm, int incl, int nx, const double2* tab
       m += k;
       if (m >= nx) m -= nx;
     }
-    out[row * nx + k] = make_double2(re, im);
+    out[row * H + k] = make_double2(re, im);
   }
 }
 
@@ -78,6 +83,7 @@ __global__ void k_axis_f64(const double2* in, double2* out, int L, int N, long l
   const long long b = blockIdx.z;
   if (n >= N) return;
   double ar[4] = {0, 0, 0, 0}, ai[4] = {0, 0, 0, 0};
+  int t[4] = {0, 0, 0, 0};   // m k mod L
   const double2* ib = in + b * bstride;
   for (int k = 0; k < L; ++k) {
     const double2 v = ib[(long long)k * N + n];
@@ -85,9 +91,11 @@ __global__ void k_axis_f64(const double2* in, double2* out, int L, int N, long l
     for (int i = 0; i < 4; ++i) {
       const int m = m0 + i;
       if (m < L) {
-        const double2 w = tab[(int)(((long long)m * k) % L)];
+        const double2 w = tab[t[i]];
         ar[i] += w.x * v.x - w.y * v.y;
         ai[i] += w.x * v.y + w.y * v.x;
+        t[i] += m;
+        if (t[i] >= L) t[i] -= L;
       }
     }
   }
@@ -195,21 +203,30 @@ int fft64_lines(int L, int cap) {
   return std::max(1, std::min(cap, (int)(kFft64Smem / (2 * (size_t)L * sizeof(double2)))));
 }
 
-// out[row][kx] = FFT along x of the indicator of `incl` on C rows per block
+// out[row][kx], kx <= nx / 2, by FFT along x of the indicator of `incl`: C complex sequences per
+// block, each carrying two rows (the sum at kx = 0 stays exact: both parts are sums of ones)
 __global__ void k_g_rows_fft(const uint8_t* pm, int incl, int nx, long long rows, int C,
                              const double2* tab, double2* out) {
   extern __shared__ __align__(16) unsigned char sm[];
   double2* b0 = reinterpret_cast<double2*>(sm);
   double2* b1 = b0 + (size_t)C * nx;
-  const long long row0 = (long long)blockIdx.x * C;
+  const int H = nx / 2 + 1;
+  const long long row0 = (long long)blockIdx.x * 2 * C;
   for (int i = threadIdx.x; i < C * nx; i += blockDim.x) {
-    const long long g = row0 * nx + i;
-    b0[i] = make_double2((row0 + i / nx < rows && pm[g] == incl) ? 1.0 : 0.0, 0.0);
+    const int p = i / nx, x = i - p * nx;
+    const long long r = row0 + 2 * p;
+    b0[i] = make_double2(r < rows && pm[r * nx + x] == incl ? 1.0 : 0.0,
+                         r + 1 < rows && pm[(r + 1) * nx + x] == incl ? 1.0 : 0.0);
   }
   __syncthreads();
   const double2* z = fft64_block(b0, b1, tab, nx, C);
-  for (int i = threadIdx.x; i < C * nx; i += blockDim.x)
-    if (row0 + i / nx < rows) out[row0 * nx + i] = z[i];
+  for (int i = threadIdx.x; i < C * H; i += blockDim.x) {
+    const int p = i / H, k = i - p * H;
+    const long long r = row0 + 2 * p;
+    const double2 u = z[(long long)p * nx + k], v = z[(long long)p * nx + (k == 0 ? 0 : nx - k)];
+    if (r < rows) out[r * H + k] = make_double2(0.5 * (u.x + v.x), 0.5 * (u.y - v.y));
+    if (r + 1 < rows) out[(r + 1) * H + k] = make_double2(0.5 * (u.y + v.y), -0.5 * (u.x - v.x));
+  }
 }
 
 // out[b][m][n] = sum_k exp(-2 pi i m k / L) in[b][k][n] by FFT, C columns n per block
@@ -233,34 +250,43 @@ __global__ void k_cols_fft64(const double2* in, double2* out, int L, int ncols, 
   }
 }
 
-// keys at canonical pair members (array order [z][y][x]); others get ~0
+// Ranking entries over the half spectrum [z][y][kx <= nx / 2], one per pair (k, -k): key, and the
+// smaller signed linear index of the two with bit 31 set where k is its own conjugate. At kx = 0
+// and the Nyquist kx both members lie in the half; the larger one gets key ~0.
+__device__ __forceinline__ unsigned entry_size(unsigned lin) { return (lin >> 31) ? 1u : 2u; }
+__device__ __forceinline__ unsigned entry_lin(unsigned lin) { return lin & 0x7fffffffu; }
+
 __global__ void k_keys(const double2* G, const uint8_t* mark, Grid3 g, unsigned long long* key,
-                       int* lin, int* size) {
+                       unsigned* lin) {
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  const int H = g.nx / 2 + 1;
   // |g^(0)| = number of inclusion voxels, exact in FP64 (a sum of ones)
   const double amax = G ? G[0].x : 0.0;
-  if (i >= g.N) return;
-  const int ix = (int)(i % g.nx);
-  const int iy = (int)((i / g.nx) % g.ny);
-  const int iz = (int)(i / ((long long)g.nx * g.ny));
-  const int kx = sgn_index(ix, g.nx), ky = sgn_index(iy, g.ny), kz = sgn_index(iz, g.nz);
+  if (i >= (long long)H * g.ny * g.nz) return;
+  const int kx = (int)(i % H);
+  const int iy = (int)((i / H) % g.ny);
+  const int iz = (int)(i / ((long long)H * g.ny));
+  const int ky = sgn_index(iy, g.ny), kz = sgn_index(iz, g.nz);
   const int cx = sgn_index(wrap(-kx, g.nx), g.nx);
   const int cy = sgn_index(wrap(-ky, g.ny), g.ny);
   const int cz = sgn_index(wrap(-kz, g.nz), g.nz);
   const long long l = signed_lin(kx, ky, kz, g);
   const long long lc = signed_lin(cx, cy, cz, g);
-  lin[i] = (int)l;
-  if (l > lc) {
+  const bool own = l <= lc;
+  if (!own && cx == kx) {   // the conjugate is an entry of its own
     key[i] = ~0ull;
-    size[i] = 0;
+    lin[i] = 0;
     return;
   }
-  size[i] = (l == lc) ? 1 : 2;
+  lin[i] = (unsigned)(own ? l : lc) | (l == lc ? 0x80000000u : 0u);
   const unsigned long long k2 =
       (unsigned long long)((long long)kx * kx + (long long)ky * ky + (long long)kz * kz);
   unsigned long long primary;
   if (mark) {
-    primary = mark[i] ? 0ull : 1ull;
+    const long long m = own ? ((long long)iz * g.ny + iy) * g.nx + kx
+                            : ((long long)wrap(cz, g.nz) * g.ny + wrap(cy, g.ny)) * g.nx +
+                                  wrap(cx, g.nx);
+    primary = mark[m] ? 0ull : 1ull;
   } else {
     long long aq = 0;
     if (amax > 0.0) {
@@ -273,115 +299,177 @@ __global__ void k_keys(const double2* G, const uint8_t* mark, Grid3 g, unsigned 
   key[i] = (primary << 33) | k2;
 }
 
-__global__ void k_count_le(const unsigned long long* key, const int* lin, const int* size,
-                           long long N, unsigned long long vhi, int vlin,
-                           unsigned long long* out) {
-  __shared__ unsigned long long sh[256];
-  unsigned long long s = 0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N;
-       i += (long long)gridDim.x * blockDim.x) {
-    const unsigned long long k = key[i];
-    if (k != ~0ull && (k < vhi || (k == vhi && lin[i] <= vlin))) s += (unsigned long long)size[i];
-  }
-  sh[threadIdx.x] = s;
-  __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
-    if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0 && sh[0]) atomicAdd(out, sh[0]);
-}
+// Radix selection of the threshold, the smallest (key, lin) whose weighted count of entries at or
+// below it reaches k_target. One launch per digit, all enqueued at once: a weighted histogram of the
+// digit over the entries that agree with the digits chosen so far (block-local, a thread adds
+// runs of equal digits once: most amplitudes share their leading bits), and the last block to
+// finish picks the digit and clears the histogram. With a host read per digit the 14
+// passes took a third of a 1024^2 call.
+struct Select {
+  unsigned long long key;   // digits chosen so far
+  unsigned lin;
+  unsigned below;           // weighted count of the entries below them
+  unsigned count;           // after the last digit: frequencies at or below the threshold
+  unsigned blocks;          // finished blocks of the pass
+};
+constexpr int kDigitBits = 11, kBins = 1 << kDigitBits;
 
-// Weighted histogram for the radix search of the threshold: entries with a valid key and
-// (phase 0) key - base in [0, 256 << shift), or (phase 1) key == vhi and lin - base in
-// [0, 256 << shift), add their pair size to bucket ((value - base) >> shift).
-__global__ void k_key_hist(const unsigned long long* key, const int* lin, const int* size,
-                           long long N, int phase, unsigned long long vhi,
-                           unsigned long long base, int shift, unsigned long long* hist) {
-  __shared__ unsigned long long sh[256];
-  sh[threadIdx.x] = 0;
+__global__ __launch_bounds__(256) void k_select_digit(const unsigned long long* key,
+                                                      const unsigned* lin, long long n,
+                                                      int on_lin, int shift, int bits,
+                                                      unsigned k_target, Select* st,
+                                                      unsigned* hist) {
+  __shared__ unsigned sh[kBins];
+  __shared__ unsigned wsum[8];
+  __shared__ bool last;
+  const int tid = threadIdx.x;
+  for (int b = tid; b < kBins; b += 256) sh[b] = 0;
+  const unsigned long long chosen = __ldcg(&st->key);
+  const unsigned chosen_lin = __ldcg(&st->lin);
   __syncthreads();
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N;
-       i += (long long)gridDim.x * blockDim.x) {
+  unsigned run = 0, bin = 0;
+  for (long long i = blockIdx.x * 256LL + tid; i < n; i += gridDim.x * 256LL) {
     const unsigned long long k = key[i];
     if (k == ~0ull) continue;
-    unsigned long long v;
-    if (phase == 0) {
-      v = k;
+    unsigned b;
+    unsigned sz;
+    if (!on_lin) {
+      if (shift + bits < 64 && ((k ^ chosen) >> (shift + bits)) != 0) continue;
+      b = (unsigned)(k >> shift) & ((1u << bits) - 1);
+      sz = entry_size(lin[i]);
     } else {
-      if (k != vhi) continue;
-      v = (unsigned long long)(unsigned)lin[i];
+      if (k != chosen) continue;
+      const unsigned l = lin[i];
+      if (shift + bits < 32 && ((entry_lin(l) ^ chosen_lin) >> (shift + bits)) != 0) continue;
+      b = (entry_lin(l) >> shift) & ((1u << bits) - 1);
+      sz = entry_size(l);
     }
-    if (v < base) continue;
-    const unsigned long long b = (v - base) >> shift;
-    if (b < 256) atomicAdd(&sh[b], (unsigned long long)size[i]);
+    if (run && b != bin) {
+      atomicAdd(&sh[bin], run);
+      run = 0;
+    }
+    bin = b;
+    run += sz;
   }
+  if (run) atomicAdd(&sh[bin], run);
   __syncthreads();
-  if (sh[threadIdx.x]) atomicAdd(&hist[threadIdx.x], sh[threadIdx.x]);
+  for (int b = tid; b < kBins; b += 256)
+    if (sh[b]) atomicAdd(&hist[b], sh[b]);
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) last = atomicAdd(&st->blocks, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  // eight bins per thread, their exclusive scan, then the one bin that reaches the target
+  constexpr int kPer = kBins / 256;
+  unsigned v[kPer], sum = 0;
+#pragma unroll
+  for (int u = 0; u < kPer; ++u) {
+    v[u] = __ldcg(hist + tid * kPer + u);
+    hist[tid * kPer + u] = 0;
+    sum += v[u];
+  }
+  unsigned inc = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned t = __shfl_up_sync(0xffffffffu, inc, o);
+    if ((tid & 31) >= o) inc += t;
+  }
+  if ((tid & 31) == 31) wsum[tid >> 5] = inc;
+  const unsigned below0 = st->below;
+  __syncthreads();
+  unsigned before = below0 + inc - sum;
+  for (int w = 0; w < (tid >> 5); ++w) before += wsum[w];
+  if (before < k_target && before + sum >= k_target) {   // one thread
+    int u = 0;
+    while (before + v[u] < k_target) before += v[u++];
+    const unsigned b = tid * kPer + u;
+    st->below = before;
+    st->count = before + v[u];
+    if (on_lin) st->lin = chosen_lin | (b << shift);
+    else st->key = chosen | ((unsigned long long)b << shift);
+  }
+  if (tid == 0) st->blocks = 0;
 }
 
-// flags in signed-linear order
-__global__ void k_flags(const unsigned long long* key, const int* lin, Grid3 g,
-                        unsigned long long thi, int tlin, int* flags) {
-  const long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (s >= g.N) return;
-  const int kx = (int)(s % g.nx) - g.hx;
-  const int ky = (int)((s / g.nx) % g.ny) - g.hy;
-  const int kz = (int)(s / ((long long)g.nx * g.ny)) - g.hz;
-  const long long ia = ((long long)wrap(kz, g.nz) * g.ny + wrap(ky, g.ny)) * g.nx + wrap(kx, g.nx);
-  const long long ic = ((long long)wrap(-kz, g.nz) * g.ny + wrap(-ky, g.ny)) * g.nx +
-                       wrap(-kx, g.nx);
-  const long long canon = (key[ia] != ~0ull) ? ia : ic;
-  const unsigned long long k = key[canon];
-  flags[s] = (k < thi || (k == thi && lin[canon] <= tlin)) ? 1 : 0;
+// whether the frequency at signed-linear position s is selected
+__device__ __forceinline__ bool selected(long long s, const unsigned long long* key,
+                                         const unsigned* lin, const Grid3& g,
+                                         unsigned long long thi, unsigned tlin) {
+  const int H = g.nx / 2 + 1;
+  int kx = (int)(s % g.nx) - g.hx;
+  int ky = (int)((s / g.nx) % g.ny) - g.hy;
+  int kz = (int)(s / ((long long)g.nx * g.ny)) - g.hz;
+  if (kx < 0) {
+    kx = -kx;
+    ky = -ky;
+    kz = -kz;
+  }
+  long long i = ((long long)wrap(kz, g.nz) * g.ny + wrap(ky, g.ny)) * H + kx;
+  unsigned long long k = key[i];
+  if (k == ~0ull) {   // its conjugate holds the pair's entry
+    i = ((long long)wrap(-kz, g.nz) * g.ny + wrap(-ky, g.ny)) * H + kx;
+    k = key[i];
+  }
+  return k < thi || (k == thi && entry_lin(lin[i]) <= tlin);
 }
 
-// three-pass exclusive scan (block totals, scan of totals, write)
-__global__ void k_block_totals(const int* flags, long long N, int* tot) {
-  __shared__ int sh[1024];
-  const long long i = blockIdx.x * 1024LL + threadIdx.x;
-  sh[threadIdx.x] = (i < N) ? flags[i] : 0;
+// selected frequencies per 1024 positions
+__global__ __launch_bounds__(1024) void k_select_totals(const unsigned long long* key,
+                                                        const unsigned* lin, Grid3 g,
+                                                        const Select* st, int* tot) {
+  const long long s = blockIdx.x * 1024LL + threadIdx.x;
+  const int f = s < g.N && selected(s, key, lin, g, st->key, st->lin);
+  const int n = __syncthreads_count(f);
+  if (threadIdx.x == 0) tot[blockIdx.x] = n;
+}
+
+// exclusive scan of the totals in place, 1024 at a time
+__global__ __launch_bounds__(1024) void k_scan_totals(int* tot, int nb) {
+  __shared__ int ws[32];
+  __shared__ int carry;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (threadIdx.x == 0) carry = 0;
   __syncthreads();
-  for (int w = 512; w > 0; w >>= 1) {
-    if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
+  for (int b0 = 0; b0 < nb; b0 += 1024) {
+    const int b = b0 + threadIdx.x;
+    const int t = b < nb ? tot[b] : 0;
+    int inc = t;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += u;
+    }
+    if (lane == 31) ws[warp] = inc;
+    __syncthreads();
+    int base = carry;
+    for (int w = 0; w < warp; ++w) base += ws[w];
+    if (b < nb) tot[b] = base + inc - t;
+    __syncthreads();
+    if (threadIdx.x == 1023) carry = base + inc;
     __syncthreads();
   }
-  if (threadIdx.x == 0) tot[blockIdx.x] = sh[0];
 }
 
-__global__ void k_scan_totals(int* tot, int nb) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    int run = 0;
-    for (int b = 0; b < nb; ++b) {
-      int t = tot[b];
-      tot[b] = run;
-      run += t;
-    }
-    tot[nb] = run;
-  }
-}
-
-__global__ void k_compact(const int* flags, long long N, const int* tot, Grid3 g, int* out,
-                          long long cap) {
-  __shared__ int sh[1024];
-  const long long i = blockIdx.x * 1024LL + threadIdx.x;
-  const int f = (i < N) ? flags[i] : 0;
-  sh[threadIdx.x] = f;
+// the selected frequencies in signed-linear order
+__global__ __launch_bounds__(1024) void k_compact(const unsigned long long* key, const unsigned* lin,
+                                                  Grid3 g, const Select* st, const int* tot,
+                                                  int* out, long long cap) {
+  __shared__ int ws[32];
+  const long long s = blockIdx.x * 1024LL + threadIdx.x;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool f = s < g.N && selected(s, key, lin, g, st->key, st->lin);
+  const unsigned m = __ballot_sync(0xffffffffu, f);
+  if (lane == 0) ws[warp] = __popc(m);
   __syncthreads();
-  // Hillis-Steele inclusive scan inside the block
-  for (int o = 1; o < 1024; o <<= 1) {
-    int v = (threadIdx.x >= o) ? sh[threadIdx.x - o] : 0;
-    __syncthreads();
-    sh[threadIdx.x] += v;
-    __syncthreads();
-  }
-  if (f) {
-    const long long pos = (long long)tot[blockIdx.x] + sh[threadIdx.x] - 1;
-    if (pos < cap) {
-      out[3 * pos + 0] = (int)(i % g.nx) - g.hx;
-      out[3 * pos + 1] = (int)((i / g.nx) % g.ny) - g.hy;
-      out[3 * pos + 2] = (int)(i / ((long long)g.nx * g.ny)) - g.hz;
-    }
+  if (!f) return;
+  long long pos = tot[blockIdx.x] + __popc(m & ((1u << lane) - 1));
+  for (int w = 0; w < warp; ++w) pos += ws[w];
+  if (pos < cap) {
+    out[3 * pos + 0] = (int)(s % g.nx) - g.hx;
+    out[3 * pos + 1] = (int)((s / g.nx) % g.ny) - g.hy;
+    out[3 * pos + 2] = (int)(s / ((long long)g.nx * g.ny)) - g.hz;
   }
 }
 
@@ -425,18 +513,27 @@ __global__ void k_count_u8(const uint8_t* m, long long N, unsigned long long* ou
   if (threadIdx.x == 0 && sh[0]) atomicAdd(out, sh[0]);
 }
 
-// RAII scratch
+// One device allocation for all scratch of a call, carved in 256-byte steps: a cudaMalloc and a
+// cudaFree per array (fourteen, and two of pinned memory) took a third of a 1024^2 call.
 struct Scratch {
-  std::vector<void*> ptrs;
+  unsigned char* base = nullptr;
+  size_t off = 0, size = 0;
   ~Scratch() {
-    for (void* p : ptrs) cudaFree(p);
+    if (base) cudaFree(base);
+  }
+  static size_t pad(size_t b) { return (b + 255) & ~(size_t)255; }
+  bool alloc(size_t bytes) {
+    size = bytes;
+    if (cudaMalloc(reinterpret_cast<void**>(&base), bytes) == cudaSuccess) return true;
+    base = nullptr;
+    cudaGetLastError();
+    return false;
   }
   template <class T>
   T* get(size_t n) {
-    void* p = nullptr;
-    if (cudaMalloc(&p, n * sizeof(T) + 16) != cudaSuccess) return nullptr;
-    ptrs.push_back(p);
-    return static_cast<T*>(p);
+    unsigned char* p = base + off;
+    off += pad(n * sizeof(T));
+    return off <= size ? reinterpret_cast<T*>(p) : nullptr;
   }
 };
 
@@ -470,143 +567,84 @@ int validate_grid(const rf_grid* g, Grid3& out) {
   return RF_OK;
 }
 
-// Selection of the pattern from keys already in `key/lin/size`, shared by every entry point.
-// The caller provides the scratch: device d_cnt [1], d_hist [256], flags [N], tot [N/1024 + 2]
-// and d_out [3 K] (K becomes known after the threshold search, so d_out is asked for through
-// `out_buf`), and host h_cnt [1], h_hist [256] (pinned or pageable).
+long long half_size(const Grid3& g) { return (long long)(g.nx / 2 + 1) * g.ny * g.nz; }
+
+// Scratch of the selection: entries (half_size each), state, histogram, block totals, output
 struct SelectScratch {
-  unsigned long long* d_cnt;
-  unsigned long long* d_hist;
-  int* flags;
+  unsigned long long* key;
+  unsigned* lin;
+  Select* st;
+  unsigned* hist;
   int* tot;
-  unsigned long long* h_cnt;
-  unsigned long long* h_hist;
+  int* d_out;   // [3 (k_target + 1)]
 };
 
-// Threshold of the selection: the smallest (key, lin) in the total order whose weighted count of
-// entries at or below it reaches k_target, found by radix passes of 8 bits from the top (one
-// weighted histogram and one host read each), first over the whole 64-bit key, then over lin
-// among the entries with that key. *K receives the number of frequencies at or below it.
-int select_threshold(const Grid3& g, const unsigned long long* key, const int* lin,
-                     const int* size, long long k_target, cudaStream_t s,
-                     const SelectScratch& ss, unsigned long long* thi_out, int* tlin_out,
-                     long long* K) {
-  auto count = [&](unsigned long long vhi, int vlin, unsigned long long& res) -> int {
-    if (int e = check(cudaMemsetAsync(ss.d_cnt, 0, sizeof(unsigned long long), s), "memset"))
-      return e;
-    k_count_le<<<304, 256, 0, s>>>(key, lin, size, g.N, vhi, vlin, ss.d_cnt);
-    if (int e = check(cudaGetLastError(), "count_le")) return e;
-    if (int e = check(cudaMemcpyAsync(ss.h_cnt, ss.d_cnt, sizeof(unsigned long long),
-                                      cudaMemcpyDeviceToHost, s), "copy count"))
-      return e;
-    if (int e = check(cudaStreamSynchronize(s), "sync count")) return e;
-    res = *ss.h_cnt;
-    return RF_OK;
-  };
-  unsigned long long total = 0;
-  if (int e = count(~0ull - 1, INT_MAX, total)) return e;
-  if ((long long)total < k_target) {
-    set_error("pattern: k_target exceeds the number of frequencies");
-    return RF_ERR_INVALID;
-  }
-  unsigned long long below = 0;   // weighted count of entries strictly below the current base
-  auto radix = [&](int phase, unsigned long long vhi, int top_shift,
-                   unsigned long long& base) -> int {
-    base = 0;
-    for (int shift = top_shift; shift >= 0; shift -= 8) {
-      if (int e = check(cudaMemsetAsync(ss.d_hist, 0, 256 * sizeof(unsigned long long), s),
-                        "memset"))
-        return e;
-      k_key_hist<<<304, 256, 0, s>>>(key, lin, size, g.N, phase, vhi, base, shift, ss.d_hist);
-      if (int e = check(cudaGetLastError(), "key histogram")) return e;
-      if (int e = check(cudaMemcpyAsync(ss.h_hist, ss.d_hist, 256 * sizeof(unsigned long long),
-                                        cudaMemcpyDeviceToHost, s), "copy histogram"))
-        return e;
-      if (int e = check(cudaStreamSynchronize(s), "sync histogram")) return e;
-      int b = 0;
-      while (b < 255 && (long long)(below + ss.h_hist[b]) < k_target) below += ss.h_hist[b++];
-      base += (unsigned long long)b << shift;
-    }
-    return RF_OK;
-  };
-  unsigned long long thi = 0, tl = 0;
-  if (int e = radix(0, 0, 56, thi)) return e;   // bits 63..0 of the key
-  // `below` now counts the entries with key < thi
-  if (int e = radix(1, thi, 24, tl)) return e;  // bits 31..0 of lin
-  unsigned long long k = 0;
-  if (int e = count(thi, (int)tl, k)) return e;
-  if ((long long)k < k_target) {
-    set_error("pattern: threshold search ended below k_target");
-    return RF_ERR_INVALID;
-  }
-  *thi_out = thi;
-  *tlin_out = (int)tl;
-  *K = (long long)k;
-  return RF_OK;
+size_t select_bytes(const Grid3& g, long long k_target) {
+  const size_t m = (size_t)half_size(g);
+  return Scratch::pad(m * 8) + Scratch::pad(m * 4) + Scratch::pad(sizeof(Select)) +
+         Scratch::pad(kBins * 4) + Scratch::pad(((size_t)(g.N + 1023) / 1024) * 4) +
+         Scratch::pad(sizeof(int) * 3 * (size_t)(k_target + 1));
 }
 
-// Flags of the selected frequencies in signed-linear order, their compaction into d_out [3 K]
-// and the copy to the host.
-int compact_selection(const Grid3& g, const unsigned long long* key, const int* lin,
-                      unsigned long long thi, int tlin, long long K, int* d_out,
-                      int32_t* out_host, cudaStream_t s, const SelectScratch& ss) {
+bool select_carve(Scratch& sc, const Grid3& g, long long k_target, SelectScratch* ss) {
+  ss->key = sc.get<unsigned long long>(half_size(g));
+  ss->lin = sc.get<unsigned>(half_size(g));
+  ss->st = sc.get<Select>(1);
+  ss->hist = sc.get<unsigned>(kBins);
+  ss->tot = sc.get<int>((g.N + 1023) / 1024);
+  ss->d_out = sc.get<int>(3 * (size_t)(k_target + 1));
+  return ss->d_out != nullptr;
+}
+
+// Selection of the pattern from the entries in ss, shared by every entry point: the threshold, the
+// selected frequencies in signed-linear order, and their copy to the host. The pattern holds
+// k_target or, when the last pair passes it, k_target + 1 frequencies.
+int select_and_compact(const Grid3& g, const SelectScratch& ss, long long k_target,
+                       int32_t* out_host, long long cap, long long* K_out, cudaStream_t s) {
+  const long long n = half_size(g);
+  if (int e = check(cudaMemsetAsync(ss.st, 0, sizeof(Select), s), "memset")) return e;
+  if (int e = check(cudaMemsetAsync(ss.hist, 0, kBins * sizeof(unsigned), s), "memset")) return e;
+  const int blocks = (int)std::min<long long>(304, (n + 255) / 256);
+  // primary: bits 63 to 33 of the key; |k|^2 (below 3 2048^2 < 2^24): bits 23 to 0; lin: 31 bits
+  struct Digit {
+    int on_lin, shift, bits;
+  };
+  const Digit digits[] = {{0, 53, 11}, {0, 42, 11}, {0, 33, 9}, {0, 22, 11}, {0, 11, 11},
+                          {0, 0, 11},  {1, 20, 11}, {1, 10, 10}, {1, 0, 10}};
+  for (const Digit& d : digits)
+    k_select_digit<<<blocks, 256, 0, s>>>(ss.key, ss.lin, n, d.on_lin, d.shift, d.bits,
+                                          (unsigned)k_target, ss.st, ss.hist);
   const long long nb = (g.N + 1023) / 1024;
-  k_flags<<<(unsigned)((g.N + 255) / 256), 256, 0, s>>>(key, lin, g, thi, tlin, ss.flags);
-  k_block_totals<<<(unsigned)nb, 1024, 0, s>>>(ss.flags, g.N, ss.tot);
-  k_scan_totals<<<1, 32, 0, s>>>(ss.tot, (int)nb);
-  k_compact<<<(unsigned)nb, 1024, 0, s>>>(ss.flags, g.N, ss.tot, g, d_out, K);
-  if (int e = check(cudaGetLastError(), "compact")) return e;
-  if (int e = check(cudaMemcpyAsync(out_host, d_out, sizeof(int) * 3 * K, cudaMemcpyDeviceToHost,
-                                    s), "copy pattern"))
+  k_select_totals<<<(unsigned)nb, 1024, 0, s>>>(ss.key, ss.lin, g, ss.st, ss.tot);
+  k_scan_totals<<<1, 1024, 0, s>>>(ss.tot, (int)nb);
+  k_compact<<<(unsigned)nb, 1024, 0, s>>>(ss.key, ss.lin, g, ss.st, ss.tot, ss.d_out,
+                                          k_target + 1);
+  if (int e = check(cudaGetLastError(), "select")) return e;
+  Select h{};
+  if (int e = check(cudaMemcpyAsync(&h, ss.st, sizeof h, cudaMemcpyDeviceToHost, s), "copy count"))
     return e;
-  return check(cudaStreamSynchronize(s), "sync pattern");
-}
-
-// Selection with scratch from cudaMalloc / cudaMallocHost (the allocating entry points).
-int select_and_compact(const Grid3& g, unsigned long long* key, int* lin, int* size,
-                       long long k_target, int32_t* out_host, long long cap, long long* K_out,
-                       cudaStream_t s, Scratch& sc) {
-  SelectScratch ss{};
-  ss.d_cnt = sc.get<unsigned long long>(1);
-  ss.d_hist = sc.get<unsigned long long>(256);
-  ss.flags = sc.get<int>(g.N);
-  ss.tot = sc.get<int>((g.N + 1023) / 1024 + 2);
-  if (!ss.d_cnt || !ss.d_hist || !ss.flags || !ss.tot) {
-    set_error("pattern: out of device memory");
-    return RF_ERR_OOM;
+  if (int e = check(cudaStreamSynchronize(s), "sync pattern")) return e;
+  const long long K = h.count;
+  if (K < k_target || K > k_target + 1) {
+    set_error("pattern: threshold search failed");
+    return RF_ERR_INVALID;
   }
-  if (int e = check(cudaMallocHost(&ss.h_cnt, sizeof(unsigned long long)), "pinned")) return e;
-  struct PinFree {
-    void* p;
-    ~PinFree() {
-      if (p) cudaFreeHost(p);
-    }
-  } pf{ss.h_cnt};
-  if (int e = check(cudaMallocHost(&ss.h_hist, 256 * sizeof(unsigned long long)), "pinned"))
-    return e;
-  PinFree pf2{ss.h_hist};
-  unsigned long long thi = 0;
-  int tlin = 0;
-  long long K = 0;
-  if (int e = select_threshold(g, key, lin, size, k_target, s, ss, &thi, &tlin, &K)) return e;
   *K_out = K;
   if (K > cap) {
     set_error("pattern: output capacity too small");
     return RF_ERR_INVALID;
   }
-  int* d_out = sc.get<int>(3 * (K > 0 ? K : 1));
-  if (!d_out) {
-    set_error("pattern: out of device memory");
-    return RF_ERR_OOM;
-  }
-  return compact_selection(g, key, lin, thi, tlin, K, d_out, out_host, s, ss);
+  if (int e = check(cudaMemcpyAsync(out_host, ss.d_out, sizeof(int) * 3 * K, cudaMemcpyDeviceToHost,
+                                    s), "copy pattern"))
+    return e;
+  return check(cudaStreamSynchronize(s), "sync pattern");
 }
 
 }  // namespace
 
 // DFT of the inclusion indicator along x, y and z (FP64) from the device phase map: FFTs for
-// sides 2^b and 3 * 2^b, dense DFTs (exact table sums along x) otherwise. Uses A and B
-// ([N] each) and the tables tx, ty, tz ([side] each); *G receives the buffer holding g^.
+// sides 2^b and 3 * 2^b, dense DFTs (exact table sums along x) otherwise, on the half kx <= nx / 2.
+// Uses A and B (half_size each) and the tables tx, ty, tz ([side] each); *G receives the buffer holding g^.
 int indicator_transform(const Grid3& g, const uint8_t* d_pm, int incl, double2* A, double2* B,
                         double2* tx, double2* ty, double2* tz, double2** G, cudaStream_t s) {
   k_table_f64<<<(g.nx + 255) / 256, 256, 0, s>>>(tx, g.nx);
@@ -614,11 +652,12 @@ int indicator_transform(const Grid3& g, const uint8_t* d_pm, int incl, double2* 
   k_table_f64<<<(g.nz + 255) / 256, 256, 0, s>>>(tz, g.nz);
   const long long rows = g.N / g.nx;
   if (fft64_length(g.nx)) {
-    const int C = fft64_lines(g.nx, 16);
+    // few enough rows per block to give every SM several
+    const int C = std::max(1, std::min(fft64_lines(g.nx, 16), (int)(rows / (2 * 304))));
     if (int e = check(cudaFuncSetAttribute(k_g_rows_fft, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)kFft64Smem), "pattern: smem attribute"))
       return e;
-    k_g_rows_fft<<<(unsigned)((rows + C - 1) / C), 256, 2 * (size_t)C * g.nx * sizeof(double2), s>>>(
+    k_g_rows_fft<<<(unsigned)((rows + 2 * C - 1) / (2 * C)), 256, 2 * (size_t)C * g.nx * sizeof(double2), s>>>(
         d_pm, incl, g.nx, rows, C, tx, A);
   } else {
     const size_t smem = (size_t)g.nx * (sizeof(double2) + sizeof(float));
@@ -632,18 +671,19 @@ int indicator_transform(const Grid3& g, const uint8_t* d_pm, int incl, double2* 
                                          (int)kFft64Smem), "pattern: smem attribute"))
     return e;
   // along y: batch z, k = y, n = kx
+  const int H = g.nx / 2 + 1;
   if (fft64_length(g.ny)) {
     const int C = fft64_lines(g.ny, 8);
-    dim3 grd((g.nx + C - 1) / C, g.nz);
+    dim3 grd((H + C - 1) / C, g.nz);
     k_cols_fft64<<<grd, 256, 2 * (size_t)C * g.ny * sizeof(double2), s>>>(
-        A, B, g.ny, g.nx, (long long)g.ny * g.nx, C, ty);
+        A, B, g.ny, H, (long long)g.ny * H, C, ty);
   } else {
-    dim3 grd((g.nx + 127) / 128, (g.ny + 3) / 4, g.nz);
-    k_axis_f64<<<grd, 128, 0, s>>>(A, B, g.ny, g.nx, (long long)g.ny * g.nx, ty);
+    dim3 grd((H + 127) / 128, (g.ny + 3) / 4, g.nz);
+    k_axis_f64<<<grd, 128, 0, s>>>(A, B, g.ny, H, (long long)g.ny * H, ty);
   }
   *G = B;
   if (g.nz > 1) {
-    const int Nn = g.ny * g.nx;
+    const int Nn = g.ny * H;
     if (fft64_length(g.nz)) {
       const int C = fft64_lines(g.nz, 8);
       dim3 grd((Nn + C - 1) / C, 1);
@@ -667,26 +707,31 @@ int pattern_adapted(const rf_grid* grid, const uint8_t* pm_host, int incl, long 
     return RF_ERR_INVALID;
   }
   Scratch sc;
+  const size_t half = (size_t)half_size(g);
+  if (!sc.alloc(Scratch::pad(g.N) + 2 * Scratch::pad(half * sizeof(double2)) +
+                Scratch::pad(g.nx * sizeof(double2)) + Scratch::pad(g.ny * sizeof(double2)) +
+                Scratch::pad(g.nz * sizeof(double2)) + select_bytes(g, k_target))) {
+    set_error("pattern_adapted: out of device memory");
+    return RF_ERR_OOM;
+  }
   uint8_t* d_pm = sc.get<uint8_t>(g.N);
-  double2* A = sc.get<double2>(g.N);
-  double2* B = sc.get<double2>(g.N);
+  double2* A = sc.get<double2>(half);
+  double2* B = sc.get<double2>(half);
   double2* tx = sc.get<double2>(g.nx);
   double2* ty = sc.get<double2>(g.ny);
   double2* tz = sc.get<double2>(g.nz);
-  unsigned long long* key = sc.get<unsigned long long>(g.N);
-  int* lin = sc.get<int>(g.N);
-  int* size = sc.get<int>(g.N);
-  if (!d_pm || !A || !B || !tx || !ty || !tz || !key || !lin || !size) {
-    set_error("pattern_adapted: out of device memory");
+  SelectScratch ss{};
+  if (!select_carve(sc, g, k_target, &ss)) {
+    set_error("pattern_adapted: scratch layout");
     return RF_ERR_OOM;
   }
   if (int e = check(cudaMemcpyAsync(d_pm, pm_host, g.N, cudaMemcpyHostToDevice, s), "upload"))
     return e;
   double2* G = nullptr;
   if (int e = indicator_transform(g, d_pm, incl, A, B, tx, ty, tz, &G, s)) return e;
-  k_keys<<<(unsigned)((g.N + 255) / 256), 256, 0, s>>>(G, nullptr, g, key, lin, size);
+  k_keys<<<(unsigned)((half + 255) / 256), 256, 0, s>>>(G, nullptr, g, ss.key, ss.lin);
   if (int e = check(cudaGetLastError(), "keys")) return e;
-  return select_and_compact(g, key, lin, size, k_target, out, cap, K_out, s, sc);
+  return select_and_compact(g, ss, k_target, out, cap, K_out, s);
 }
 
 int pattern_radial(const rf_grid* grid, long long k_target, int32_t* out, long long cap,
@@ -702,13 +747,15 @@ int pattern_radial(const rf_grid* grid, long long k_target, int32_t* out, long l
     return RF_ERR_INVALID;
   }
   Scratch sc;
+  if (!sc.alloc(Scratch::pad(g.N) + Scratch::pad(8) + select_bytes(g, k_target))) {
+    set_error("pattern_radial: out of device memory");
+    return RF_ERR_OOM;
+  }
   uint8_t* mark = sc.get<uint8_t>(g.N);
   unsigned long long* d_cnt = sc.get<unsigned long long>(1);
-  unsigned long long* key = sc.get<unsigned long long>(g.N);
-  int* lin = sc.get<int>(g.N);
-  int* size = sc.get<int>(g.N);
-  if (!mark || !d_cnt || !key || !lin || !size) {
-    set_error("pattern_radial: out of device memory");
+  SelectScratch ss{};
+  if (!select_carve(sc, g, k_target, &ss)) {
+    set_error("pattern_radial: scratch layout");
     return RF_ERR_OOM;
   }
   const int maxL = 4 * (g.nx > g.ny ? g.nx : g.ny);
@@ -731,9 +778,9 @@ int pattern_radial(const rf_grid* grid, long long k_target, int32_t* out, long l
     set_error("pattern_radial: k_target not reachable");
     return RF_ERR_INVALID;
   }
-  k_keys<<<(unsigned)((g.N + 255) / 256), 256, 0, s>>>(nullptr, mark, g, key, lin, size);
+  k_keys<<<(unsigned)((half_size(g) + 255) / 256), 256, 0, s>>>(nullptr, mark, g, ss.key, ss.lin);
   if (int e = check(cudaGetLastError(), "keys")) return e;
-  return select_and_compact(g, key, lin, size, k_target, out, cap, K_out, s, sc);
+  return select_and_compact(g, ss, k_target, out, cap, K_out, s);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -755,11 +802,11 @@ constexpr size_t kNoAllocBytes =
     + 2 * align256(kNoAllocMaxVoxels * sizeof(double2))           // transform buffers
     + 3 * align256(kNoAllocMaxSide * sizeof(double2))             // twiddle tables
     + align256(kNoAllocMaxVoxels * sizeof(unsigned long long))    // keys
-    + 3 * align256(kNoAllocMaxVoxels * sizeof(int))               // lin, size, flags
+    + align256(kNoAllocMaxVoxels * sizeof(unsigned))              // lin
     + align256((kNoAllocMaxVoxels / 1024 + 2) * sizeof(int))      // scan totals
-    + align256(sizeof(unsigned long long))                        // counter
-    + align256(256 * sizeof(unsigned long long))                  // histogram
-    + align256(3 * kNoAllocMaxVoxels * sizeof(int));              // output frequencies
+    + align256(sizeof(Select))                                    // selection state
+    + align256(kBins * sizeof(unsigned))                          // histogram
+    + align256(3 * (kNoAllocMaxVoxels + 1) * sizeof(int));        // output frequencies
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
 
@@ -816,39 +863,25 @@ int pattern_adapted_noalloc(const rf_grid* grid, const uint8_t* pm_host, int inc
   double2* tx = reinterpret_cast<double2*>(carve(kNoAllocMaxSide * sizeof(double2)));
   double2* ty = reinterpret_cast<double2*>(carve(kNoAllocMaxSide * sizeof(double2)));
   double2* tz = reinterpret_cast<double2*>(carve(kNoAllocMaxSide * sizeof(double2)));
-  auto* key = reinterpret_cast<unsigned long long*>(
+  // (the half spectrum never has more entries than the grid has voxels)
+  SelectScratch ss{};
+  ss.key = reinterpret_cast<unsigned long long*>(
       carve(kNoAllocMaxVoxels * sizeof(unsigned long long)));
-  int* lin = reinterpret_cast<int*>(carve(kNoAllocMaxVoxels * sizeof(int)));
-  int* size = reinterpret_cast<int*>(carve(kNoAllocMaxVoxels * sizeof(int)));
-  int* flags = reinterpret_cast<int*>(carve(kNoAllocMaxVoxels * sizeof(int)));
-  int* tot = reinterpret_cast<int*>(carve((kNoAllocMaxVoxels / 1024 + 2) * sizeof(int)));
-  auto* d_cnt = reinterpret_cast<unsigned long long*>(carve(sizeof(unsigned long long)));
-  auto* d_hist = reinterpret_cast<unsigned long long*>(carve(256 * sizeof(unsigned long long)));
-  int* d_out = reinterpret_cast<int*>(carve(3 * kNoAllocMaxVoxels * sizeof(int)));
+  ss.lin = reinterpret_cast<unsigned*>(carve(kNoAllocMaxVoxels * sizeof(unsigned)));
+  ss.tot = reinterpret_cast<int*>(carve((kNoAllocMaxVoxels / 1024 + 2) * sizeof(int)));
+  ss.st = reinterpret_cast<Select*>(carve(sizeof(Select)));
+  ss.hist = reinterpret_cast<unsigned*>(carve(kBins * sizeof(unsigned)));
+  ss.d_out = reinterpret_cast<int*>(carve(3 * (kNoAllocMaxVoxels + 1) * sizeof(int)));
 
-  // the transform and key kernels of rf_pattern_adapted
+  // the transform, key and selection code of rf_pattern_adapted on carved scratch; the state and
+  // the histogram, the only scratch that must start at zero, are cleared before every use
   if (int e = check(cudaMemcpyAsync(d_pm, pm_host, g.N, cudaMemcpyHostToDevice, s), "upload"))
     return e;
   double2* G = nullptr;
   if (int e = indicator_transform(g, d_pm, incl, A, B, tx, ty, tz, &G, s)) return e;
-  k_keys<<<(unsigned)((g.N + 255) / 256), 256, 0, s>>>(G, nullptr, g, key, lin, size);
+  k_keys<<<(unsigned)((half_size(g) + 255) / 256), 256, 0, s>>>(G, nullptr, g, ss.key, ss.lin);
   if (int e = check(cudaGetLastError(), "noalloc: keys")) return e;
-
-  // the selection code of rf_pattern_adapted, on carved scratch and host buffers on the stack
-  // (pageable: the copies complete before each read); the counter and the histogram, the only
-  // scratch that must start at zero, are cleared before every use
-  unsigned long long h_cnt = 0, h_hist[256];
-  const SelectScratch ss{d_cnt, d_hist, flags, tot, &h_cnt, h_hist};
-  unsigned long long thi = 0;
-  int tlin = 0;
-  long long K = 0;
-  if (int e = select_threshold(g, key, lin, size, k_target, s, ss, &thi, &tlin, &K)) return e;
-  *K_out = K;
-  if (K > cap) {
-    set_error("pattern: output capacity too small");
-    return RF_ERR_INVALID;
-  }
-  return compact_selection(g, key, lin, thi, tlin, K, d_out, out_host, s, ss);
+  return select_and_compact(g, ss, k_target, out_host, cap, K_out, s);
 }
 
 

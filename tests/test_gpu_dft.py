@@ -24,9 +24,9 @@ def rel(a, b):
     return float(np.linalg.norm(np.asarray(a) - b) / max(np.linalg.norm(b), 1e-300))
 
 
-def field(t):
-    g = t[0] if t.shape[0] == 1 else t
-    return np.stack([g[..., i, j] for (i, j) in VOIGT])
+def field(t, shape):
+    """oracle [Nz,Ny,Nx,3,3] -> [6, *shape]"""
+    return np.stack([t[..., i, j] for (i, j) in VOIGT]).reshape((6,) + tuple(shape))
 
 
 def check(lib, shape, phases, ratio, macro, full=False, n=3):
@@ -40,8 +40,8 @@ def check(lib, shape, phases, ratio, macro, full=False, n=3):
     co = s.rf_get_reduced_strain()
     s.close()
     r = O.solve(pm, phases, macro, pat, tol=0.0, max_iter=n)
-    assert rel(eps, field(r.eps)) <= EPS_TOL
-    assert rel(sig, field(r.sigma)) <= EPS_TOL
+    assert rel(eps, field(r.eps, shape)) <= EPS_TOL
+    assert rel(sig, field(r.sigma, shape)) <= EPS_TOL
     assert rel(out["sigma_bar"], r.sigma_bar) <= SBAR_TOL
     want = np.stack([r.eps_hat[:, i, j] for (i, j) in VOIGT], axis=1)
     assert rel(co[..., 0] + 1j * co[..., 1], want) <= EPS_TOL
