@@ -294,6 +294,8 @@ void release_pattern_buffers(rf_ctx* c) {
   dfree(c->d_bar);
   dfree(c->d_fin);
   dfree(c->d_zrange);
+  dfree(c->d_pmap);
+  dfree(c->d_red);
   dfree(c->d_Wi);
   dfree(c->d_Wf);
   dfree(c->d_ymap);
@@ -825,18 +827,16 @@ int rf_set_pattern(rf_ctx* c, const int32_t* freqs, int64_t K) {
     return (long long)(std::lower_bound(hk_sorted.begin(), hk_sorted.end(), hkey(kx, ky, kz)) -
                        hk_sorted.begin());
   };
-  c->map_h.assign(K, 0);
-  c->map_conj.assign(K, 0);
+  std::vector<int32_t> pmap(K);
   c->h_src.assign(c->Kh, -1);
   for (long long p = 0; p < K; ++p) {
     const int kx = freqs[3 * p], ky = freqs[3 * p + 1], kz = freqs[3 * p + 2];
     if (kx >= 0) {
-      c->map_h[p] = hpos(std::make_tuple(kx, ky, kz));
-      c->map_conj[p] = 0;
-      c->h_src[c->map_h[p]] = p;
+      const long long h = hpos(std::make_tuple(kx, ky, kz));
+      pmap[p] = (int32_t)h;
+      c->h_src[h] = p;
     } else {
-      c->map_h[p] = hpos(conj(kx, ky, kz));
-      c->map_conj[p] = 1;
+      pmap[p] = ~(int32_t)hpos(conj(kx, ky, kz));
     }
   }
   auto pos = [](const std::vector<int>& v, int x) {
@@ -885,6 +885,7 @@ int rf_set_pattern(rf_ctx* c, const int32_t* freqs, int64_t K) {
   if (!err) err = palloc(c, &c->d_kzm, c->Kz, "pattern");
   if (!err) err = palloc(c, &c->d_fac, c->Kx, "pattern");
   if (!err) err = palloc(c, &c->d_hidx, c->Kh, "pattern");
+  if (!err) err = palloc(c, &c->d_pmap, K, "pattern");
   if (!err) err = palloc(c, &c->d_hn, c->Kh, "pattern");
   if (!err) err = palloc(c, &c->d_ER, c->rect, "coefficients");
   if (!err) err = palloc(c, &c->d_T1, (size_t)c->rows * NCK, "line transforms");
@@ -934,6 +935,7 @@ int rf_set_pattern(rf_ctx* c, const int32_t* freqs, int64_t K) {
   if (!err) err = ck(cudaMemcpyAsync(c->d_fac, fac.data(), sizeof(float) * c->Kx, cudaMemcpyHostToDevice, c->stream), "up");
   if (!err) err = ck(cudaMemcpyAsync(c->d_hidx, c->h_hidx.data(), sizeof(HIdx) * c->Kh, cudaMemcpyHostToDevice, c->stream), "up");
   if (!err) err = ck(cudaMemcpyAsync(d_hk, hk.data(), sizeof(int) * hk.size(), cudaMemcpyHostToDevice, c->stream), "up");
+  if (!err) err = ck(cudaMemcpyAsync(c->d_pmap, pmap.data(), sizeof(int32_t) * K, cudaMemcpyHostToDevice, c->stream), "up");
   if (!err) err = launch_hinfo(c, d_hk, c->Kh);
   if (!err && c->d_jent) err = launch_gather_jentries(c);
   if (!err && fuse_ok && c->dim == 2) {
@@ -1154,32 +1156,14 @@ int rf_get_reduced_strain(rf_ctx* c, float* coeffs) {
     return RF_ERR_STATE;
   }
   DeviceGuard dg(c->dev);
-  std::vector<float2> er(c->rect);
-  if (int e = ck(cudaMemcpyAsync(er.data(), c->d_ER, sizeof(float2) * c->rect,
+  // in the pattern's order on the device: one copy of what the caller asked for (the rectangle of
+  // a 128^3 pattern is four times as large, and the host's gather over it took a millisecond)
+  if (int e = palloc(c, &c->d_red, (size_t)c->K * 6, "reduced strain")) return e;
+  if (int e = launch_gather_pattern(c)) return e;
+  if (int e = ck(cudaMemcpyAsync(coeffs, c->d_red, sizeof(float2) * 6 * c->K,
                                  cudaMemcpyDeviceToHost, c->stream), "copy coefficients"))
     return e;
-  if (int e = ck(cudaStreamSynchronize(c->stream), "sync")) return e;
-  for (long long p = 0; p < c->K; ++p) {
-    const HIdx& hi = c->h_hidx[c->map_h[p]];
-    const long long base = ((long long)(hi.iz * c->Ky + hi.iy) * c->nc) * c->Kx + hi.j;
-    const float sg = c->map_conj[p] ? -1.f : 1.f;
-    for (int i = 0; i < 6; ++i) {
-      int comp = -1;
-      if (c->nc == 6) comp = i;
-      else if (i == 0) comp = 0;
-      else if (i == 1) comp = 1;
-      else if (i == 5) comp = 2;
-      float re = 0.f, im = 0.f;
-      if (comp >= 0) {
-        const float2 v = er[base + (long long)comp * c->Kx];
-        re = v.x;
-        im = sg * v.y;
-      }
-      coeffs[(p * 6 + i) * 2] = re;
-      coeffs[(p * 6 + i) * 2 + 1] = im;
-    }
-  }
-  return RF_OK;
+  return ck(cudaStreamSynchronize(c->stream), "sync");
 }
 
 struct StateHeader {

@@ -482,6 +482,31 @@ int launch_scatter_full(rf_ctx* c, rf_ctx* f) {
   return launch_check(c, "scatter to the full set");
 }
 
+// Coefficients in the pattern's order, [K][6] (components outside the plane zero in 2D); one thread
+// per value, neighbouring threads write neighbouring words.
+__global__ void k_gather_pattern(const float2* ER, const HIdx* hidx, const int32_t* pmap,
+                                 long long K, int NC, int Kx, int Ky, float2* out) {
+  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (t >= 6 * K) return;
+  const long long p = t / 6;
+  const int i = (int)(t - 6 * p);
+  const int c = NC == 6 ? i : i == 0 ? 0 : i == 1 ? 1 : i == 5 ? 2 : -1;
+  float2 v = make_float2(0.f, 0.f);
+  if (c >= 0) {
+    const int m = pmap[p];
+    const HIdx hi = hidx[m < 0 ? ~m : m];
+    v = ER[((long long)(hi.iz * Ky + hi.iy) * NC + c) * Kx + hi.j];
+    if (m < 0) v.y = -v.y;
+  }
+  out[t] = v;
+}
+
+int launch_gather_pattern(rf_ctx* c) {
+  k_gather_pattern<<<(unsigned)((6 * c->K + 255) / 256), 256, 0, c->stream>>>(
+      c->d_ER, c->d_hidx, c->d_pmap, c->K, c->nc, c->Kx, c->Ky, c->d_red);
+  return launch_check(c, "gather pattern");
+}
+
 // Error measures of Sec. 5 between two stress fields [6][N] (tensor shear components, counted
 // twice in the Frobenius norm): per block, the sum over its voxels of |sig - ref| / |ref| in FP64
 // (voxels with |ref| = 0 add nothing), in a fixed order.
