@@ -12,6 +12,11 @@
 // the buffer's mbarrier. Either operand may be K-contiguous or M/N-contiguous in global memory
 // (the transposes of the backward pass); the conversion step writes the canonical layout.
 // Epilogues fuse bias, GELU (storing the pre-activation for the backward pass) and GELU'.
+// Minibatches give few 128 x 128 tiles, and one CTA then walks the whole K alone, staging bound
+// (64 x 512 x 512: 4 CTAs, 85 us). Such products take tiles of 32 columns and split K over a
+// cluster of up to eight CTAs; each leaves its partial tile in its own shared memory and adds
+// up a share of the columns over the cluster in rank order (loss and gradients of 64 RVEs with
+// their read-back: 566 -> 265 us).
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -33,9 +38,11 @@ using tc::smem_u32;
 
 constexpr int kTM = 128;                 // output rows per tile (tensor-memory lanes)
 constexpr int kTN = 128;                 // output columns per tile (tensor-memory columns)
+constexpr int kTNs = 32;                 // ... where K is split over a cluster
 constexpr int kChunk = 128;              // K bytes per staged chunk row
 constexpr int kTileBytes = kTM * kChunk; // 16 KB per operand chunk
-constexpr size_t kGemmSmem = 4 * kTileBytes + 64;
+// two buffers of both operands' chunks, barriers
+constexpr size_t gemm_smem(int tn) { return 2 * (kTileBytes + tn * kChunk) + 64; }
 
 enum { EPI_STORE = 0, EPI_BIAS = 1, EPI_BIAS_GELU = 2, EPI_DGELU = 3 };
 
@@ -94,15 +101,16 @@ __device__ __forceinline__ void put1(unsigned char* tile, int row, int k, float 
   }
 }
 
-// Stage rows [r0, r0 + 128) x K chunk [k0, k0 + per) of an operand. KC: the operand is
+// Stage rows [r0, r0 + ROWS) x K chunk [k0, k0 + per) of an operand. KC: the operand is
 // K-contiguous (element (row, k) at src[row ld + k]), else row-contiguous (src[k ld + row]).
-// Out-of-range elements are zero. ld and the base are multiples of 4 floats (checked on the
+// K values past the end are zero; rows past the end only feed outputs that are not stored and are
+// left alone. ld and the base are multiples of 4 floats (checked on the
 // host), so every float4 below starts inside its row and is 16-byte aligned.
-template <class E, bool KC>
+template <class E, bool KC, int ROWS>
 __device__ __forceinline__ void stage(unsigned char* tile, const float* __restrict__ src,
                                       long long ld, int rows, int r0, int K, int k0) {
   constexpr int per = kChunk / E::kBytes;
-  constexpr int items = kTM * per / 4 / 128;   // float4 per thread
+  constexpr int items = ROWS * per / 4 / 128;   // float4 per thread
   float4 v[items];
   if constexpr (KC) {
 #pragma unroll
@@ -122,13 +130,13 @@ __device__ __forceinline__ void stage(unsigned char* tile, const float* __restri
 #pragma unroll
     for (int i = 0; i < items; ++i) {
       const int it = threadIdx.x + i * 128;
-      put4<E>(tile, it / (per / 4), 4 * (it % (per / 4)), v[i]);
+      if (r0 + it / (per / 4) < rows) put4<E>(tile, it / (per / 4), 4 * (it % (per / 4)), v[i]);
     }
   } else {
 #pragma unroll
     for (int i = 0; i < items; ++i) {
       const int it = threadIdx.x + i * 128;
-      const int kk = it / (kTM / 4), r = 4 * (it % (kTM / 4));
+      const int kk = it / (ROWS / 4), r = 4 * (it % (ROWS / 4));
       const int k = k0 + kk, row = r0 + r;
       float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
       if (k < K && row < rows) {
@@ -142,7 +150,8 @@ __device__ __forceinline__ void stage(unsigned char* tile, const float* __restri
 #pragma unroll
     for (int i = 0; i < items; ++i) {
       const int it = threadIdx.x + i * 128;
-      const int kk = it / (kTM / 4), r = 4 * (it % (kTM / 4));
+      const int kk = it / (ROWS / 4), r = 4 * (it % (ROWS / 4));
+      if (r0 + r >= rows) continue;
       put1<E>(tile, r + 0, kk, v[i].x);
       put1<E>(tile, r + 1, kk, v[i].y);
       put1<E>(tile, r + 2, kk, v[i].z);
@@ -151,15 +160,36 @@ __device__ __forceinline__ void stage(unsigned char* tile, const float* __restri
   }
 }
 
-template <class E, bool AK, bool BK, int EPI>
+// one output with the epilogue
+template <int EPI>
+__device__ __forceinline__ void put_out(const GemmArgs& g, int m, int n, float x) {
+  if constexpr (EPI == EPI_BIAS) x += g.bias[n];
+  if constexpr (EPI == EPI_BIAS_GELU) {
+    x += g.bias[n];
+    if (g.Zout) g.Zout[(long long)m * g.ldz + n] = x;
+    x = gelu(x);
+  }
+  if constexpr (EPI == EPI_DGELU) x *= gelu_grad(g.Zin[(long long)m * g.ldz + n]);
+  g.C[(long long)m * g.ldc + n] = x;
+}
+
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// TN = kTN: one CTA per tile. TN = kTNs: gridDim.z CTAs of one cluster share a tile's K chunks.
+template <class E, bool AK, bool BK, int EPI, int TN>
 __global__ __launch_bounds__(128) void k_gemm(GemmArgs g) {
   constexpr int per = kChunk / E::kBytes;
+  constexpr int kPair = kTileBytes + TN * kChunk;   // one buffer: A chunk, B chunk
   extern __shared__ __align__(1024) unsigned char smem[];
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + 4 * kTileBytes);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + 2 * kPair);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 2);
   int* s_err = reinterpret_cast<int*>(tslot + 1);
   const int tid = threadIdx.x, warp = tid >> 5;
-  const int n0 = blockIdx.x * kTN, m0 = blockIdx.y * kTM;
+  const int n0 = blockIdx.x * TN, m0 = blockIdx.y * kTM;
+  const int S = TN == kTN ? 1 : gridDim.z, rank = TN == kTN ? 0 : blockIdx.z;
 
   if (tid == 0) {
     tc::mbar_init(&bars[0], 1);
@@ -170,25 +200,27 @@ __global__ __launch_bounds__(128) void k_gemm(GemmArgs g) {
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(tslot)),
-                 "r"(kTN));
+                 "r"(TN));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = *tslot;
-  const uint32_t id = tc::idesc<E>(kTM, kTN);
-  const int nch = (g.K + per - 1) / per;
+  const uint32_t id = tc::idesc<E>(kTM, TN);
+  const int all = (g.K + per - 1) / per;
+  // this CTA's chunks [ch0, ch0 + nch)
+  const int ch0 = all * rank / S, nch = all * (rank + 1) / S - ch0;
   bool ok = true;
 
   for (int c = 0; c < nch; ++c) {
     const int b = c & 1;
-    unsigned char* As = smem + b * 2 * kTileBytes;
+    unsigned char* As = smem + b * kPair;
     unsigned char* Bs = As + kTileBytes;
     // buffer b is free once the MMAs of chunk c - 2 completed
     if (c >= 2 && !tc::mbar_wait(&bars[b], ((c - 2) >> 1) & 1)) atomicOr(s_err, 1);
-    stage<E, AK>(As, g.A, g.lda, g.M, m0, g.K, c * per);
-    stage<E, BK>(Bs, g.B, g.ldb, g.N, n0, g.K, c * per);
+    stage<E, AK, kTM>(As, g.A, g.lda, g.M, m0, g.K, (ch0 + c) * per);
+    stage<E, BK, TN>(Bs, g.B, g.ldb, g.N, n0, g.K, (ch0 + c) * per);
     asm volatile("fence.proxy.async.shared::cta;");
     __syncthreads();
     ok = (*s_err == 0);
@@ -212,10 +244,10 @@ __global__ __launch_bounds__(128) void k_gemm(GemmArgs g) {
   __syncthreads();
   ok = (*s_err == 0);
   asm volatile("tcgen05.fence::after_thread_sync;");
-  if (ok) {
+  const uint32_t lane = (uint32_t)(32 * warp) << 16;
+  if constexpr (TN == kTN) {
     const int m = m0 + tid;
-    const uint32_t lane = (uint32_t)(32 * warp) << 16;
-    for (int c0 = 0; c0 < kTN && n0 + c0 < g.N; c0 += 16) {   // uniform across the CTA
+    for (int c0 = 0; ok && c0 < TN && n0 + c0 < g.N; c0 += 16) {   // uniform across the CTA
       float v[16];
       tc::tmem_ld16(tmem + lane + c0, v);
       if (m >= g.M) continue;
@@ -223,22 +255,43 @@ __global__ __launch_bounds__(128) void k_gemm(GemmArgs g) {
       for (int i = 0; i < 16; ++i) {
         const int n = n0 + c0 + i;
         if (n >= g.N) break;
-        float x = v[i];
-        if constexpr (EPI == EPI_BIAS) x += g.bias[n];
-        if constexpr (EPI == EPI_BIAS_GELU) {
-          x += g.bias[n];
-          if (g.Zout) g.Zout[(long long)m * g.ldz + n] = x;
-          x = gelu(x);
-        }
-        if constexpr (EPI == EPI_DGELU) x *= gelu_grad(g.Zin[(long long)m * g.ldz + n]);
-        g.C[(long long)m * g.ldc + n] = x;
+        put_out<EPI>(g, m, n, v[i]);
       }
     }
+  } else {
+    // the partial tile, column by column, into this CTA's staging buffers (its MMAs are done)
+    float* part = reinterpret_cast<float*>(smem);
+    for (int c0 = 0; c0 < TN; c0 += 16) {
+      float v[16];
+#pragma unroll
+      for (int i = 0; i < 16; ++i) v[i] = 0.f;
+      if (ok && nch > 0) tc::tmem_ld16(tmem + lane + c0, v);   // uniform across the CTA
+#pragma unroll
+      for (int i = 0; i < 16; ++i) part[(c0 + i) * kTM + tid] = v[i];
+    }
+    cluster_sync();
+    // this CTA's share of the columns, summed over the cluster in rank order
+    const int m = m0 + tid;
+    for (int c = TN * rank / S; c < TN * (rank + 1) / S; ++c) {
+      float x = 0.f;
+      for (int q = 0; q < S; ++q) {
+        uint32_t src;
+        asm("mapa.shared::cluster.u32 %0, %1, %2;"
+            : "=r"(src)
+            : "r"(smem_u32(part + c * kTM + tid)), "r"(q));
+        float y;
+        asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(y) : "r"(src) : "memory");
+        x += y;
+      }
+      if (m < g.M && n0 + c < g.N) put_out<EPI>(g, m, n0 + c, x);
+    }
+    __syncwarp();
+    cluster_sync();   // no CTA leaves while another still reads its tile
   }
   __syncthreads();
   asm volatile("tcgen05.fence::before_thread_sync;");
   if (warp == 0)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTN));
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TN));
   if (!ok && tid == 0) atomicOr(g.err, 1);
 }
 
@@ -404,13 +457,23 @@ __global__ __launch_bounds__(256) void k_slot_reduce(const rf_slot* __restrict__
   if (threadIdx.x < kOut) dO[(long long)r * ldo + threadIdx.x] = (float)(scal[0] * (double)acc);
 }
 
-// db[n] = sum_b D[b][n]
-__global__ void k_colsum(const float* __restrict__ D, long long ld, int B, int N, float* db) {
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= N) return;
+// db[n] = sum_b D[b][n]: 32 columns per block, row sums of eight warps added in order (one
+// thread per column walked all rows on two blocks: 7 us for 64 rows)
+__global__ __launch_bounds__(256) void k_colsum(const float* __restrict__ D, long long ld, int B,
+                                                int N, float* db) {
+  __shared__ float sh[8][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, n = blockIdx.x * 32 + lane;
   float s = 0.f;
-  for (int b = 0; b < B; ++b) s += D[(long long)b * ld + n];
-  db[n] = s;
+  if (n < N)
+    for (int b = w; b < B; b += 8) s += D[(long long)b * ld + n];
+  sh[w][lane] = s;
+  __syncthreads();
+  if (w == 0 && n < N) {
+    float t = sh[0][lane];
+#pragma unroll
+    for (int i = 1; i < 8; ++i) t += sh[i][lane];
+    db[n] = t;
+  }
 }
 
 // Adam over the flat parameter buffer (bias corrections c1 = 1 / (1 - beta1^t), c2 likewise)
@@ -497,6 +560,7 @@ struct rf_mlp {
   long long off[6] = {0, 0, 0, 0, 0, 0};
   long long total = 0;
   float *d_p = nullptr, *d_g = nullptr, *d_m = nullptr, *d_v = nullptr;
+  float* d_flat = nullptr;    // [n_params] parameters or gradients on their way to the host
   float *d_Z1 = nullptr, *d_H1 = nullptr, *d_Z2 = nullptr, *d_H2 = nullptr, *d_O = nullptr;
   float *d_dZ1 = nullptr, *d_dZ2 = nullptr;
   double* d_part = nullptr;   // [maxB][2] loss partials
@@ -529,15 +593,38 @@ template <class E, bool AK, bool BK, int EPI>
 int gemm(rf_mlp* n, const GemmArgs& a) {
   static bool attr = false;
   if (!attr) {
-    cudaFuncSetAttribute(k_gemm<E, AK, BK, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)kGemmSmem);
+    cudaFuncSetAttribute(k_gemm<E, AK, BK, EPI, kTN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)gemm_smem(kTN));
+    cudaFuncSetAttribute(k_gemm<E, AK, BK, EPI, kTNs>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)gemm_smem(kTNs));
     attr = true;
   }
   if (a.M < 1 || a.N < 1 || a.K < 1) return mfail("mlp gemm: empty operand");
   if ((a.lda & 3) || (a.ldb & 3) || !aligned16(a.A) || !aligned16(a.B))
     return mfail("mlp gemm: operands must be 16-byte aligned with leading dimensions % 4 == 0");
-  dim3 grid((a.N + kTN - 1) / kTN, (a.M + kTM - 1) / kTM);
-  k_gemm<E, AK, BK, EPI><<<grid, 128, kGemmSmem, n->stream>>>(a);
+  const dim3 grid((a.N + kTN - 1) / kTN, (a.M + kTM - 1) / kTM);
+  if (grid.x * grid.y >= 76) {   // wide tiles reach half the SMs: they stage the least
+    k_gemm<E, AK, BK, EPI, kTN><<<grid, 128, gemm_smem(kTN), n->stream>>>(a);
+    return launched(n, "mlp gemm");
+  }
+  // narrow tiles, and K over as many CTAs as keep two chunks each and about two CTAs per SM
+  const int chunks = (a.K * E::kBytes + kChunk - 1) / kChunk;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((a.N + kTNs - 1) / kTNs, grid.y, 1);
+  int S = 1;
+  while (S < 8 && 2 * S * 2 <= chunks && cfg.gridDim.x * cfg.gridDim.y * 2 * S <= 304) S *= 2;
+  cfg.gridDim.z = S;
+  cfg.blockDim = dim3(128);
+  cfg.dynamicSmemBytes = gemm_smem(kTNs);
+  cfg.stream = n->stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = S;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_gemm<E, AK, BK, EPI, kTNs>, a);
+  if (e != cudaSuccess) return cuda_fail(e, "mlp gemm");
   return launched(n, "mlp gemm");
 }
 
@@ -695,18 +782,6 @@ static void pack(const rf_mlp* n, const float* src, std::vector<float>& dst) {
     }
 }
 
-static void unpack(const rf_mlp* n, const std::vector<float>& src, float* dst) {
-  long long s = 0;
-  const long long rows[6] = {n->in, 1, n->H, 1, n->H, 1};
-  const long long cols[6] = {n->H, n->H, n->H, n->H, n->out, n->out};
-  const long long ld[6] = {n->H, n->H, n->H, n->H, n->out_ld, n->out_ld};
-  for (int i = 0; i < 6; ++i)
-    for (long long r = 0; r < rows[i]; ++r) {
-      std::memcpy(dst + s, &src[n->off[i] + r * ld[i]], sizeof(float) * cols[i]);
-      s += cols[i];
-    }
-}
-
 int rf_mlp_set_params(rf_mlp* n, const float* params) {
   if (!n || !params) return mfail("rf_mlp_set_params: null argument");
   std::vector<float> h;
@@ -721,23 +796,51 @@ int rf_mlp_set_params(rf_mlp* n, const float* params) {
   return RF_OK;
 }
 
-static int get_flat(const rf_mlp* n, const float* d, float* out, const char* what) {
+// padded rows -> the flat caller's order (one block per row of the six arrays)
+__global__ void k_unpack(const float* __restrict__ src, float* __restrict__ dst, int in, int H,
+                         int out, int out_ld) {
+  int r = blockIdx.x;
+  const int rows[6] = {in, 1, H, 1, H, 1};
+  long long so = 0, d = 0;
+  int cols = H, ld = H;
+  for (int i = 0; i < 6; ++i) {
+    cols = i < 4 ? H : out;
+    ld = i < 4 ? H : out_ld;
+    if (r < rows[i]) break;
+    r -= rows[i];
+    so += (long long)rows[i] * ld;
+    d += (long long)rows[i] * cols;
+  }
+  for (int c = threadIdx.x; c < cols; c += blockDim.x)
+    dst[d + (long long)r * cols + c] = src[so + (long long)r * ld + c];
+}
+
+// The padding of the rows goes on the device, so that one copy fills the caller's array (a copy
+// into a host buffer and row by row from there took as long again).
+static int get_flat(rf_mlp* n, const float* d, float* out, const char* what) {
   if (!n || !out) return mfail("rf_mlp_get: null argument");
-  std::vector<float> h(n->total);
-  cudaError_t e = cudaMemcpyAsync(h.data(), d, sizeof(float) * n->total, cudaMemcpyDeviceToHost,
+  const long long count = (long long)n->in * n->H + n->H + (long long)n->H * n->H + n->H +
+                          (long long)n->H * n->out + n->out;
+  if (!n->d_flat && cudaMalloc(&n->d_flat, sizeof(float) * count) != cudaSuccess) {
+    cudaGetLastError();
+    n->d_flat = nullptr;
+    return mfail("rf_mlp_get: out of device memory", RF_ERR_OOM);
+  }
+  k_unpack<<<n->in + 2 * n->H + 3, 128, 0, n->stream>>>(d, n->d_flat, n->in, n->H, n->out,
+                                                        n->out_ld);
+  if (int e = launched(n, what)) return e;
+  cudaError_t e = cudaMemcpyAsync(out, n->d_flat, sizeof(float) * count, cudaMemcpyDeviceToHost,
                                   n->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(n->stream);
-  if (e != cudaSuccess) return cuda_fail(e, what);
-  unpack(n, h, out);
-  return RF_OK;
+  return e == cudaSuccess ? RF_OK : cuda_fail(e, what);
 }
 
 int rf_mlp_get_params(const rf_mlp* n, float* params) {
-  return get_flat(n, n ? n->d_p : nullptr, params, "rf_mlp_get_params");
+  return get_flat(const_cast<rf_mlp*>(n), n ? n->d_p : nullptr, params, "rf_mlp_get_params");
 }
 
 int rf_mlp_get_grads(const rf_mlp* n, float* grads) {
-  return get_flat(n, n ? n->d_g : nullptr, grads, "rf_mlp_get_grads");
+  return get_flat(const_cast<rf_mlp*>(n), n ? n->d_g : nullptr, grads, "rf_mlp_get_grads");
 }
 
 int rf_mlp_forward(rf_mlp* n, int32_t B, const float* d_x, float* d_out, int32_t precision) {
@@ -807,7 +910,7 @@ int rf_mlp_loss_grad(rf_mlp* n, int32_t B, const float* d_x, const float* d_e,
   GemmArgs a = args(n->d_H2, n->H, n->d_O, n->out_ld, g + n->off[4], n->out_ld, n->H, n->out, B,
                     n->d_err);
   if (int e = gemm<ETf32, false, false, EPI_STORE>(n, a)) return e;
-  k_colsum<<<(n->out + 255) / 256, 256, 0, n->stream>>>(n->d_O, n->out_ld, B, n->out,
+  k_colsum<<<(n->out + 31) / 32, 256, 0, n->stream>>>(n->d_O, n->out_ld, B, n->out,
                                                          g + n->off[5]);
   if (int e = launched(n, "mlp colsum")) return e;
   // dZ2 = (dO W3^T) * GELU'(Z2)
@@ -818,7 +921,7 @@ int rf_mlp_loss_grad(rf_mlp* n, int32_t B, const float* d_x, const float* d_e,
   // dW2 = H1^T dZ2, db2
   a = args(n->d_H1, n->H, n->d_dZ2, n->H, g + n->off[2], n->H, n->H, n->H, B, n->d_err);
   if (int e = gemm<ETf32, false, false, EPI_STORE>(n, a)) return e;
-  k_colsum<<<(n->H + 255) / 256, 256, 0, n->stream>>>(n->d_dZ2, n->H, B, n->H, g + n->off[3]);
+  k_colsum<<<(n->H + 31) / 32, 256, 0, n->stream>>>(n->d_dZ2, n->H, B, n->H, g + n->off[3]);
   if (int e = launched(n, "mlp colsum")) return e;
   // dZ1 = (dZ2 W2^T) * GELU'(Z1)
   a = args(n->d_dZ2, n->H, W2, n->H, n->d_dZ1, n->H, B, n->H, n->H, n->d_err);
@@ -828,7 +931,7 @@ int rf_mlp_loss_grad(rf_mlp* n, int32_t B, const float* d_x, const float* d_e,
   // dW1 = X^T dZ1, db1
   a = args(d_x, n->in, n->d_dZ1, n->H, g + n->off[0], n->H, n->in, n->H, B, n->d_err);
   if (int e = gemm<ETf32, false, false, EPI_STORE>(n, a)) return e;
-  k_colsum<<<(n->H + 255) / 256, 256, 0, n->stream>>>(n->d_dZ1, n->H, B, n->H, g + n->off[1]);
+  k_colsum<<<(n->H + 31) / 32, 256, 0, n->stream>>>(n->d_dZ1, n->H, B, n->H, g + n->off[1]);
   if (int e = launched(n, "mlp colsum")) return e;
   if (loss) {
     if (int e = sync_read(n)) return e;
@@ -883,6 +986,7 @@ int rf_mlp_destroy(rf_mlp* n) {
   if (n->stream) cudaStreamSynchronize(n->stream);
   cudaFree(n->d_p);
   cudaFree(n->d_g);
+  cudaFree(n->d_flat);
   cudaFree(n->d_m);
   cudaFree(n->d_v);
   cudaFree(n->d_Z1);
