@@ -1159,6 +1159,8 @@ __global__ __launch_bounds__(kResThreads, 2) void kb_resident(BArgs a, const int
   }
 }
 
+#include "rf_batch_cell.cuh"
+
 __global__ __launch_bounds__(256) void kb_row(BArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ double red[8];
@@ -1702,6 +1704,9 @@ struct rf_batch {
   int* d_order = nullptr;          // RVEs, largest first
   unsigned* d_queue = nullptr;
   float2* d_scratch = nullptr;
+  // cell-resident solve (kb_cell): pruned DFTs on every RVE, each fits a block's shared memory
+  size_t cell_smem = 0;            // 0: the batch does not qualify
+  int cell = 0;                    // 1: solves run as kb_cell
 };
 
 using namespace rfk;
@@ -2120,6 +2125,19 @@ int launch_resident(rf_batch* b) {
   return e == cudaSuccess ? RF_OK : bfail(e, "batch resident");
 }
 
+int launch_cell(rf_batch* b) {
+  cudaError_t e = cudaMemsetAsync(b->d_queue, 0, sizeof(unsigned), b->stream);
+  if (e != cudaSuccess) return bfail(e, "batch cells");
+  int sms = 152;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->dev);
+  kb_cell<<<std::min(b->n, sms), kCellThreads, b->cell_smem, b->stream>>>(batch_args(b, -1),
+                                                                          b->d_order, b->n,
+                                                                          b->d_queue);
+  b->launches += 1;
+  e = cudaGetLastError();
+  return e == cudaSuccess ? RF_OK : bfail(e, "batch cells");
+}
+
 int run_solve(rf_batch* b, const double* macro, bool use_warm, const float2* pwarm = nullptr) {
   if (int e = set_status(b, macro)) return e;
   BArgs a = batch_args(b, -1);
@@ -2130,6 +2148,10 @@ int run_solve(rf_batch* b, const double* macro, bool use_warm, const float2* pwa
   if (b->resident) {
     b->last_while = false;
     return launch_resident(b);
+  }
+  if (b->cell) {
+    b->last_while = false;
+    return launch_cell(b);
   }
   return iterate(b);
 }
@@ -2230,8 +2252,11 @@ int autotune(rf_batch* b, const double* macro) {
   // options.batch_resident: -1 never, 1 always (where the batch qualifies), 0 the faster of a
   // three-update solve each way (the sweeps without their final pass, the resident kernel with)
   b->resident = 0;
+  b->cell = 0;
   if (!err && b->res_ok && b->opt.batch_resident > 0) b->resident = 1;
-  if (!err && b->res_ok && b->opt.batch_resident == 0) {
+  // the cell-resident solve (pruned DFTs) against the sweeps in the same way, unless -1
+  const bool try_res = b->res_ok && b->opt.batch_resident == 0;
+  if (!err && (try_res || b->cell_smem > 0)) {
     auto time_solve = [&](bool res, float* ms) -> int {
       *ms = 1e30f;
       for (int rep = 0; rep < 2; ++rep) {
@@ -2240,7 +2265,7 @@ int autotune(rf_batch* b, const double* macro) {
         kb_init<<<b->n, 256, 0, b->stream>>>(batch_args(b, -1), b->n, nullptr, b->d_warm_off,
                                              nullptr);
         if (res) {
-          if (int e = launch_resident(b)) return e;
+          if (int e = try_res ? launch_resident(b) : launch_cell(b)) return e;
         } else {
           for (int i = 0; i < 3; ++i)
             if (int e = launch_update(b)) return e;
@@ -2257,7 +2282,7 @@ int autotune(rf_batch* b, const double* macro) {
     float t_sweep = 0.f, t_res = 0.f;
     err = time_solve(false, &t_sweep);
     if (!err) err = time_solve(true, &t_res);
-    if (!err) b->resident = t_res < t_sweep ? 1 : 0;
+    if (!err && t_res < t_sweep) (try_res ? b->resident : b->cell) = 1;
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
@@ -2269,7 +2294,7 @@ int finish_solve(rf_batch* b, double* hom_stress, int32_t* iters, double* residu
                  int32_t* status) {
   // final pass: fields of the converged coefficients -> homogenised stresses (kb_resident
   // ran its own)
-  if (!b->resident) {
+  if (!b->resident && !b->cell) {
     BArgs a0 = batch_args(b, 0);
     a0.final_pass = 1;
     if (b->n_items[0] > 0) kb_inv_y<<<b->grid, 256, b->col_smem, b->stream>>>(a0);
@@ -2631,10 +2656,27 @@ int rf_batch_create(rf_batch** out, int32_t n_rve, const rf_grid* grids,
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kb_resident, kResThreads, kResSmem);
       b->res_grid = sms * std::max(1, per_sm);
       b->res_slot = (slot + 1) & ~1LL;   // 16-byte aligned slots
+      if (!err) err = balloc(&b->d_scratch, (size_t)b->res_grid * b->res_slot, "batch scratch");
+    }
+    // the cell-resident solve: pruned DFTs along both axes of every RVE, in shared memory
+    size_t cell = 0;
+    auto fft_side = [&](int v) {
+      const int p2 = v % 3 == 0 ? v / 3 : v;
+      return b->use_fft && (p2 & (p2 - 1)) == 0;
+    };
+    for (const BDesc& d : b->desc) {
+      const bool fits = !fft_side(d.nx) && !fft_side(d.ny) && (d.nx / 2 + 2) / 2 <= kCellThreads;
+      cell = std::max(cell, fits ? cell_layout(d.nx, d.ny, d.Kx, d.Ky, d.Kh).bytes
+                                 : kCellSmemMax + 1);
+    }
+    if (cell <= kCellSmemMax && opt->batch_resident >= 0) {
+      b->cell_smem = cell;
+      cudaFuncSetAttribute(kb_cell, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCellSmemMax);
+    }
+    if (b->res_ok || b->cell_smem > 0) {
       if (!err) err = balloc(&b->d_order, order.size(), "batch queue");
       up(b->d_order, order.data(), sizeof(int) * order.size());
       if (!err) err = balloc(&b->d_queue, 1, "batch queue");
-      if (!err) err = balloc(&b->d_scratch, (size_t)b->res_grid * b->res_slot, "batch scratch");
     }
   }
   if (!err) {
