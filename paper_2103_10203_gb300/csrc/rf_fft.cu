@@ -1348,6 +1348,10 @@ int fft_autotune(rf_ctx* c) {
       hs.mu0 = c->mu0;
       float ms = 1e30f;
       const int e = time_it([&] {
+        if (mode != kColPersistW && c->team_on) {
+          if (int e2 = launch_team_begin(c, hs.ebar, 2)) return e2;
+          return launch_team_solve(c, nullptr, 0);
+        }
         if (int e2 = tck(cudaMemcpyAsync(c->d_status, c->h_status, sizeof(Status),
                                          cudaMemcpyHostToDevice, c->stream), "tuner"))
           return e2;

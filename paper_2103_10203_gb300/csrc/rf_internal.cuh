@@ -204,7 +204,7 @@ struct rf_ctx {
   size_t persist_smem = 0;
   // the persistent solve on team FFTs (rf_team.cu), used by kColPersistent where it is faster:
   // blocks, and the same number when they form one cluster (0: a co-resident grid)
-  bool team_on = false;
+  bool team_on = false, team_stream = false;
   int team_G = 0, team_cluster = 0, team_threads = 0;
   bool final_queued = false;            // the final pass went out behind the solve (rf_team.cu)
   double* d_fin = nullptr;              // [blocks][8] partials of the team solve's final pass

@@ -70,7 +70,7 @@ int lanes_of(int L) {
   switch (L) {
 #define X(L_, R, M) \
   case L_: return R * M;
-    RF_TEAM_SIDES(X)
+    RF_TEAM_SIDES_2D(X)
 #undef X
   }
   return 0;
@@ -79,7 +79,7 @@ int twiddles_of(int L) {
   switch (L) {
 #define X(L_, R, M) \
   case L_: return Plan<R, M>::kTw;
-    RF_TEAM_SIDES(X)
+    RF_TEAM_SIDES_2D(X)
 #undef X
   }
   return 0;
@@ -93,7 +93,7 @@ Kernel solve_kernel(const rf_ctx* c) {
 
 // Block shape of a launch on G blocks with `W` workers at most: teams per block, rounds, shared
 // memory; false if a round's teams or the shared memory do not fit.
-bool shape(const rf_ctx* c, int G, bool final_pass, Args& a, size_t* smem) {
+bool shape_with(const rf_ctx* c, int G, bool final_pass, bool stream, Args& a, size_t* smem) {
   const int gx = 3 * lanes_of(c->nx), gy = 3 * lanes_of(c->ny);
   const int units = c->ny / 2;
   const int ux = (units + G - 1) / G, uy = (c->Kx + G - 1) / G;   // per block, at most
@@ -118,7 +118,8 @@ bool shape(const rf_ctx* c, int G, bool final_pass, Args& a, size_t* smem) {
   const size_t by = final_pass ? 0 : (size_t)a.Py * 6 * (c->ny + c->ny / 16 + 2);
   a.o_buf = take(sizeof(float2) * std::max(bx, by));
   if (!final_pass) {
-    a.o_twy = take(sizeof(float2) * twiddles_of(c->ny));
+    // (a square cell's transforms share the table)
+    a.o_twy = c->nx == c->ny ? a.o_twx : take(sizeof(float2) * twiddles_of(c->ny));
     a.o_red = take(sizeof(double) * a.W);
     a.o_eb = take(sizeof(double) * 8);
     const int nslot = a.Py * a.rounds_y;
@@ -132,7 +133,9 @@ bool shape(const rf_ctx* c, int G, bool final_pass, Args& a, size_t* smem) {
     }
     a.o_en = take(sizeof(float4) * a.entries_cap);
     a.o_ep = take(sizeof(int) * a.entries_cap);
-    a.o_st = take((size_t)a.Px * a.rounds_x * 2 * c->nx * (c->has_plastic ? 17 : 1));
+    a.st_stream = stream;
+    a.o_p8 = take((size_t)a.Px * a.rounds_x * 2 * c->nx);
+    a.o_st = take(!c->has_plastic ? 0 : (size_t)a.Px * (stream ? 1 : a.rounds_x) * 2 * c->nx * 16);
     if (a.cluster) {
       a.o_ts = take(sizeof(float4) * 3 * (size_t)a.Px * a.rounds_x * c->Kx);
       a.o_tp = take(sizeof(float2) * 3 * (size_t)nslot * c->ny);
@@ -140,6 +143,10 @@ bool shape(const rf_ctx* c, int G, bool final_pass, Args& a, size_t* smem) {
   }
   *smem = o;
   return gx <= kMaxWorkers && gy <= kMaxWorkers && o <= kSmemMax;
+}
+
+bool shape(const rf_ctx* c, int G, bool final_pass, Args& a, size_t* smem) {
+  return shape_with(c, G, final_pass, c->team_stream, a, smem);
 }
 
 Args make_args(rf_ctx* c) {
@@ -202,6 +209,7 @@ bool team_geometry(rf_ctx* c, int cluster) {
   Args a{};
   size_t smem = 0;
   const int units = c->ny / 2;
+  c->team_stream = false;
   if (cluster > 0) {
     a.cluster = 1;
     if (cluster > units || !shape(c, cluster, false, a, &smem)) return false;
@@ -225,7 +233,12 @@ bool team_geometry(rf_ctx* c, int cluster) {
   } else {
     const int sms = sm_count(c);
     bool found = false;
-    for (int per = 4; per >= 1 && !found; --per) {
+    // as many blocks per SM as it takes to give each a row pair of its own; internal variables
+    // held where that leaves room for them, else streamed
+    for (int q = 0; q < 8 && !found; ++q) {
+      const int per = 4 - q / 2;
+      c->team_stream = q & 1;
+      if (c->team_stream && !c->has_plastic) continue;
       const int G = std::min(units, per * sms);
       if (per > 1 && G <= (per - 1) * sms) continue;   // fewer blocks per SM hold it
       int occ = 0;
@@ -250,7 +263,7 @@ void init_attributes_team() {
 #define X(L, R, M) \
   all.push_back(kernel_plastic(L)); \
   all.push_back(kernel_elastic(L));
-  RF_TEAM_SIDES(X)
+  RF_TEAM_SIDES_2D(X)
 #undef X
   for (Kernel k : all) {
     cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);

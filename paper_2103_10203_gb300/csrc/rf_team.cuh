@@ -16,15 +16,19 @@
 //     position to kx index, most positions empty): no zeroed buffer, no scatter, and one load
 //     latency. The reduced coefficients of a kx stay in the shared memory of the block that owns
 //     it for the whole solve (dense along y, zeros outside the pattern), as do the phase ids and
-//     internal variables of its rows.
+//     internal variables of its rows (of large J2 cells the internal variables are fetched by
+//     asynchronous copies behind the inverse transform of their rows).
 //   - the decision of update u (the same in every block, from block partials in a fixed order)
 //     is taken by a warp of its own while the other warps already run the row phase of update
 //     u + 1, which writes only scratch; a finished solve leaves after that phase.
 //   - one arrival and one poll per grid barrier on a counter that only grows; or, for small
 //     cells, the whole grid is one thread-block cluster: its hardware barrier, and the line
 //     transforms are written straight into the shared memory of the block that reads them.
-// Line transforms in global memory are column-major, T[(c Kx + j) Ny + y], as in the other
-// persistent solve; data of other blocks is read through L2. A second kernel runs the final pass.
+// Line transforms in global memory lie as their reader takes them, the strain lines by row pair,
+// [u][3][Kx][2 rows], the polarization lines by column, [(c Kx + j) Ny + y]: whole sectors are read
+// and 16 bytes written at a time (both by column, the row phase of a 512^2 update took 6.9 us, so
+// 6.2 us, and of a 1024^2 update 35 us, so 23 us). Data of other blocks is read through L2. A
+// second kernel runs the final pass.
 #pragma once
 
 #include <algorithm>
@@ -41,8 +45,8 @@ namespace team {
 constexpr int kMaxWorkers = 384;   // threads of all teams of a block
 
 struct Args {
-  float2* T1;            // strain lines, [(c Kx + j) Ny + y]
-  float2* T1p;           // polarization lines, same layout
+  float2* T1;            // strain lines, [u][3][Kx][2 rows]
+  float2* T1p;           // polarization lines, [(c Kx + j) Ny + y]
   float2* ER;            // [Ky][NC][Kx]
   const uint8_t* phase;
   float* state;
@@ -58,9 +62,10 @@ struct Args {
   int Px, Py;            // teams per block in the row and the column phase
   int rounds_x, rounds_y;   // row pairs and kx of one team, at most
   int cluster;           // the grid is one cluster
+  int st_stream;         // internal variables copied per row pair instead of held
   int entries_cap;       // pattern entries a block holds, at most
   // shared-memory offsets in bytes
-  int o_twx, o_twy, o_buf, o_w, o_en, o_ep, o_jmap, o_kx, o_slot, o_st, o_ph, o_red, o_eb;
+  int o_twx, o_twy, o_buf, o_w, o_en, o_ep, o_jmap, o_kx, o_slot, o_st, o_p8, o_ph, o_red, o_eb;
   int o_ts, o_tp;        // cluster: strain lines [slot][3][Kx][2 rows], polarization [slot][3][Ny]
   long long N;
   float invN;
@@ -193,6 +198,19 @@ __device__ __forceinline__ void row_phase(const Args& a, double* sb) {
     const int u = blockIdx.x + gridDim.x * (team + a.Px * rd);
     const bool on = team < a.Px && u < units;
     const int row0 = 2 * u;
+    if (PLASTIC && !FINAL && a.st_stream && on) {
+      // the pair's internal variables, plane by plane [4][2 L], 16 bytes per copy
+      float* sd = at<float>(a.o_st) + team * 8 * L;
+      constexpr int per = 2 * L / 4;
+      for (int i = w; i < 4 * per; i += 3 * G) {
+        const int p = i / per, o = 4 * (i - p * per);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                         (unsigned)__cvta_generic_to_shared(sd + p * 2 * L + o)),
+                     "l"(a.state + p * a.N + (long long)row0 * L + o)
+                     : "memory");
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    }
     float2 v[R];
     const int row = row0 + (seq == 1 ? 1 : 0);   // the row whose voxels this thread takes (seq < 2)
     const int slot = team + a.Px * rd;
@@ -204,9 +222,10 @@ __device__ __forceinline__ void row_phase(const Args& a, double* sb) {
         const int p = t + G * q;
         const int j = jmap[p <= L / 2 ? p : L - p];
         ca[q] = cb[q] = make_float2(0.f, 0.f);
+        // the pair's lines [3][Kx][2 rows]
+        const int o = ((seq < 2 ? 0 : 2) * Kx + j) * 2;
         if (j >= 0 && !FINAL && a.cluster) {
-          // [slot][3][Kx][2 rows]
-          const float2* s = at<float2>(a.o_ts) + ((slot * 3 + (seq < 2 ? 0 : 2)) * Kx + j) * 2;
+          const float2* s = at<float2>(a.o_ts) + slot * 6 * Kx + o;
           if (seq < 2) {
             ca[q] = s[seq];
             cb[q] = s[2 * Kx + seq];
@@ -215,13 +234,12 @@ __device__ __forceinline__ void row_phase(const Args& a, double* sb) {
             cb[q] = s[1];
           }
         } else if (j >= 0) {
+          const float2* s = a.T1 + (long long)u * 6 * Kx + o;
           if (seq < 2) {
-            const float2* s = a.T1 + (long long)j * Ny + row;
-            ca[q] = __ldcg(s);
-            cb[q] = __ldcg(s + (long long)Kx * Ny);
+            ca[q] = __ldcg(s + seq);
+            cb[q] = __ldcg(s + 2 * Kx + seq);
           } else {
-            const float4 f =
-                __ldcg(reinterpret_cast<const float4*>(a.T1 + (long long)(2 * Kx + j) * Ny + row0));
+            const float4 f = __ldcg(reinterpret_cast<const float4*>(s));
             ca[q] = make_float2(f.x, f.y);
             cb[q] = make_float2(f.z, f.w);
           }
@@ -250,6 +268,7 @@ __device__ __forceinline__ void row_phase(const Args& a, double* sb) {
         for (int q = 0; q < R; ++q) x[sw(t + G * q)] = v[q];
       }
     }
+    if (PLASTIC && !FINAL && a.st_stream) asm volatile("cp.async.wait_all;" ::: "memory");
     workers_sync(a.W);
     if (FINAL) {
       if (on) final_voxels<L, PLASTIC>(a, base + (M == 1 ? span : 0), 2 * span, row0, w, 3 * G, phs, sb);
@@ -257,10 +276,10 @@ __device__ __forceinline__ void row_phase(const Args& a, double* sb) {
       continue;
     }
     if (on && seq < 2) {
-      const uint8_t* ph8 = at<uint8_t>(a.o_st);   // phase ids, then the internal variables
+      const uint8_t* ph8 = at<uint8_t>(a.o_p8);
       const float4* st4 = at<float4>(a.o_st);
+      const float* sd = at<float>(a.o_st) + team * 8 * L + seq * L;
       const int rs = (slot * 2 + seq) * L;
-      if (PLASTIC) ph8 += (long long)a.rounds_x * a.Px * 2 * L * 16;
 #pragma unroll
       for (int q = 0; q < R; ++q) {
         const int x = t + G * q;
@@ -270,7 +289,8 @@ __device__ __forceinline__ void row_phase(const Args& a, double* sb) {
         float ep[6] = {0, 0, 0, 0, 0, 0};
         float alpha = 0.f;
         if (PLASTIC) {
-          const float4 s = st4[rs + x];
+          const float4 s = a.st_stream ? make_float4(sd[x], sd[2 * L + x], sd[4 * L + x], sd[6 * L + x])
+                                       : st4[rs + x];
           ep[0] = s.x;
           ep[1] = s.y;
           ep[5] = s.z;
@@ -447,9 +467,12 @@ __device__ __forceinline__ void col_phase(const Args& a, bool full) {
                     v[q]);
         }
       } else {
-        float2* d = a.T1 + (long long)(c * Kx + j) * L + t;
+        float2* d = a.T1 + (c * Kx + j) * 2;
 #pragma unroll
-        for (int q = 0; q < R; ++q) __stcg(d + G * q, v[q]);
+        for (int q = 0; q < R; ++q) {
+          const int y = t + G * q;
+          __stcg(d + (long long)(y >> 1) * 6 * Kx + (y & 1), v[q]);
+        }
       }
     }
     if (full && ((int)blockIdx.x + (int)gridDim.x * a.Py * (rd + 1) >= Kx || rd + 1 == a.rounds_y)) {
@@ -467,7 +490,7 @@ __device__ __forceinline__ void rows(const Args& a, double* sb) {
   switch (SIDE ? SIDE : a.Nx) {
 #define X(L, R, M) \
   case L: row_phase<R, M, PLASTIC, FINAL>(a, sb); break;
-    RF_TEAM_SIDES(X)
+    RF_TEAM_SIDES_2D(X)
 #undef X
   }
 }
@@ -477,7 +500,7 @@ __device__ __forceinline__ void cols(const Args& a, bool full) {
   switch (SIDE ? SIDE : a.Ny) {
 #define X(L, R, M) \
   case L: col_phase<R, M>(a, full); break;
-    RF_TEAM_SIDES(X)
+    RF_TEAM_SIDES_2D(X)
 #undef X
   }
 }
@@ -486,7 +509,7 @@ __device__ inline void fill_twiddles(int L, const float2* tab, float2* tw) {
   switch (L) {
 #define X(L_, R, M) \
   case L_: Plan<R, M>::twiddles(tab, tw); break;
-    RF_TEAM_SIDES(X)
+    RF_TEAM_SIDES_2D(X)
 #undef X
   }
 }
@@ -567,14 +590,13 @@ __global__ __launch_bounds__(kMaxWorkers + 32, 1) void k_team2d(const __grid_con
   {
     const int units = a.Ny / 2, L = a.Nx;
     const int nu = (int)blockIdx.x < units ? (units - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
-    uint8_t* ph8 = at<uint8_t>(a.o_st);
+    uint8_t* ph8 = at<uint8_t>(a.o_p8);
     float4* st4 = at<float4>(a.o_st);
-    if (PLASTIC) ph8 += (long long)a.rounds_x * a.Px * 2 * L * 16;
     for (int i = tid; i < nu * 2 * L; i += nt) {
       const int s = i / (2 * L), r = i - s * 2 * L;
       const long long g = (long long)2 * (blockIdx.x + gridDim.x * s) * L + r;
       ph8[i] = a.phase[g];
-      if (PLASTIC)
+      if (PLASTIC && !a.st_stream)
         st4[i] = make_float4(a.state[g], a.state[a.N + g], a.state[2 * a.N + g], a.state[3 * a.N + g]);
     }
   }
@@ -686,7 +708,7 @@ __global__ __launch_bounds__(kMaxWorkers + 32, 1) void k_team2d(const __grid_con
     const int nu = (int)blockIdx.x < units ? (units - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
     for (int i = tid; i < nu * 3 * a.Kx; i += nt) {
       const int s = i / (3 * a.Kx), q = i - s * 3 * a.Kx;   // q = c Kx + j
-      reinterpret_cast<float4*>(a.T1)[((long long)q * a.Ny >> 1) + blockIdx.x + gridDim.x * s] =
+      reinterpret_cast<float4*>(a.T1)[(long long)(blockIdx.x + gridDim.x * s) * 3 * a.Kx + q] =
           at<float4>(a.o_ts)[i];
     }
   }

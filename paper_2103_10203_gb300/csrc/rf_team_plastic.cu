@@ -8,7 +8,7 @@ Kernel kernel_plastic(int side) {
   switch (side) {
 #define X(L, R, M) \
   case L: return k_team2d<L, true>;
-    RF_TEAM_SIDES(X)
+    RF_TEAM_SIDES_2D(X)
 #undef X
   }
   return nullptr;

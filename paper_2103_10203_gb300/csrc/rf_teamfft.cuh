@@ -82,6 +82,45 @@ struct Dft<8, S> {   // 2 x 4
   }
 };
 
+template <int S>
+struct Dft<12, S> {   // 4 x 3: n = 4 a + b, q = q3 + 3 q4
+  static __device__ __forceinline__ void run(float2* v) {
+    float2 w[4][3];
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+#pragma unroll
+      for (int a = 0; a < 3; ++a) w[b][a] = v[4 * a + b];
+      Dft<3, S>::run(w[b]);
+    }
+    // exp(S 2 pi i b q3 / 12)
+    const float h = 0.86602540378443865f, s = (float)S;
+    w[1][1] = cmul(w[1][1], make_float2(h, 0.5f * s));
+    w[1][2] = cmul(w[1][2], make_float2(0.5f, h * s));
+    w[2][1] = cmul(w[2][1], make_float2(0.5f, h * s));
+    w[2][2] = cmul(w[2][2], make_float2(-0.5f, h * s));
+    w[3][1] = make_float2(-s * w[3][1].y, s * w[3][1].x);
+    w[3][2] = make_float2(-w[3][2].x, -w[3][2].y);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      float2 u[4] = {w[0][q], w[1][q], w[2][q], w[3][q]};
+      Dft<4, S>::run(u);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) v[q + 3 * k] = u[k];
+    }
+  }
+};
+template <int S>
+struct Dft<16, S> {
+  static __device__ __forceinline__ void run(float2* v) {
+    fftc::dft16(v, S);
+    float2 u[16];
+#pragma unroll
+    for (int q = 0; q < 16; ++q) u[q] = v[4 * (q & 3) + (q >> 2)];
+#pragma unroll
+    for (int q = 0; q < 16; ++q) v[q] = u[q];
+  }
+};
+
 // ---- the three passes of a sequence of L = R M R points, thread t < G = R M of its team
 template <int R, int M>
 struct Plan {
@@ -152,6 +191,9 @@ struct Plan {
 #define RF_TEAM_SIDES(X) \
   X(32, 4, 2) X(48, 4, 3) X(64, 8, 1) X(96, 4, 6) X(128, 8, 2) X(192, 8, 3) X(256, 8, 4) \
   X(384, 8, 6) X(512, 8, 8)
+
+// ... and the longer ones that only the persistent 2D solve takes
+#define RF_TEAM_SIDES_2D(X) RF_TEAM_SIDES(X) X(768, 8, 12) X(1024, 8, 16)
 
 }  // namespace team
 }  // namespace rfk

@@ -2,7 +2,7 @@
 persistent 2D solve and the 3D updates, at every side they take, against the oracle.
 
 Tolerances as in test_gpu_parity.py: relative L2 error of fields and coefficients 1e-5 (FP32
-transforms of at most 512 points: some ten roundings of 2^-24 per pass, three passes per
+transforms of at most 1024 points: some ten roundings of 2^-24 per pass, three passes per
 direction and a handful of updates stay two orders below), homogenised stress 1e-6.
 """
 
@@ -64,7 +64,8 @@ def check(lib, pm, phases, pat, macro, n=4, **opts):
 
 @pytest.mark.parametrize("shape", [(32, 32), (48, 48), (64, 64), (96, 96), (128, 128), (192, 192),
                                    (256, 256), (384, 384), (512, 512), (32, 512), (96, 48),
-                                   (384, 64), (128, 192)])
+                                   (384, 64), (128, 192), (768, 768), (1024, 1024),
+                                   (64, 1024), (1024, 32), (768, 48), (96, 768)])
 @pytest.mark.parametrize("plastic", [False, True])
 def test_persistent_solve_sides(lib, shape, plastic):
     """Every side of the plans, square and mixed; a pattern of a few per cent."""
