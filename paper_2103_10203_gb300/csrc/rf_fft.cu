@@ -987,10 +987,12 @@ int fft_autotune(rf_ctx* c) {
   const bool warp_need = c->fft_colmode == kColWarp || c->fft_colmode == kColPersistW;
   const bool warp_auto = !rows_pinned && c->opt.fft_row_warps == 0 && row_warp_ok(c) && !warp_need;
   // the persistent solve: compared with the other modes (fft_fuse 0, unless the row kernel's
-  // tiles are pinned) or only its geometry chosen (fft_fuse 3); needs the barrier words set up
-  // with the pattern
-  const bool persist_auto = c->dim == 2 && c->d_jptr && c->d_bar &&
-                            ((c->opt.fft_fuse == 0 && !rows_pinned) || c->opt.fft_fuse == 3);
+  // tiles are pinned or its warp-FFT form asked for) or only its geometry chosen (fft_fuse 3);
+  // needs the barrier words set up with the pattern
+  const bool row_warp_pinned = c->opt.fft_row_warps > 0 && row_warp_ok(c);
+  const bool persist_auto =
+      c->dim == 2 && c->d_jptr && c->d_bar &&
+      ((c->opt.fft_fuse == 0 && !rows_pinned && !row_warp_pinned) || c->opt.fft_fuse == 3);
   if (rows_pinned && c->opt.fft_cols > 0 && !fuse_auto && !fuse_shape && !persist_auto &&
       !colw_shape)
     return RF_OK;
