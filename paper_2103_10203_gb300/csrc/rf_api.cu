@@ -254,9 +254,6 @@ int get_while_graph(rf_ctx* c) {
 // forgets the current pattern; its device buffers stay for the next one (palloc)
 void free_pattern(rf_ctx* c) {
   free_graphs(c);
-  for (TcAxis* ax : {&c->tc_yf, &c->tc_yi, &c->tc_zf, &c->tc_zi}) {
-    ax->M = ax->K = ax->nMT = ax->nKC = 0;
-  }
   c->fft_colmode = kColSeparate;
   c->team_on = false;
   c->have_pattern = false;
@@ -283,7 +280,6 @@ void release_pattern_buffers(rf_ctx* c) {
   dfree(c->d_warm);
   dfree(c->d_phiI);
   dfree(c->d_phiF);
-  for (TcAxis* ax : {&c->tc_yf, &c->tc_yi, &c->tc_zf, &c->tc_zi}) dfree(ax->A);
   dfree(c->d_Tout);
   dfree(c->d_tc_err);
   dfree(c->d_jptr);
@@ -945,7 +941,8 @@ int rf_set_pattern(rf_ctx* c, const int32_t* freqs, int64_t K) {
     if (pe && c->opt.fft_fuse == 3) err = pe;
     else if (pe) set_error("");
   }
-  if (!err && c->opt.transform == RF_TRANSFORM_FFT) err = fft3_setup(c, kym.data());
+  if (!err) err = fft3_setup(c, kym.data());
+  if (!err && c->opt.transform == RF_TRANSFORM_DFT && fft3_yz_ok(c)) c->fft_colmode = kColZ;
   c->dft_U = 0;
   if (!err && c->opt.transform == RF_TRANSFORM_DFT) err = dft_setup(c);
   if (!err && c->opt.precision != RF_PREC_FP32) err = tc_setup(c);

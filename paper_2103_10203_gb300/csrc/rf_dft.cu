@@ -292,6 +292,8 @@ struct AxisDftArgs {
   const float2* in;
   float2* out;
   long long in_bstride, out_bstride;
+  int splits;           // dense input: partial sums to add up (row passes over slices of x), ...
+  long long split_stride;
   int L, N, S;          // length, columns, sparse rows
   const int* vals;      // [S] frequency (mod L) of each sparse row
   const float2* table;  // exp(+2 pi i t / L)
@@ -351,6 +353,23 @@ __global__ __launch_bounds__(128) void k_axis_dft(const __grid_constant__ AxisDf
           if (FWD && y > 0 && 2 * y != L) q[u] = __ldcg(in + (long long)(L - y) * a.N + n);
         }
       }
+      if (FWD && n < a.N)
+        for (int s = 1; s < a.splits; ++s) {
+          const float2* is = in + s * a.split_stride + n;
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            const int r = r0 + 4 * u, y = k0 + r;
+            if (r >= kn) break;
+            const float2 e = __ldcg(is + (long long)y * a.N);
+            p[u].x += e.x;
+            p[u].y += e.y;
+            if (y > 0 && 2 * y != L) {
+              const float2 f = __ldcg(is + (long long)(L - y) * a.N);
+              q[u].x += f.x;
+              q[u].y += f.y;
+            }
+          }
+        }
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         const int r = r0 + 4 * u, y = k0 + r;
@@ -501,10 +520,12 @@ int launch_row_dft(rf_ctx* c, const int* done, bool final_pass, int commit, int*
 }
 
 // sign +1: S sparse rows -> L dense ones, -1: the reverse; N columns, `batch` arrays
-int launch_axis_dft(rf_ctx* c, const float2* in, long long in_bs, float2* out, long long out_bs,
-                    int L, int N, int S, int batch, const int* vals, const float2* table, int sign,
-                    const int* done) {
+int launch_axis_dft(rf_ctx* c, const float2* in, int splits, long long split_stride,
+                    long long in_bs, float2* out, long long out_bs, int L, int N, int S, int batch,
+                    const int* vals, const float2* table, int sign, const int* done) {
   AxisDftArgs a{};
+  a.splits = splits;
+  a.split_stride = split_stride;
   a.in = in;
   a.out = out;
   a.in_bstride = in_bs;

@@ -52,19 +52,21 @@ int done3(rf_ctx* c, cudaError_t e, const char* what) {
 
 }  // namespace
 
+bool fft3_yz_ok(const rf_ctx* c) {
+  Shape3 s;
+  return c->dim == 3 && c->nc == 6 && shape_of(c->ny, &s) && shape_of(c->nz, &s) && c->d_zrange;
+}
+
 bool fft3_ok(const rf_ctx* c) {
   Shape3 s;
-  return c->dim == 3 && c->nc == 6 && c->opt.transform == RF_TRANSFORM_FFT &&
-         shape_of(c->nx, &s) && shape_of(c->ny, &s) && shape_of(c->nz, &s) && c->Kx <= 32767 &&
-         c->d_zrange;
+  return fft3_yz_ok(c) && c->opt.transform == RF_TRANSFORM_FFT && shape_of(c->nx, &s);
 }
 
 // Pattern tables: first half-pattern entry and count of every (ky, kx) (the half pattern is sorted
 // by kx, ky, kz), and the rectangle row of each position along y.
 int fft3_setup(rf_ctx* c, const int* kym) {
   Shape3 s;
-  if (c->dim != 3 || !shape_of(c->nx, &s) || !shape_of(c->ny, &s) || !shape_of(c->nz, &s))
-    return RF_OK;
+  if (c->dim != 3 || !shape_of(c->ny, &s) || !shape_of(c->nz, &s)) return RF_OK;
   std::vector<int2> range((size_t)c->Ky * c->Kx, make_int2(0, 0));
   for (long long h = 0; h < c->Kh; ++h) {
     int2& r = range[(size_t)c->h_hidx[h].iy * c->Kx + c->h_hidx[h].j];
@@ -135,14 +137,18 @@ int launch_fft3_row(rf_ctx* c, const int* done, bool final_pass, int commit, int
   return done3(c, launch_pdl(k, dim3(grid), dim3(threads), smem, c->stream, a), "3D row pass");
 }
 
-// sign +1: T2 -> T1 (sparse rows in), -1: T1p -> T2f (sparse rows out)
-int launch_fft3_y(rf_ctx* c, int sign, const int* done) {
+// sign +1: T2 -> T1 (sparse rows in), -1: T1p (or `splits` partial sums at `in`) -> T2f (sparse rows
+// out)
+int launch_fft3_y(rf_ctx* c, int sign, const int* done, const float2* in, int splits,
+                  long long split_stride) {
   Shape3 s;
   shape_of(c->ny, &s);
   const int NCK = c->nc * c->Kx;
   const long long sparse = (long long)c->Ky * NCK, dense = (long long)c->ny * NCK;
   ColArgs3 a{};
-  a.in = sign > 0 ? c->d_T2 : c->d_T1p;
+  a.in = sign > 0 ? c->d_T2 : in ? in : c->d_T1p;
+  a.splits = splits;
+  a.split_stride = split_stride;
   a.out = sign > 0 ? c->d_T1 : c->d_T2f;
   a.in_bstride = sign > 0 ? sparse : dense;
   a.out_bstride = sign > 0 ? dense : sparse;

@@ -224,6 +224,8 @@ struct ColArgs3 {
   const float2* in;
   float2* out;
   long long in_bstride, out_bstride;
+  int splits;            // S = -1: partial sums to add up (row passes over slices of x), ...
+  long long split_stride;
   const short* map;      // [L] row of each position on the sparse side, -1: not in the pattern
   const float2* table;
   int ncols, cgroups, total;   // column groups per batch entry, groups in all
@@ -269,6 +271,16 @@ __global__ __launch_bounds__(512) void k_cols3(const __grid_constant__ ColArgs3 
       v[q] = make_float2(0.f, 0.f);
       if (on && r >= 0) v[q] = __ldcg(in + (long long)r * a.ncols);
     }
+    if (S < 0 && on)
+      for (int s = 1; s < a.splits; ++s) {
+        const float2* is = in + s * a.split_stride;
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+          const float2 u = __ldcg(is + (long long)(t + G * q) * a.ncols);
+          v[q].x += u.x;
+          v[q].y += u.y;
+        }
+      }
     P::template first<S>(v, b0, t);
     __syncthreads();
     if (M > 1) {

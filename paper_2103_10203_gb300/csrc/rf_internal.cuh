@@ -116,12 +116,6 @@ struct GammaArgs {
 
 }  // namespace rfk
 
-// split-precision transform along y or z: precomputed A tiles (see rf_tc.cu)
-struct TcAxis {
-  unsigned char* A = nullptr;
-  int M = 0, K = 0, nMT = 0, nKC = 0;
-};
-
 struct rf_ctx {
   int dev = 0;
   int dim = 2, nx = 1, ny = 1, nz = 1, nc = 3, ns = 0;
@@ -195,7 +189,8 @@ struct rf_ctx {
   // line coefficients in kx slabs (kColWarp, 1024 x 1024, warp-FFT row kernel); 5 the
   // persistent solve on the same passes (kColPersistW). Modes 1, 2 and 4 start a solve with one
   // inverse y of the start coefficients (3 and 5 inside their launch). 3D: 0, or 6 the updates on
-  // team FFTs (kColZ), which start with the inverse along z.
+  // team FFTs (kColZ), which start with the inverse along z
+  // (in the DFT transform where the sides along y and z allow, with its own row pass).
   int fft_colmode = 0;
   int fft_M = 1, fft_M_threads = 256;   // kx columns and threads per fused block
   // persistent 2D solve (column mode kColPersistent): grid, block size, dynamic shared memory,
@@ -236,7 +231,6 @@ struct rf_ctx {
   // split-precision (tensor-core) transforms along x
   unsigned char* d_phiI = nullptr;
   unsigned char* d_phiF = nullptr;
-  TcAxis tc_yf, tc_yi, tc_zf, tc_zi;   // forward / inverse along y and z
   // capacities of the pattern-scoped device buffers (kept across patterns, see palloc)
   std::unordered_map<const void*, size_t> pcap;
   int* d_hk = nullptr;                 // pattern upload staging
@@ -434,9 +428,6 @@ int launch_fft_row(rf_ctx* c, const int* done, bool final_pass, int commit);
 int fft_inverse_stages(rf_ctx* c, const int* done);
 int fft_forward_stages(rf_ctx* c, const int* done);
 int launch_fft_colphase(rf_ctx* c, const int* done);
-int launch_tc_axis(rf_ctx* c, const TcAxis& ax, const float2* in, int in_splits,
-                   long long in_split_stride, long long in_bstride, float2* out,
-                   long long out_bstride, int N, int batch, const int* done);
 int launch_fft_green_inv(rf_ctx* c, const int* done);
 int launch_gather_jentries(rf_ctx* c);
 constexpr int kColSeparate = 0, kColFused = 1, kColGreenInv = 2, kColPersistent = 3,
@@ -451,15 +442,17 @@ int persist_setup(rf_ctx* c);
 int dft_setup(rf_ctx* c);
 void init_attributes_dft();
 int launch_row_dft(rf_ctx* c, const int* done, bool final_pass, int commit, int* blocks);
-int launch_axis_dft(rf_ctx* c, const float2* in, long long in_bs, float2* out, long long out_bs,
-                    int L, int N, int S, int batch, const int* vals, const float2* table, int sign,
-                    const int* done);
+int launch_axis_dft(rf_ctx* c, const float2* in, int splits, long long split_stride,
+                    long long in_bs, float2* out, long long out_bs, int L, int N, int S, int batch,
+                    const int* vals, const float2* table, int sign, const int* done);
 // rf_fft3.cu: 3D updates on team FFTs (column mode kColZ)
-bool fft3_ok(const rf_ctx* c);
+bool fft3_yz_ok(const rf_ctx* c);   // the sides along y and z (any row pass)
+bool fft3_ok(const rf_ctx* c);      // all three (FFT transform)
 int fft3_setup(rf_ctx* c, const int* kym);
 void init_attributes_fft3();
 int launch_fft3_row(rf_ctx* c, const int* done, bool final_pass, int commit, int* blocks);
-int launch_fft3_y(rf_ctx* c, int sign, const int* done);
+int launch_fft3_y(rf_ctx* c, int sign, const int* done, const float2* in = nullptr, int splits = 1,
+                  long long split_stride = 0);
 int launch_fft3_z(rf_ctx* c, bool full, const int* done);
 // rf_team.cu
 bool team_ok(const rf_ctx* c);

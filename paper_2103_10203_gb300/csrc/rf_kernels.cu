@@ -704,32 +704,31 @@ static int row_dispatch(rf_ctx* c, const RowArgs& a, bool final_pass) {
 
 int launch_gamma_finalize(rf_ctx* c, const int* done);
 
-// transforms along y and z: tensor cores (split operands) in the split-precision modes, the
-// SIMT DFT otherwise (rf_dft.cu). sign +1: S sparse rows -> L dense ones, -1: the reverse.
-static int axis(rf_ctx* c, const TcAxis& ax, const float2* in, int in_splits, long long iss,
-                long long ibs, float2* out, long long obs, int L, int N, int S, int batch,
-                const int* vals, const float2* tab, int sign, const int* done) {
-  if (c->opt.precision != RF_PREC_FP32)
-    return launch_tc_axis(c, ax, in, in_splits, iss, ibs, out, obs, N, batch, done);
-  return launch_axis_dft(c, in, ibs, out, obs, L, N, S, batch, vals, tab, sign, done);
-}
-
 static int inverse_stages(rf_ctx* c, const int* done) {
   const int NCK = c->nc * c->Kx;
   if (c->dim == 3) {
     // along z: T2[z][ky][c][kx] = sum_kz exp(+..kz z) ER[kz][ky][c][kx]
     trace_stage(c, 0);
-    if (int e = axis(c, c->tc_zi, c->d_ER, 1, 0, 0, c->d_T2, 0, c->nz, c->Ky * NCK, c->Kz, 1,
-                     c->d_kzm, c->d_twz, +1, done))
+    if (int e = launch_axis_dft(c, c->d_ER, 1, 0, 0, c->d_T2, 0, c->nz, c->Ky * NCK, c->Kz, 1,
+                                c->d_kzm, c->d_twz, +1, done))
       return e;
     // along y, batched over z
     trace_stage(c, 1);
-    return axis(c, c->tc_yi, c->d_T2, 1, 0, (long long)c->Ky * NCK, c->d_T1,
-                (long long)c->ny * NCK, c->ny, NCK, c->Ky, c->nz, c->d_kym, c->d_twy, +1, done);
+    return launch_axis_dft(c, c->d_T2, 1, 0, (long long)c->Ky * NCK, c->d_T1,
+                           (long long)c->ny * NCK, c->ny, NCK, c->Ky, c->nz, c->d_kym, c->d_twy, +1,
+                           done);
   }
   trace_stage(c, 1);
-  return axis(c, c->tc_yi, c->d_ER, 1, 0, 0, c->d_T1, 0, c->ny, NCK, c->Ky, 1, c->d_kym, c->d_twy,
-              +1, done);
+  return launch_axis_dft(c, c->d_ER, 1, 0, 0, c->d_T1, 0, c->ny, NCK, c->Ky, 1, c->d_kym, c->d_twy,
+                         +1, done);
+}
+
+// the row pass of the DFT transform, T1 -> T1p (split precision: partial sums per 128-wide slice
+// of x in d_Tout)
+static int dft_row(rf_ctx* c, const int* done) {
+  if (c->opt.precision != RF_PREC_FP32) return launch_tc_row(c, done);
+  if (c->dft_U > 0) return launch_row_dft(c, done, false, 0, nullptr);
+  return row_dispatch(c, row_args(c, done), false);
 }
 
 int launch_iteration(rf_ctx* c) {
@@ -749,13 +748,16 @@ int launch_iteration(rf_ctx* c) {
     if (int e = launch_fft_row(c, done, false, 0)) return e;
     return launch_fft_colphase_warp(c, done);
   }
-  if (fftm && c->fft_colmode == kColZ) {
+  if (c->fft_colmode == kColZ) {
     trace_stage(c, 1);
     if (int e = launch_fft3_y(c, +1, done)) return e;
     trace_stage(c, 2);
-    if (int e = launch_fft3_row(c, done, false, 0, nullptr)) return e;
+    if (int e = fftm ? launch_fft3_row(c, done, false, 0, nullptr) : dft_row(c, done)) return e;
     trace_stage(c, 3);
-    if (int e = launch_fft3_y(c, -1, done)) return e;
+    const bool part = c->opt.precision != RF_PREC_FP32;
+    if (int e = launch_fft3_y(c, -1, done, part ? reinterpret_cast<const float2*>(c->d_Tout) : nullptr,
+                              part ? c->tc_nXS : 1, (long long)c->rows * c->nc * c->Kx))
+      return e;
     trace_stage(c, 6);
     const int e = launch_fft3_z(c, true, done);
     trace_end(c);
@@ -776,34 +778,27 @@ int launch_iteration(rf_ctx* c) {
     return launch_gamma_finalize(c, done);
   }
   if (int e = inverse_stages(c, done)) return e;
-  const bool tcm = c->opt.precision != RF_PREC_FP32;
   trace_stage(c, 2);
-  if (tcm) {
-    if (int e = launch_tc_row(c, done)) return e;
-  } else if (c->dft_U > 0) {
-    if (int e = launch_row_dft(c, done, false, 0, nullptr)) return e;
-  } else {
-    RowArgs ra = row_args(c, done);
-    if (int e = row_dispatch(c, ra, false)) return e;
-  }
+  if (int e = dft_row(c, done)) return e;
   const int NCK = c->nc * c->Kx;
+  const bool tcm = c->opt.precision != RF_PREC_FP32;
   // the tensor-core row kernel leaves one partial sum per 128-wide x slice
   const float2* fin = tcm ? reinterpret_cast<const float2*>(c->d_Tout) : c->d_T1p;
   const int fsplits = tcm ? c->tc_nXS : 1;
   const long long fstride = (long long)c->rows * NCK;
   trace_stage(c, 3);
   if (c->dim == 3) {
-    if (int e = axis(c, c->tc_yf, fin, fsplits, fstride, (long long)c->ny * NCK, c->d_T2f,
-                     (long long)c->Ky * NCK, c->ny, NCK, c->Ky, c->nz, c->d_kym, c->d_twy, -1,
-                     done))
+    if (int e = launch_axis_dft(c, fin, fsplits, fstride, (long long)c->ny * NCK, c->d_T2f,
+                                (long long)c->Ky * NCK, c->ny, NCK, c->Ky, c->nz, c->d_kym,
+                                c->d_twy, -1, done))
       return e;
     trace_stage(c, 4);
-    if (int e = axis(c, c->tc_zf, c->d_T2f, 1, 0, 0, c->d_OUT, 0, c->nz, c->Ky * NCK, c->Kz, 1,
-                     c->d_kzm, c->d_twz, -1, done))
+    if (int e = launch_axis_dft(c, c->d_T2f, 1, 0, 0, c->d_OUT, 0, c->nz, c->Ky * NCK, c->Kz, 1,
+                                c->d_kzm, c->d_twz, -1, done))
       return e;
   } else {
-    if (int e = axis(c, c->tc_yf, fin, fsplits, fstride, 0, c->d_OUT, 0, c->ny, NCK, c->Ky, 1,
-                     c->d_kym, c->d_twy, -1, done))
+    if (int e = launch_axis_dft(c, fin, fsplits, fstride, 0, c->d_OUT, 0, c->ny, NCK, c->Ky, 1,
+                                c->d_kym, c->d_twy, -1, done))
       return e;
   }
   return launch_gamma_finalize(c, done);
@@ -860,11 +855,13 @@ int launch_final(rf_ctx* c, int commit) {
     trace_end(c);
     return e;
   }
-  if (c->opt.transform == RF_TRANSFORM_FFT && c->fft_colmode == kColZ) {
+  if (c->fft_colmode == kColZ && (c->opt.transform == RF_TRANSFORM_FFT || c->dft_U > 0)) {
     // the last z phase left the final coefficients transformed along z
     int blocks = 0;
     int ie = launch_fft3_y(c, +1, nullptr);
-    if (!ie) ie = launch_fft3_row(c, nullptr, true, commit, &blocks);
+    if (!ie)
+      ie = c->opt.transform == RF_TRANSFORM_FFT ? launch_fft3_row(c, nullptr, true, commit, &blocks)
+                                                : launch_row_dft(c, nullptr, true, commit, &blocks);
     c->tracing = tr;
     if (ie) return ie;
     k_reduce_sbar<<<1, kReduceThreads, 0, c->stream>>>(c->d_sbar_part, c->d_viol_part, blocks,
@@ -884,7 +881,7 @@ int launch_final(rf_ctx* c, int commit) {
     trace_end(c);
     return e;
   }
-  int ie = inverse_stages(c, nullptr);
+  int ie = c->fft_colmode == kColZ ? launch_fft3_y(c, +1, nullptr) : inverse_stages(c, nullptr);
   c->tracing = tr;
   if (ie) return ie;
   if (c->dft_U > 0) {
