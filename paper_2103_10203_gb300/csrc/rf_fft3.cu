@@ -12,16 +12,14 @@ namespace {
 constexpr int kSmem3 = 200 * 1024;
 
 struct Shape3 {
-  int lanes, tw, teams, cols, kx;   // threads per sequence, twiddles, and what a block takes
+  int lanes, tw, cols, kx;   // threads per sequence, twiddles, and what a block takes
 };
 
 bool shape_of(int L, Shape3* s) {
   switch (L) {
 #define X(L_, R, M)                                                                              \
   case L_:                                                                                       \
-    *s = Shape3{R * M, Plan<R, M>::kTw, R * M <= 12 ? 8 : R * M == 16 || R * M == 24 ? 4         \
-                                        : R * M <= 48 ? 2 : 1,                                   \
-                cols_per_block<R, M>(), kx_per_block<R, M>()};                                   \
+    *s = Shape3{R * M, Plan<R, M>::kTw, cols_per_block<R, M>(), kx_per_block<R, M>()};           \
     return true;
     RF_TEAM_SIDES(X)
 #undef X
@@ -109,8 +107,8 @@ int launch_fft3_row(rf_ctx* c, const int* done, bool final_pass, int commit, int
   a.table = c->d_twx;
   a.Kx = c->Kx;
   a.rows = c->rows;
-  a.teams = s.teams;
-  a.groups = (c->rows + s.teams - 1) / s.teams;
+  a.teams = 256 / s.lanes;
+  a.groups = (c->rows + a.teams - 1) / a.teams;
   a.N = c->N;
   a.invN = (float)(1.0 / (double)c->N);
   a.law = c->law;
@@ -125,8 +123,8 @@ int launch_fft3_row(rf_ctx* c, const int* done, bool final_pass, int commit, int
   }
   RowKernel k = c->has_plastic ? row_kernel_plastic(c->nx, final_pass)
                                : row_kernel_elastic(c->nx, final_pass);
-  const int threads = s.teams * 3 * s.lanes;
-  const size_t smem = sizeof(float2) * (((s.tw + 1) & ~1) + (size_t)s.teams * 6 * even_span(c->nx)) +
+  const int threads = a.teams * s.lanes;
+  const size_t smem = sizeof(float2) * (((s.tw + 1) & ~1) + (size_t)a.teams * 3 * even_span(c->nx)) +
                       sizeof(int) * c->Kx + sizeof(short) * (c->nx / 2 + 1) + 16;
   const int grid = fill(c, (const void*)k, threads, smem, a.groups);
   if (blocks) *blocks = grid;

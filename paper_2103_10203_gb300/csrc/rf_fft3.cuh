@@ -1,6 +1,6 @@
 // 3D updates of the FFT transform mode on team FFTs (FP32): four kernels per update,
 //   inverse y     T2 -> T1, only the pattern's ky rows are read
-//   row pass      inverse along x, law, forward along x (T1 -> T1p), a team of 3 G threads per grid
+//   row pass      inverse along x, law, forward along x (T1 -> T1p), a team of G threads per grid
 //                 row: its six lines are three packed complex sequences
 //   forward y     T1p -> T2f, only the pattern's ky rows are written
 //   z phase       per (ky, kx): forward along z, Green operator and decision, inverse along z
@@ -10,8 +10,8 @@
 // by six launches; here the sizes are compile-time constants, every transform's first pass
 // reads global memory straight into registers and its last pass writes it straight back (sparse
 // sides through a position map), and the frequencies of one (ky, kx) never leave the block between
-// the two transforms along z. 128^3, K = 2 %: row 81 -> 44 us, y 30 + 30 -> 17 + 17, z and Green
-// 20 + 15 + 20 -> 31 us (traced), 175 -> 94 us per update.
+// the two transforms along z. 128^3, K = 2 %: row 81 -> 36 us, y 30 + 30 -> 17 + 17, z and Green
+// 20 + 15 + 20 -> 31 us (traced), 175 -> 86 us per update.
 #pragma once
 
 #include <algorithm>
@@ -48,21 +48,24 @@ struct RowArgs3 {
   const int* done;
 };
 
-// One row pass over all rows: a block of `teams` teams takes groups of that many rows in turn.
+// One row pass over all rows: a block of `teams` teams of G threads takes groups of that many rows
+// in turn. A thread carries its points of all three sequences, so the law runs on registers and
+// only the passes of the transforms cross shared memory, with warp barriers up to 256 points (3 G
+// threads per row, the strains and polarizations staged through shared memory: 44 us at 128^3; so:
+// 36 us).
 template <int R, int M, bool PLASTIC, bool FINAL>
-__global__ __launch_bounds__(288) void k_row3(const __grid_constant__ RowArgs3 a) {
+__global__ __launch_bounds__(256, 2) void k_row3(const __grid_constant__ RowArgs3 a) {
   using P = Plan<R, M>;
-  constexpr int L = P::L, G = P::G, NT = 3 * G, NS = 7;
+  constexpr int L = P::L, G = P::G;
   constexpr int span = (L + L / 16 + 2) & ~1;
-  constexpr int NV = (L + NT - 1) / NT;   // voxels per thread in the law
   __shared__ DevPhase phs[kMaxPhases];
   __shared__ double red[32];
   float2* tw = reinterpret_cast<float2*>(z_smem);
   float2* bufs = tw + ((P::kTw + 1) & ~1);
-  int* kxs = reinterpret_cast<int*>(bufs + a.teams * 6 * span);
+  int* kxs = reinterpret_cast<int*>(bufs + a.teams * 3 * span);
   short* jmap = reinterpret_cast<short*>(kxs + a.Kx);
   const int tid = threadIdx.x;
-  const int team = tid / NT, w = tid - team * NT, seq = w / G, t = w - seq * G;
+  const int team = tid / G, t = tid - team * G;
   const int Kx = a.Kx;
   P::twiddles(a.table, tw);
   for (int i = tid; i <= L / 2; i += blockDim.x) jmap[i] = -1;
@@ -76,139 +79,140 @@ __global__ __launch_bounds__(288) void k_row3(const __grid_constant__ RowArgs3 a
   grid_dep_wait();
   if (!FINAL && a.done && __ldcg(a.done)) return;   // the same flag value for every thread
   __syncthreads();
-  float2* base = bufs + team * 6 * span;   // sequence s: base + 2 s span, and a second buffer
-  float2* b0 = base + seq * 2 * span;
-  float2* b1 = b0 + span;
-  float2* const X = M == 1 ? b1 : b0;      // the sequence in space
-  float2* const Y = M == 1 ? b0 : b1;
+  float2* b = bufs + team * 3 * span;
   const float lam0 = a.law.lam0, mu0 = a.law.mu0;
   double sb[6] = {0, 0, 0, 0, 0, 0}, vmax = 0.0;
   for (int g = blockIdx.x; g < a.groups; g += gridDim.x) {
     const int row = g * a.teams + team;
     const bool on = row < a.rows;
-    float2 v[R];
-    uint8_t pid[NV];
+    float2 v[3][R];
+    uint8_t pid[R];
     if (on) {
-      const float2* s0 = a.T + ((long long)row * 6 + 2 * seq) * Kx;
-      float2 ca[R], cb[R];
+      const float2* s0 = a.T + (long long)row * 6 * Kx;
 #pragma unroll
       for (int q = 0; q < R; ++q) {
         const int p = t + G * q;
         const int j = jmap[p <= L / 2 ? p : L - p];
-        ca[q] = cb[q] = make_float2(0.f, 0.f);
-        if (j >= 0) {
-          ca[q] = __ldcg(s0 + j);
-          cb[q] = __ldcg(s0 + Kx + j);
+        float2 c[6];
+#pragma unroll
+        for (int i = 0; i < 6; ++i) {
+          c[i] = make_float2(0.f, 0.f);
+          if (j >= 0) c[i] = __ldcg(s0 + i * Kx + j);
+        }
+#pragma unroll
+        for (int s = 0; s < 3; ++s) {
+          float2 x = c[2 * s], y = c[2 * s + 1];
+          if (p == 0 || 2 * p == L) x.y = y.y = 0.f;   // self-conjugate positions of real lines
+          v[s][q] = 2 * p <= L ? make_float2(x.x - y.y, x.y + y.x) : make_float2(x.x + y.y, y.x - x.y);
         }
       }
+      if (!FINAL) {
 #pragma unroll
-      for (int i = 0; i < NV; ++i) {
-        const int x = w + NT * i;
-        pid[i] = x < L ? a.phase[(long long)row * L + x] : 0;
+        for (int q = 0; q < R; ++q) pid[q] = a.phase[(long long)row * L + t + G * q];
       }
-#pragma unroll
-      for (int q = 0; q < R; ++q) {
-        const int p = t + G * q;
-        float2 x = ca[q], y = cb[q];
-        if (p == 0 || 2 * p == L) x.y = y.y = 0.f;   // self-conjugate positions of real lines
-        v[q] = 2 * p <= L ? make_float2(x.x - y.y, x.y + y.x) : make_float2(x.x + y.y, y.x - x.y);
-      }
-      P::template first<+1>(v, b0, t);
+      P::template first3<+1>(v, b, span, t);
     }
-    __syncthreads();
+    P::sync(team);
     if (M > 1) {
-      if (on) P::template middle<+1>(b0, b1, tw, t);
-      __syncthreads();
+      if (on) P::template middle3<+1>(b, span, tw, t);
+      P::sync(team);
     }
-    if (on) {
-      P::template last<+1>(M == 1 ? b0 : b1, v, tw, t);
+    if (on) P::template last3<+1>(b, span, v, tw, t);
+    P::sync(team);
+    if (FINAL) {
+      // one voxel per step (this code runs once per solve, so its instructions come from memory)
+      if (on) {
 #pragma unroll
-      for (int q = 0; q < R; ++q) X[sw(t + G * q)] = v[q];
-    }
-    __syncthreads();
-    if (on) {
-      float2* x0 = base + (M == 1 ? span : 0);
+        for (int q = 0; q < R; ++q)
 #pragma unroll
-      for (int i = 0; i < NV; ++i) {
-        const int x = w + NT * i;
-        if (x >= L) break;
-        float2* z = x0 + sw(x);
-        const float2 z0 = z[0], z1 = z[2 * span], z2 = z[4 * span];
+          for (int s = 0; s < 3; ++s) b[s * span + sw(t + G * q)] = v[s][q];
+      }
+      P::sync(team);
+#pragma unroll 1
+      for (int x = t; on && x < L; x += G) {
+        const float2* z = b + sw(x);
+        const float2 z0 = z[0], z1 = z[span], z2 = z[2 * span];
         const float e6[6] = {z0.x * a.invN, z0.y * a.invN, z1.x * a.invN,
                              z1.y * a.invN, z2.x * a.invN, z2.y * a.invN};
         const long long gv = (long long)row * L + x;
         float ep[6] = {0, 0, 0, 0, 0, 0};
         float alpha = 0.f;
         if (PLASTIC) load_state<6>(a.state, a.N, gv, ep, alpha);
-        const DevPhase& ph = phs[pid[i]];
+        const DevPhase& ph = phs[a.phase[gv]];
         LawOut o;
         stress6<PLASTIC>(e6, ph, ep, alpha, o);
-        if (!FINAL) {
-          const float lt = lam0 * (e6[0] + e6[1] + e6[2]);
-          z[0] = make_float2(o.s[0] - (lt + 2.f * mu0 * e6[0]), o.s[1] - (lt + 2.f * mu0 * e6[1]));
-          z[2 * span] = make_float2(o.s[2] - (lt + 2.f * mu0 * e6[2]), o.s[3] - 2.f * mu0 * e6[3]);
-          z[4 * span] = make_float2(o.s[4] - 2.f * mu0 * e6[4], o.s[5] - 2.f * mu0 * e6[5]);
-        } else {
 #pragma unroll
-          for (int q = 0; q < 6; ++q) {
-            sb[q] += (double)o.s[q];
-            a.eps_out[q * a.N + gv] = e6[q];
-            a.sig_out[q * a.N + gv] = o.s[q];
+        for (int q = 0; q < 6; ++q) {
+          sb[q] += (double)o.s[q];
+          a.eps_out[q * a.N + gv] = e6[q];
+          a.sig_out[q * a.N + gv] = o.s[q];
+        }
+        if (PLASTIC) {
+          if (a.commit) store_state<6>(a.state, a.N, gv, o.ep, o.alpha);
+          a.alpha_out[gv] = o.alpha;
+          if (o.yielded) {
+            // FP64 consistency check of the FP32 return map: sigma_eq(sigma) = sy + H alpha
+            const double s0 = o.s[0], s1 = o.s[1], s2 = o.s[2];
+            const double pmd = (s0 + s1 + s2) / 3.0;
+            const double d0 = s0 - pmd, d1 = s1 - pmd, d2 = s2 - pmd;
+            const double qq = d0 * d0 + d1 * d1 + d2 * d2 +
+                              2.0 * ((double)o.s[3] * o.s[3] + (double)o.s[4] * o.s[4] +
+                                     (double)o.s[5] * o.s[5]);
+            const double yl = (double)ph.sy + (double)ph.H * (double)o.alpha;
+            vmax = fmax(vmax, fabs(sqrt(1.5 * qq) - yl) / (double)ph.sy);
           }
-          if (PLASTIC) {
-            if (a.commit) store_state<6>(a.state, a.N, gv, o.ep, o.alpha);
-            a.alpha_out[gv] = o.alpha;
-            if (o.yielded) {
-              // FP64 consistency check of the FP32 return map: sigma_eq(sigma) = sy + H alpha
-              const double s0 = o.s[0], s1 = o.s[1], s2 = o.s[2];
-              const double pmd = (s0 + s1 + s2) / 3.0;
-              const double d0 = s0 - pmd, d1 = s1 - pmd, d2 = s2 - pmd;
-              const double qq = d0 * d0 + d1 * d1 + d2 * d2 +
-                                2.0 * ((double)o.s[3] * o.s[3] + (double)o.s[4] * o.s[4] +
-                                       (double)o.s[5] * o.s[5]);
-              const double yl = (double)ph.sy + (double)ph.H * (double)o.alpha;
-              vmax = fmax(vmax, fabs(sqrt(1.5 * qq) - yl) / (double)ph.sy);
-            }
-          } else {
-            a.alpha_out[gv] = 0.f;
-          }
+        } else {
+          a.alpha_out[gv] = 0.f;
         }
       }
+      P::sync(team);
+      continue;
     }
-    __syncthreads();
-    if (FINAL) continue;
     if (on) {
 #pragma unroll
-      for (int q = 0; q < R; ++q) v[q] = X[sw(t + G * q)];
-      P::template first<-1>(v, Y, t);
+      for (int q = 0; q < R; ++q) {
+        const float e6[6] = {v[0][q].x * a.invN, v[0][q].y * a.invN, v[1][q].x * a.invN,
+                             v[1][q].y * a.invN, v[2][q].x * a.invN, v[2][q].y * a.invN};
+        float ep[6] = {0, 0, 0, 0, 0, 0};
+        float alpha = 0.f;
+        if (PLASTIC) load_state<6>(a.state, a.N, (long long)row * L + t + G * q, ep, alpha);
+        LawOut o;
+        stress6<PLASTIC>(e6, phs[pid[q]], ep, alpha, o);
+        const float lt = lam0 * (e6[0] + e6[1] + e6[2]);
+        v[0][q] = make_float2(o.s[0] - (lt + 2.f * mu0 * e6[0]), o.s[1] - (lt + 2.f * mu0 * e6[1]));
+        v[1][q] = make_float2(o.s[2] - (lt + 2.f * mu0 * e6[2]), o.s[3] - 2.f * mu0 * e6[3]);
+        v[2][q] = make_float2(o.s[4] - 2.f * mu0 * e6[4], o.s[5] - 2.f * mu0 * e6[5]);
+      }
+      P::template first3<-1>(v, b, span, t);
     }
-    __syncthreads();
+    P::sync(team);
     if (M > 1) {
-      if (on) P::template middle<-1>(Y, X, tw, t);
-      __syncthreads();
+      if (on) P::template middle3<-1>(b, span, tw, t);
+      P::sync(team);
     }
+    if (on) P::template last3<-1>(b, span, v, tw, t);
+    P::sync(team);
     if (on) {
-      P::template last<-1>(M == 1 ? Y : X, v, tw, t);
-      float2* z = M == 1 ? X : Y;
 #pragma unroll
-      for (int q = 0; q < R; ++q) z[sw(t + G * q)] = v[q];
+      for (int q = 0; q < R; ++q)
+#pragma unroll
+        for (int s = 0; s < 3; ++s) b[s * span + sw(t + G * q)] = v[s][q];
     }
-    __syncthreads();
+    P::sync(team);
     if (on) {
-      const float2* z = base + span;   // both cases leave the spectra in the second buffers
       float2* o = a.Tout + (long long)row * 6 * Kx;
-      for (int j = w; j < Kx; j += NT) {
+      for (int j = t; j < Kx; j += G) {
         const int k = kxs[j];
         const int ik = sw(k), im = sw(k == 0 ? 0 : L - k);
 #pragma unroll
         for (int s = 0; s < 3; ++s) {
-          const float2 zk = z[s * 2 * span + ik], zm = z[s * 2 * span + im];
+          const float2 zk = b[s * span + ik], zm = b[s * span + im];
           o[(2 * s) * Kx + j] = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));
           o[(2 * s + 1) * Kx + j] = make_float2(0.5f * (zk.y + zm.y), -0.5f * (zk.x - zm.x));
         }
       }
     }
-    __syncthreads();
+    P::sync(team);
   }
   if (FINAL) {
     for (int i = 0; i < 6; ++i) {

@@ -185,6 +185,72 @@ struct Plan {
     }
     Dft<R, S>::run(v);
   }
+
+  // ---- three sequences per thread, `ld` entries apart, each in one buffer: the middle pass leaves
+  // output q of task j in the places that the task read (place(q), which keeps the last pass's
+  // reads on different banks where M allows it); a team sync between passes and before the next
+  // first pass. Addresses, twiddles and barriers are shared by the three sequences, and the law
+  // runs on registers between the transforms.
+  static __host__ __device__ constexpr int place(int q) {
+    return M % 4 == 0 ? (q & ~3) | ((q & 1) << 1) | ((q >> 1) & 1) : q;
+  }
+  template <int S>
+  static __device__ __forceinline__ void first3(float2 (&v)[3][R], float2* b, int ld, int t) {
+#pragma unroll
+    for (int s = 0; s < 3; ++s) first<S>(v[s], b + s * ld, t);
+  }
+  template <int S>
+  static __device__ __forceinline__ void middle3(float2* b, int ld, const float2* tw, int t) {
+    constexpr int T = R * R, pq = T + T / 16;
+#pragma unroll 1
+    for (int i = t; i < 3 * T; i += G) {
+      const int s = i / T, j = i - s * T, k = j % R;
+      float2* d = b + s * ld + sw(j);
+      float2 v[M];
+#pragma unroll
+      for (int q = 0; q < M; ++q) v[q] = d[q * pq];
+#pragma unroll
+      for (int q = 1; q < M; ++q) {
+        float2 w = tw[(q - 1) * R + k];
+        if (S < 0) w.y = -w.y;
+        v[q] = cmul(v[q], w);
+      }
+      Dft<M, S>::run(v);
+#pragma unroll
+      for (int q = 0; q < M; ++q) d[place(q) * pq] = v[q];
+    }
+  }
+  template <int S>
+  static __device__ __forceinline__ void last3(const float2* b, int ld, float2 (&v)[3][R],
+                                               const float2* tw, int t) {
+    constexpr int pq = R * R + R * R / 16;
+    const float2* d = b + place(t / R) * pq;
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+      const int o = sw(q * R + t % R);
+#pragma unroll
+      for (int s = 0; s < 3; ++s) v[s][q] = d[s * ld + o];
+    }
+#pragma unroll
+    for (int q = 1; q < R; ++q) {
+      float2 w = tw[kTw2 + (q - 1) * G + t];
+      if (S < 0) w.y = -w.y;
+#pragma unroll
+      for (int s = 0; s < 3; ++s) v[s][q] = cmul(v[s][q], w);
+    }
+#pragma unroll
+    for (int s = 0; s < 3; ++s) Dft<R, S>::run(v[s]);
+  }
+  // barrier of the G threads of one team of a block whose threads are teams 0, 1, ... in order:
+  // within a warp, or a barrier of its own, or (teams that share warps unevenly) the whole block
+  static constexpr bool kOwnSync = G % 32 == 0 || 32 % G == 0;
+  static __device__ __forceinline__ void sync(int team) {
+    if constexpr (32 % G == 0) __syncwarp();
+    else if constexpr (G % 32 == 0)
+      asm volatile("bar.sync %0, %1;" ::"r"(3 + team), "n"(G) : "memory");
+    else
+      __syncthreads();
+  }
 };
 
 // sides with a plan: L, R, M
