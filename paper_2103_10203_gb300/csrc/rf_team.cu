@@ -94,10 +94,13 @@ Kernel solve_kernel(const rf_ctx* c) {
 // Block shape of a launch on G blocks with `W` workers at most: teams per block, rounds, shared
 // memory; false if a round's teams or the shared memory do not fit.
 bool shape_with(const rf_ctx* c, int G, bool final_pass, bool stream, Args& a, size_t* smem) {
-  const int gx = 3 * lanes_of(c->nx), gy = 3 * lanes_of(c->ny);
+  // the kernels of long square cells carry three sequences per thread of the row phase
+  const bool three = !final_pass && c->nx == c->ny && three_in_one(c->nx);
+  const int cap = three ? kMaxWorkers3 : kMaxWorkers;
+  const int gx = (three ? 1 : 3) * lanes_of(c->nx), gy = 3 * lanes_of(c->ny);
   const int units = c->ny / 2;
   const int ux = (units + G - 1) / G, uy = (c->Kx + G - 1) / G;   // per block, at most
-  auto teams = [](int want, int g) { return std::max(1, std::min(want, kMaxWorkers / g)); };
+  auto teams = [cap](int want, int g) { return std::max(1, std::min(want, cap / g)); };
   a.Px = teams(ux, gx);
   a.Py = final_pass ? 1 : teams(uy, gy);
   a.rounds_x = (ux + a.Px - 1) / a.Px;
@@ -114,7 +117,7 @@ bool shape_with(const rf_ctx* c, int G, bool final_pass, bool stream, Args& a, s
   a.o_twx = take(sizeof(float2) * twiddles_of(c->nx));
   a.o_kx = take(sizeof(int) * c->Kx);
   a.o_jmap = take(sizeof(short) * (c->nx / 2 + 1));
-  const size_t bx = (size_t)a.Px * 6 * (c->nx + c->nx / 16 + 2);
+  const size_t bx = (size_t)a.Px * (three ? 3 : 6) * (c->nx + c->nx / 16 + 2);
   const size_t by = final_pass ? 0 : (size_t)a.Py * 6 * (c->ny + c->ny / 16 + 2);
   a.o_buf = take(sizeof(float2) * std::max(bx, by));
   if (!final_pass) {
@@ -135,14 +138,16 @@ bool shape_with(const rf_ctx* c, int G, bool final_pass, bool stream, Args& a, s
     a.o_ep = take(sizeof(int) * a.entries_cap);
     a.st_stream = stream;
     a.o_p8 = take((size_t)a.Px * a.rounds_x * 2 * c->nx);
-    a.o_st = take(!c->has_plastic ? 0 : (size_t)a.Px * (stream ? 1 : a.rounds_x) * 2 * c->nx * 16);
+    const int held = stream ? (three ? 0 : 1) : a.rounds_x;   // row pairs of a team
+    a.o_st = take(!c->has_plastic ? 0 : (size_t)a.Px * held * 2 * c->nx * 16);
     if (a.cluster) {
       a.o_ts = take(sizeof(float4) * 3 * (size_t)a.Px * a.rounds_x * c->Kx);
       a.o_tp = take(sizeof(float2) * 3 * (size_t)nslot * c->ny);
     }
   }
   *smem = o;
-  return gx <= kMaxWorkers && gy <= kMaxWorkers && o <= kSmemMax;
+  // (the long square cells have no cluster form)
+  return gx <= cap && gy <= cap && o <= kSmemMax && !(three && a.cluster);
 }
 
 bool shape(const rf_ctx* c, int G, bool final_pass, Args& a, size_t* smem) {

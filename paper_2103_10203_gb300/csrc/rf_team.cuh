@@ -42,7 +42,13 @@
 namespace rfk {
 namespace team {
 
-constexpr int kMaxWorkers = 384;   // threads of all teams of a block
+constexpr int kMaxWorkers = 384;   // threads of all teams of a block, ...
+constexpr int kMaxWorkers3 = 512;  // ... and where a thread of the row phase carries three sequences
+// Square cells of these sides have several row pairs per block: their row phase is row_phase3.
+__host__ __device__ constexpr bool three_in_one(int side) { return side > 512; }
+__host__ __device__ constexpr int max_workers(int side) {
+  return three_in_one(side) ? kMaxWorkers3 : kMaxWorkers;
+}
 
 struct Args {
   float2* T1;            // strain lines, [u][3][Kx][2 rows]
@@ -212,7 +218,6 @@ __device__ __forceinline__ void row_phase(const Args& a, double* sb) {
       asm volatile("cp.async.commit_group;" ::: "memory");
     }
     float2 v[R];
-    const int row = row0 + (seq == 1 ? 1 : 0);   // the row whose voxels this thread takes (seq < 2)
     const int slot = team + a.Px * rd;
     if (on) {
       // points t + G q of the sequence's spectrum from the coefficients at kx = min(p, L - p)
@@ -363,6 +368,140 @@ __device__ __forceinline__ void row_phase(const Args& a, double* sb) {
   }
 }
 
+// Row phase of long square cells: a team of G threads per row pair, all three sequences in each
+// thread. With several row pairs per block the phase is bound by instructions and by the block's
+// barriers, no longer by one pair's latency: addresses, twiddles and barriers are shared by three
+// sequences, both rows' laws run on registers (the internal variables of a point come straight
+// from L2, fetched one point ahead), and the pairs of a block run independently of one another,
+// four at a time instead of one. A 1024^2 J2 load path (3365 updates): 182 -> 158 ms.
+template <int R, int M, bool PLASTIC>
+__device__ __forceinline__ void row_phase3(const Args& a) {
+  using P = Plan<R, M>;
+  constexpr int L = P::L, G = P::G, span = L + L / 16 + 2;
+  static_assert(G % 32 == 0, "a team has a barrier of its own");
+  const int team = threadIdx.x / G, t = threadIdx.x - team * G;
+  if (team >= a.Px) return;
+  const int Kx = a.Kx, Ny = a.Ny, units = a.Ny / 2;
+  const float2* tw = at<float2>(a.o_twx);
+  const short* jmap = at<short>(a.o_jmap);
+  const int* kxs = at<int>(a.o_kx);
+  float2* b = at<float2>(a.o_buf) + (long long)team * 3 * span;
+  const float lam0 = a.law.lam0, mu0 = a.law.mu0;
+  const DevPhase* phs = at<DevPhase>(a.o_ph);
+  for (int rd = 0; rd < a.rounds_x; ++rd) {
+    const int slot = team + a.Px * rd;
+    const int u = blockIdx.x + gridDim.x * slot;
+    if (u >= units) break;
+    const int row0 = 2 * u;
+    float2 v[3][R];
+    {
+      // points t + G q of the spectra from the coefficients at kx = min(p, L - p)
+      const float4* s = reinterpret_cast<const float4*>(a.T1) + (long long)u * 3 * Kx;
+#pragma unroll
+      for (int q = 0; q < R; ++q) {
+        const int p = t + G * q;
+        const int j = jmap[p <= L / 2 ? p : L - p];
+        float4 f[3];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          f[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (j >= 0) f[i] = __ldcg(s + i * Kx + j);   // line i of both rows
+        }
+        if (p == 0 || 2 * p == L) {   // self-conjugate positions of real lines
+#pragma unroll
+          for (int i = 0; i < 3; ++i) f[i].y = f[i].w = 0.f;
+        }
+        // x + i y below L / 2, conj(x) + i conj(y) above: 11 + i 22 of each row, 12 of both
+        const float sg = 2 * p <= L ? 1.f : -1.f;
+        v[0][q] = make_float2(fmaf(-sg, f[1].y, f[0].x), fmaf(sg, f[0].y, f[1].x));
+        v[1][q] = make_float2(fmaf(-sg, f[1].w, f[0].z), fmaf(sg, f[0].w, f[1].z));
+        v[2][q] = make_float2(fmaf(-sg, f[2].w, f[2].x), fmaf(sg, f[2].y, f[2].z));
+      }
+    }
+    P::template first3<+1>(v, b, span, t);
+    P::sync(team);
+    P::template middle3<+1>(b, span, tw, t);
+    const float4* st4 = at<float4>(a.o_st) + (long long)slot * 2 * L;
+    const float* sg = a.state + (long long)row0 * L;
+    auto fetch = [&](int q, float4 (&s)[2]) {   // internal variables of point t + G q of both rows
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        const int x = r * L + t + G * q;
+        if (a.st_stream)
+          s[r] = make_float4(__ldcg(sg + x), __ldcg(sg + a.N + x), __ldcg(sg + 2 * a.N + x),
+                             __ldcg(sg + 3 * a.N + x));
+        else
+          s[r] = st4[x];
+      }
+    };
+    float4 sn[2];
+    if (PLASTIC) fetch(0, sn);
+    P::sync(team);
+    P::template last3<+1>(b, span, v, tw, t);
+    const uint8_t* ph8 = at<uint8_t>(a.o_p8) + slot * 2 * L + t;
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+      float4 sc[2];
+      if (PLASTIC) {
+        sc[0] = sn[0];
+        sc[1] = sn[1];
+        if (q + 1 < R) fetch(q + 1, sn);
+      }
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        float& c12 = r ? v[2][q].y : v[2][q].x;
+        const float e6[6] = {v[r][q].x * a.invN, v[r][q].y * a.invN, 0.f, 0.f, 0.f, c12 * a.invN};
+        float ep[6] = {0, 0, 0, 0, 0, 0};
+        float alpha = 0.f;
+        if (PLASTIC) {
+          ep[0] = sc[r].x;
+          ep[1] = sc[r].y;
+          ep[5] = sc[r].z;
+          ep[2] = -(ep[0] + ep[1]);
+          alpha = sc[r].w;
+        }
+        LawOut o;
+        stress6<PLASTIC>(e6, phs[ph8[r * L + G * q]], ep, alpha, o);
+        const float tr = e6[0] + e6[1];
+        v[r][q] = make_float2(o.s[0] - (lam0 * tr + 2.f * mu0 * e6[0]),
+                              o.s[1] - (lam0 * tr + 2.f * mu0 * e6[1]));
+        c12 = o.s[5] - 2.f * mu0 * e6[5];
+      }
+    }
+    P::sync(team);
+    P::template first3<-1>(v, b, span, t);
+    P::sync(team);
+    P::template middle3<-1>(b, span, tw, t);
+    P::sync(team);
+    P::template last3<-1>(b, span, v, tw, t);
+    P::sync(team);
+#pragma unroll
+    for (int q = 0; q < R; ++q)
+#pragma unroll
+      for (int s = 0; s < 3; ++s) b[s * span + sw(t + G * q)] = v[s][q];
+    P::sync(team);
+    // the pattern's columns of both rows: 11 and 22 of a row from its sequence's even and odd
+    // parts, 12 of the two rows from those of the third
+    for (int j = t; j < Kx; j += G) {
+      const int k = kxs[j];
+      const int ik = sw(k), im = sw(k == 0 ? 0 : L - k);
+      float2 re[3], od[3];
+#pragma unroll
+      for (int s = 0; s < 3; ++s) {
+        const float2 zk = b[s * span + ik], zm = b[s * span + im];
+        re[s] = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));
+        od[s] = make_float2(0.5f * (zk.y + zm.y), -0.5f * (zk.x - zm.x));
+      }
+      float4* d = reinterpret_cast<float4*>(a.T1p + (long long)j * Ny + row0);
+      const long long cs = (long long)Kx * Ny / 2;
+      __stcg(d, make_float4(re[0].x, re[0].y, re[1].x, re[1].y));
+      __stcg(d + cs, make_float4(od[0].x, od[0].y, od[1].x, od[1].y));
+      __stcg(d + 2 * cs, make_float4(re[2].x, re[2].y, od[2].x, od[2].y));
+    }
+    P::sync(team);   // the buffers are reused by the next round
+  }
+}
+
 // Column phase of a block: its teams' kx, j = block + grid (team + Py round). full = false: only
 // the inverse transform of the held coefficients (the start of a solve). Leaves each thread's
 // FP64 squared-increment sum in the block's array and arrives at barrier 2.
@@ -487,6 +626,11 @@ __device__ __forceinline__ void col_phase(const Args& a, bool full) {
 // SIDE > 0: the kernel is compiled for square cells of that side; 0: any of the sides
 template <int SIDE, bool PLASTIC, bool FINAL>
 __device__ __forceinline__ void rows(const Args& a, double* sb) {
+  if constexpr (three_in_one(SIDE) && !FINAL) {
+    if constexpr (SIDE == 768) row_phase3<8, 12, PLASTIC>(a);
+    else row_phase3<8, 16, PLASTIC>(a);
+    return;
+  }
   switch (SIDE ? SIDE : a.Nx) {
 #define X(L, R, M) \
   case L: row_phase<R, M, PLASTIC, FINAL>(a, sb); break;
@@ -565,7 +709,7 @@ __device__ __forceinline__ bool grid_barrier(const Args& a, unsigned target, int
 }
 
 template <int SIDE, bool PLASTIC>
-__global__ __launch_bounds__(kMaxWorkers + 32, 1) void k_team2d(const __grid_constant__ Args a) {
+__global__ __launch_bounds__(max_workers(SIDE) + 32, 1) void k_team2d(const __grid_constant__ Args a) {
   __shared__ int s_flag, s_done;
   const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
   const bool worker = tid < a.W;

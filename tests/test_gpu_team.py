@@ -151,3 +151,23 @@ def test_3d_updates_are_the_ones_that_run(lib):
     macro = np.array([0.01, 0, 0, 0.002, 0, 0])
     assert check3(lib, pm, elastic_phases(), pat, macro)
     assert not check3(lib, pm, elastic_phases(), pat, macro, fft_fuse=-1)
+
+
+@pytest.mark.parametrize("side", [512, 768, 1024])
+def test_persistent_solve_plastic_path(lib, side):
+    """Two increments: the second reads committed internal variables (held in shared memory, or
+    fetched from global memory on the long sides)."""
+    pm = blocks((side, side), side)
+    pat = O.pattern_adapted(pm, 1, k_target(0.02, pm.size))
+    path = np.zeros((2, 6))
+    path[:, 0] = [0.008, 0.014]
+    path[:, 1] = [-0.002, -0.004]
+    s = lib.Solver(pm, j2_phases(), pattern=pat, tol=1e-2, max_iter=500, transform="fft", fft_fuse=3)
+    out = s.rf_solve_path(path)
+    eps, _, _ = s.rf_get_fields()
+    assert s.rf_get_info()["fft_fused"] == 3
+    s.close()
+    sbar, _, r = O.solve_path(pm, j2_phases(), path, pat, fixed_iters=out["iters"])
+    for n in range(len(path)):
+        assert rel(out["sigma_bar"][n], sbar[n]) <= SBAR_TOL
+    assert rel(eps, field(r.eps)) <= EPS_TOL
