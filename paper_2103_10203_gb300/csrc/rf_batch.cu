@@ -27,6 +27,7 @@
 #include "rf_fftcore.cuh"
 #include "rf_internal.cuh"
 #include "rf_law.cuh"
+#include "rf_teamfft.cuh"
 
 namespace rfk {
 
@@ -764,7 +765,7 @@ __global__ __launch_bounds__(256, 2) void kb_row_w(BArgs a) {
 constexpr int kResWarps = 8;
 constexpr int kResThreads = 32 * kResWarps;
 constexpr int kResMaxL = 256;
-constexpr int kResPhaseBytes = 640;   // a warp item's phase ids (at most 10 rows of 64, 5 of 128)
+constexpr int kResTw = 256;   // twiddles of a row transform
 
 struct ResCtx {
   float2* T;            // the block's line transforms, [Ny][NC Kx]
@@ -789,13 +790,10 @@ struct ResShared {
   int kxs[kResMaxL / 2 + 1];
   int inv_ky[kResMaxL];   // position of ky (mod Ny) in the pattern's ky list, or -1
   int next, done;
-  __align__(16) uint8_t phs[kResWarps][kResPhaseBytes];
+  float2 tw[kResTw];
+  short jmap[kResMaxL / 2 + 1];   // index of kx in the pattern's kx list, or -1
 };
 
-__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
-}
 // 8 bytes, zero-filled when bytes = 0 (nothing is read then)
 __device__ __forceinline__ void cp_async8(void* dst, const void* src, int bytes) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
@@ -869,154 +867,167 @@ __device__ __noinline__ void res_cols(ResShared& sh, float2* Wr, int lane, int w
   }
 }
 
-// row passes: warp items of R_w = 2 S / 3 rows (3 R_w lines, packed in pairs into at most S
-// sequences at a stride of L + P entries, which keeps the transform's scattered writes free of
-// bank conflicts), each warp on its own items; one transform body for both directions. Final
-// pass: homogenised-stress sums per warp instead of the forward transform.
+// Row passes: a team of G lanes per pair of rows, each lane with its points of all three packed
+// sequences (11 + i 22 of each row, 12 of both) of a team transform; 32 / G pairs in flight per
+// warp, each warp on its own. The first inverse pass reads its points straight from the line
+// transforms through the position map (no zeroed and scattered spectra), both rows' laws run on
+// registers, and only the passes of the transforms cross the warp's region (a sequence in one
+// lane's 32 registers, with spectra, strains and polarizations staged through the region: 1024 RVEs
+// of 64 to 256 14.8 ms, so 11.9).
+// Final pass: homogenised-stress sums per warp instead of the forward transform.
+template <int P>
+struct ResPlan;
+template <>
+struct ResPlan<2> : team::Plan<8, 1> {};
+template <>
+struct ResPlan<3> : team::Plan<4, 6> {};
+template <>
+struct ResPlan<4> : team::Plan<8, 2> {};
+template <>
+struct ResPlan<6> : team::Plan<8, 3> {};
+template <>
+struct ResPlan<8> : team::Plan<8, 4> {};
+
 template <int P>
 __device__ __noinline__ void res_rows(ResShared& sh, float2* Wr, int lane, int wp, bool final) {
-  constexpr int L = 32 * P, S = 32 / P, RW = (2 * S) / 3, LS = L + P;
-  constexpr int SU = (3 * RW + 1) / 2;   // sequences in use (3 of 4 at P = 8)
-  static_assert(S * LS <= kWRegion && RW * L <= kResPhaseBytes, "region");
+  using F = ResPlan<P>;
+  using team::sw;
+  constexpr int L = F::L, G = F::G, R = L / G, M = G / R, TW = 32 / G;
+  constexpr int span = L + L / 16 + 2;
+  static_assert(L == 32 * P && TW * 3 * span <= kWRegion && F::kTw <= kResTw, "region");
   const ResCtx& c = sh.c;
   const int Kx = c.Kx, NCK = c.NCK;
-  const float2* tab = c.tab;
-  uint8_t* phs = sh.phs[wp];
-  const int items = (L + RW - 1) / RW;
+  const int tm = lane / G, t = lane - tm * G;   // (lanes beyond the last whole team are idle)
+  float2* b = Wr + min(tm, TW - 1) * 3 * span;
+  const float2* tw = sh.tw;
+  constexpr int items = (L / 2 + TW - 1) / TW;
+  double s6[6] = {0, 0, 0, 0, 0, 0};
   for (int it = wp; it < items; it += kResWarps) {
-    const int y0 = it * RW, nr = min(RW, L - y0), nl = nr * NC, nseq = (nl + 1) / 2;
-    // the item's phase ids: asynchronous 16-byte copies, waited for before the law
-    for (int k = lane; k < nr * L / 16; k += 32)
-      cp_async16(phs + 16 * k, c.phase + (long long)y0 * L + 16 * k);
-    for (int i = lane; i < SU * LS; i += 32) Wr[i] = make_float2(0.f, 0.f);
-    __syncwarp();
-    // z_p = line 2p + i line 2p+1 (line s = r NC + c of the item): z[k] = ta + i tb,
-    // z[L - k] = conj(ta) + i conj(tb)
-    float2* Tg = c.T + (long long)y0 * NCK;
-    for (int u0 = lane; u0 < nseq * Kx; u0 += 4 * 32) {
-      float2 ta[4], tb[4];
-      int jj[4], pp[4];
+    const int u = it * TW + tm;
+    const bool on = tm < TW && u < L / 2;
+    const uint8_t* ph = c.phase + (long long)2 * u * L + t;
+    float2* Tg = c.T + (long long)2 * u * NCK;
+    float2 v[3][R];
+    uint8_t pid[2][R];
+    if (on) {
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int u = u0 + q * 32;
-        pp[q] = -1;
-        if (u < nseq * Kx) {
-          const int p = fdiv(u, c.dKx), j = u - p * Kx;
-          const int s0 = 2 * p, s1 = s0 + 1;
-          ta[q] = Tg[s0 * Kx + j];
-          tb[q] = s1 < nl ? Tg[s1 * Kx + j] : make_float2(0.f, 0.f);
-          pp[q] = p;
-          jj[q] = j;
-        }
-      }
+      for (int q = 0; q < R; ++q) {
+        const int p = t + G * q;
+        const int j = sh.jmap[p <= L / 2 ? p : L - p];
+        float2 f[2][NC];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        if (pp[q] < 0) continue;
-        const int k = sh.kxs[jj[q]];
-        const bool self = (k == 0) || (2 * k == L);
-        if (self) {
-          ta[q].y = 0.f;
-          tb[q].y = 0.f;
-        }
-        float2* z = Wr + pp[q] * LS;
-        z[k] = make_float2(ta[q].x - tb[q].y, ta[q].y + tb[q].x);
-        if (!self) z[L - k] = make_float2(ta[q].x + tb[q].y, tb[q].x - ta[q].y);
-      }
-    }
-    __syncwarp();
-#pragma unroll 1
-    for (int pass = 0; pass < 2; ++pass) {
-      const float cj = pass == 0 ? -1.f : 1.f;   // pass 0: inverse, as the conjugate trick
-      float2 v[32];
+        for (int r = 0; r < 2; ++r)
 #pragma unroll
-      for (int s = 0; s < SU; ++s)
-#pragma unroll
-        for (int n1 = 0; n1 < P; ++n1) {
-          const float2 z = Wr[s * LS + 32 * n1 + lane];
-          v[s * P + n1] = make_float2(z.x, cj * z.y);
-        }
-#pragma unroll
-      for (int r = SU * P; r < 32; ++r) v[r] = make_float2(0.f, 0.f);
-      fwd_batch_cb<P, SU>(v, Wr, tab, lane, [] {});
-      if (lane < SU * P) {
-        const int s = lane / P, k1 = lane - s * P;
-#pragma unroll
-        for (int k2 = 0; k2 < 32; ++k2)
-          Wr[s * LS + k1 + P * k2] = make_float2(v[k2].x, cj * v[k2].y);
-      }
-      __syncwarp();
-      if (pass == 1) break;
-      cp_async_wait_all();
-      __syncwarp();
-      // the law on the item's voxels, two rows at a time: rows 2m and 2m + 1 hold lines
-      // 6m .. 6m + 5, i.e. whole sequences 3m, 3m + 1 and 3m + 2 (read and written as float2);
-      // a missing row 2m + 1 leaves zeros in its carriers
-      double s6[6] = {0, 0, 0, 0, 0, 0};
-      for (int vx = lane; vx < (nr + 1) / 2 * L; vx += 32) {
-        const int m = vx / L, x = vx - m * L;
-        const bool two = 2 * m + 1 < nr;
-        float2* zA = Wr + 3 * m * LS + x;
-        const float2 A = zA[0], B = zA[LS];
-        const float2 Cz = two ? zA[2 * LS] : make_float2(0.f, 0.f);
-        const float ev[2][NC] = {{A.x, A.y, B.x}, {B.y, Cz.x, Cz.y}};
-        float tv[2][NC] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          if (h == 1 && !two) break;
-          float e[NC];
-#pragma unroll
-          for (int cc = 0; cc < NC; ++cc) e[cc] = ev[h][cc] * c.invN;
-          const int pid = phs[(2 * m + h) * L + x];
-          if (final) {
-            float e6[6];
-            comp_to6<NC>(e, e6);
-            const DevPhase ph = sh.ph[pid];
-            float ep[6] = {0, 0, 0, 0, 0, 0};
-            LawOut o;
-            stress6<false>(e6, ph, ep, 0.f, o);
-#pragma unroll
-            for (int i = 0; i < 6; ++i) s6[i] += (double)o.s[i];
-          } else {
-            // elastic phases in plane strain: tau = sigma - C0 : eps
-            //   = (lambda - lambda0) tr(eps) 1 + 2 (mu - mu0) eps, components 11, 22, 12
-            const float2 dm = sh.dph[pid];
-            const float tr = e[0] + e[1];
-            tv[h][0] = fmaf(dm.y, e[0], dm.x * tr);
-            tv[h][1] = fmaf(dm.y, e[1], dm.x * tr);
-            tv[h][2] = dm.y * e[2];
+          for (int i = 0; i < NC; ++i) {
+            f[r][i] = make_float2(0.f, 0.f);
+            if (j >= 0) f[r][i] = Tg[r * NCK + i * Kx + j];
           }
-        }
-        if (!final) {
-          zA[0] = make_float2(tv[0][0], tv[0][1]);
-          zA[LS] = make_float2(tv[0][2], tv[1][0]);
-          if (two) zA[2 * LS] = make_float2(tv[1][1], tv[1][2]);
-        }
-      }
-      if (final) {
+        if (p == 0 || 2 * p == L) {   // self-conjugate positions of real lines
 #pragma unroll
-        for (int i = 0; i < 6; ++i) {
-          double t = s6[i];
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-          if (lane == 0) sh.sb[wp][i] += t;
+          for (int i = 0; i < NC; ++i) f[0][i].y = f[1][i].y = 0.f;
         }
-        break;
+        // x + i y below L / 2, conj(x) + i conj(y) above
+        const float sg = 2 * p <= L ? 1.f : -1.f;
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+          v[r][q] = make_float2(fmaf(-sg, f[r][1].y, f[r][0].x), fmaf(sg, f[r][0].y, f[r][1].x));
+        v[2][q] = make_float2(fmaf(-sg, f[1][2].y, f[0][2].x), fmaf(sg, f[0][2].y, f[1][2].x));
       }
+#pragma unroll
+      for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int q = 0; q < R; ++q) pid[r][q] = ph[r * L + G * q];
+      F::template first3<+1>(v, b, span, t);
+    }
+    __syncwarp();
+    if (M > 1) {
+      if (on) F::template middle3<+1>(b, span, tw, t);
       __syncwarp();
     }
-    if (!final) {
-      for (int u = lane; u < nl * Kx; u += 32) {
-        const int sl = fdiv(u, c.dKx), j = u - sl * Kx;
+    if (on) F::template last3<+1>(b, span, v, tw, t);
+    __syncwarp();
+    if (final) {
+      if (on) {
+#pragma unroll
+        for (int q = 0; q < R; ++q)
+#pragma unroll
+          for (int s = 0; s < 3; ++s) b[s * span + sw(t + G * q)] = v[s][q];
+        // (each lane reads what it wrote)
+#pragma unroll 1
+        for (int i = 0; i < 2 * R; ++i) {
+          const int r = i / R, q = i - r * R;
+          const float2 z = b[r * span + sw(t + G * q)], zc = b[2 * span + sw(t + G * q)];
+          const float e6[6] = {z.x * c.invN, z.y * c.invN, 0.f, 0.f, 0.f,
+                               (r ? zc.y : zc.x) * c.invN};
+          float ep[6] = {0, 0, 0, 0, 0, 0};
+          LawOut o;
+          stress6<false>(e6, sh.ph[ph[r * L + G * q]], ep, 0.f, o);
+#pragma unroll
+          for (int k = 0; k < 6; ++k) s6[k] += (double)o.s[k];
+        }
+      }
+      __syncwarp();
+      continue;
+    }
+    if (on) {
+      // elastic phases in plane strain: tau = sigma - C0 : eps
+      //   = (lambda - lambda0) tr(eps) 1 + 2 (mu - mu0) eps, components 11, 22, 12
+#pragma unroll
+      for (int q = 0; q < R; ++q)
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          const float2 dm = sh.dph[pid[r][q]];
+          float& c12 = r ? v[2][q].y : v[2][q].x;
+          const float e0 = v[r][q].x * c.invN, e1 = v[r][q].y * c.invN, e2 = c12 * c.invN;
+          const float tr = dm.x * (e0 + e1);
+          v[r][q] = make_float2(fmaf(dm.y, e0, tr), fmaf(dm.y, e1, tr));
+          c12 = dm.y * e2;
+        }
+      F::template first3<-1>(v, b, span, t);
+    }
+    __syncwarp();
+    if (M > 1) {
+      if (on) F::template middle3<-1>(b, span, tw, t);
+      __syncwarp();
+    }
+    if (on) F::template last3<-1>(b, span, v, tw, t);
+    __syncwarp();
+    if (on) {
+#pragma unroll
+      for (int q = 0; q < R; ++q)
+#pragma unroll
+        for (int s = 0; s < 3; ++s) b[s * span + sw(t + G * q)] = v[s][q];
+    }
+    __syncwarp();
+    if (on) {
+      for (int j = t; j < Kx; j += G) {
         const int k = sh.kxs[j];
-        const float2* z = Wr + (sl >> 1) * LS;
-        const float2 zk = z[k], zm = z[k == 0 ? 0 : L - k];
-        float2 out;
-        if ((sl & 1) == 0) out = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));
-        else out = make_float2(0.5f * (zk.y + zm.y), -0.5f * (zk.x - zm.x));
-        Tg[sl * Kx + j] = out;
+        const int ik = sw(k), im = sw(k == 0 ? 0 : L - k);
+        float2 re[3], od[3];
+#pragma unroll
+        for (int s = 0; s < 3; ++s) {
+          const float2 zk = b[s * span + ik], zm = b[s * span + im];
+          re[s] = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));
+          od[s] = make_float2(0.5f * (zk.y + zm.y), -0.5f * (zk.x - zm.x));
+        }
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          Tg[r * NCK + j] = re[r];
+          Tg[r * NCK + Kx + j] = od[r];
+          Tg[r * NCK + 2 * Kx + j] = r ? od[2] : re[2];
+        }
       }
     }
-    __syncwarp();   // the next item rewrites the region and the phase bytes
+    __syncwarp();   // the next item rewrites the region
+  }
+  if (final) {
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      double x = s6[i];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+      if (lane == 0) sh.sb[wp][i] = x;
+    }
   }
 }
 
@@ -1076,6 +1087,7 @@ __device__ bool res_decide(BStat& st, int* n_done, double s) {
 template <int P>
 __device__ __noinline__ void res_solve(ResShared& sh, float2* Wr, int* n_done) {
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  ResPlan<P>::twiddles(sh.c.tab, sh.tw);   // (a block barrier follows the column transforms)
   for (;;) {
     res_cols<P>(sh, Wr, lane, wp, true);
     __syncthreads();
@@ -1145,7 +1157,9 @@ __global__ __launch_bounds__(kResThreads, 2) void kb_resident(BArgs a, const int
                                         2.f * (sh.ph[threadIdx.x].mu - d.mu0));
     for (int i = threadIdx.x; i < d.Kx; i += kResThreads) sh.kxs[i] = a.kx[d.off_kx + i];
     for (int i = threadIdx.x; i < d.ny; i += kResThreads) sh.inv_ky[i] = -1;
+    for (int i = threadIdx.x; i <= nx / 2; i += kResThreads) sh.jmap[i] = -1;
     __syncthreads();
+    for (int i = threadIdx.x; i < d.Kx; i += kResThreads) sh.jmap[sh.kxs[i]] = (short)i;
     for (int i = threadIdx.x; i < d.Ky; i += kResThreads) sh.inv_ky[a.kym[d.off_ky + i]] = i;
     __syncthreads();
     switch (nx) {
