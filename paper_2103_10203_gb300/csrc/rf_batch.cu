@@ -900,11 +900,15 @@ __device__ __noinline__ void res_rows(ResShared& sh, float2* Wr, int lane, int w
   const int tm = lane / G, t = lane - tm * G;   // (lanes beyond the last whole team are idle)
   float2* b = Wr + min(tm, TW - 1) * 3 * span;
   const float2* tw = sh.tw;
-  constexpr int items = (L / 2 + TW - 1) / TW;
+  constexpr int items = L / 2 / TW;
+  static_assert(L / 2 % TW == 0, "whole items");
   double s6[6] = {0, 0, 0, 0, 0, 0};
   for (int it = wp; it < items; it += kResWarps) {
     const int u = it * TW + tm;
-    const bool on = tm < TW && u < L / 2;
+    // Lanes without a pair only skip what is written; the last passes run in every lane: behind a
+    // branch, a lane's 48 values were spilled around it (1024 RVEs 11.9 ms, so 10.5; the row passes
+    // of a 96^2 RVE 58k -> 40k clocks per update).
+    const bool on = 32 % G == 0 || tm < TW;
     const uint8_t* ph = c.phase + (long long)2 * u * L + t;
     float2* Tg = c.T + (long long)2 * u * NCK;
     float2 v[3][R];
@@ -944,19 +948,19 @@ __device__ __noinline__ void res_rows(ResShared& sh, float2* Wr, int lane, int w
       if (on) F::template middle3<+1>(b, span, tw, t);
       __syncwarp();
     }
-    if (on) F::template last3<+1>(b, span, v, tw, t);
+    F::template last3<+1>(b, span, v, tw, t);
     __syncwarp();
     if (final) {
       if (on) {
 #pragma unroll
         for (int q = 0; q < R; ++q)
 #pragma unroll
-          for (int s = 0; s < 3; ++s) b[s * span + sw(t + G * q)] = v[s][q];
+          for (int s = 0; s < 3; ++s) b[s * span + F::pt(t, q)] = v[s][q];
         // (each lane reads what it wrote)
 #pragma unroll 1
         for (int i = 0; i < 2 * R; ++i) {
           const int r = i / R, q = i - r * R;
-          const float2 z = b[r * span + sw(t + G * q)], zc = b[2 * span + sw(t + G * q)];
+          const float2 z = b[r * span + F::pt(t, q)], zc = b[2 * span + F::pt(t, q)];
           const float e6[6] = {z.x * c.invN, z.y * c.invN, 0.f, 0.f, 0.f,
                                (r ? zc.y : zc.x) * c.invN};
           float ep[6] = {0, 0, 0, 0, 0, 0};
@@ -990,13 +994,13 @@ __device__ __noinline__ void res_rows(ResShared& sh, float2* Wr, int lane, int w
       if (on) F::template middle3<-1>(b, span, tw, t);
       __syncwarp();
     }
-    if (on) F::template last3<-1>(b, span, v, tw, t);
+    F::template last3<-1>(b, span, v, tw, t);
     __syncwarp();
     if (on) {
 #pragma unroll
       for (int q = 0; q < R; ++q)
 #pragma unroll
-        for (int s = 0; s < 3; ++s) b[s * span + sw(t + G * q)] = v[s][q];
+        for (int s = 0; s < 3; ++s) b[s * span + F::pt(t, q)] = v[s][q];
     }
     __syncwarp();
     if (on) {

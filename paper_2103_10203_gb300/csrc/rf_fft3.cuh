@@ -125,7 +125,7 @@ __global__ __launch_bounds__(256, 2) void k_row3(const __grid_constant__ RowArgs
 #pragma unroll
         for (int q = 0; q < R; ++q)
 #pragma unroll
-          for (int s = 0; s < 3; ++s) b[s * span + sw(t + G * q)] = v[s][q];
+          for (int s = 0; s < 3; ++s) b[s * span + P::pt(t, q)] = v[s][q];
       }
       P::sync(team);
 #pragma unroll 1
@@ -196,7 +196,7 @@ __global__ __launch_bounds__(256, 2) void k_row3(const __grid_constant__ RowArgs
 #pragma unroll
       for (int q = 0; q < R; ++q)
 #pragma unroll
-        for (int s = 0; s < 3; ++s) b[s * span + sw(t + G * q)] = v[s][q];
+        for (int s = 0; s < 3; ++s) b[s * span + P::pt(t, q)] = v[s][q];
     }
     P::sync(team);
     if (on) {
@@ -388,11 +388,11 @@ __global__ __launch_bounds__(384, 2) void k_zphase(const __grid_constant__ ZArgs
       }
       P::template last<-1>(M == 1 ? b0 : b1, v, tw, t);
 #pragma unroll
-      for (int q = 0; q < R; ++q) Z[sw(t + G * q)] = v[q];
+      for (int q = 0; q < R; ++q) Z[P::pt(t, q)] = v[q];
     }
     __syncthreads();
 #pragma unroll
-    for (int q = 0; q < R; ++q) W[sw(t + G * q)] = make_float2(0.f, 0.f);
+    for (int q = 0; q < R; ++q) W[P::pt(t, q)] = make_float2(0.f, 0.f);
     __syncthreads();
     const float2* zc = bufs + (M == 1 ? C * pitch : 0);   // column cc of Z at zc + cc pitch
     float2* wc = bufs + (M == 1 ? 0 : C * pitch);
@@ -437,7 +437,7 @@ __global__ __launch_bounds__(384, 2) void k_zphase(const __grid_constant__ ZArgs
     }
     __syncthreads();
 #pragma unroll
-    for (int q = 0; q < R; ++q) v[q] = W[sw(t + G * q)];
+    for (int q = 0; q < R; ++q) v[q] = W[P::pt(t, q)];
     P::template first<+1>(v, Z, t);
     __syncthreads();
     if (M > 1) {

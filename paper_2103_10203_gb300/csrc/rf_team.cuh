@@ -270,7 +270,7 @@ __device__ __forceinline__ void row_phase(const Args& a, double* sb) {
       if (FINAL || seq == 2) {
         float2* x = M == 1 ? b1 : b0;   // X2 of the third sequence
 #pragma unroll
-        for (int q = 0; q < R; ++q) x[sw(t + G * q)] = v[q];
+        for (int q = 0; q < R; ++q) x[P::pt(t, q)] = v[q];
       }
     }
     if (PLASTIC && !FINAL && a.st_stream) asm volatile("cp.async.wait_all;" ::: "memory");
@@ -316,7 +316,7 @@ __device__ __forceinline__ void row_phase(const Args& a, double* sb) {
     if (on) {
       if (seq == 2) {
 #pragma unroll
-        for (int q = 0; q < R; ++q) v[q] = X2[sw(t + G * q)];
+        for (int q = 0; q < R; ++q) v[q] = X2[P::pt(t, q)];
       }
       P::template first<-1>(v, Y, t);
     }
@@ -329,7 +329,7 @@ __device__ __forceinline__ void row_phase(const Args& a, double* sb) {
       P::template last<-1>(M == 1 ? Y : Xo, v, tw, t);
       float2* z = M == 1 ? Xo : Y;
 #pragma unroll
-      for (int q = 0; q < R; ++q) z[sw(t + G * q)] = v[q];
+      for (int q = 0; q < R; ++q) z[P::pt(t, q)] = v[q];
     }
     workers_sync(a.W);
     if (on) {
@@ -478,7 +478,7 @@ __device__ __forceinline__ void row_phase3(const Args& a) {
 #pragma unroll
     for (int q = 0; q < R; ++q)
 #pragma unroll
-      for (int s = 0; s < 3; ++s) b[s * span + sw(t + G * q)] = v[s][q];
+      for (int s = 0; s < 3; ++s) b[s * span + P::pt(t, q)] = v[s][q];
     P::sync(team);
     // the pattern's columns of both rows: 11 and 22 of a row from its sequence's even and odd
     // parts, 12 of the two rows from those of the third
@@ -551,7 +551,7 @@ __device__ __forceinline__ void col_phase(const Args& a, bool full) {
         P::template last<-1>(M == 1 ? b0 : b1, v, tw, t);
         float2* z = M == 1 ? b1 : b0;
 #pragma unroll
-        for (int q = 0; q < R; ++q) z[sw(t + G * q)] = v[q];
+        for (int q = 0; q < R; ++q) z[P::pt(t, q)] = v[q];
       }
       workers_sync(a.W);
       if (on) {

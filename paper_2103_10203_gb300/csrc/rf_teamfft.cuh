@@ -126,6 +126,14 @@ template <int R, int M>
 struct Plan {
   static constexpr int L = R * R * M, G = R * M;
 
+  // sw(t + G q). Where G is no multiple of 16 the pad does not grow evenly with q; written so, the
+  // R places of a thread come from a few bases (two for G = 24) instead of an address each (which
+  // the passes of sides 96 and 192 spilled).
+  static __device__ __forceinline__ int pt(int t, int q) {
+    const int n = G * q, r = n & 15;
+    return sw(t + r) + (n - r) + (n - r) / 16;
+  }
+
   // stage-major twiddles: (M - 1) R of the middle pass, then (R - 1) G of the last
   static constexpr int kTw2 = (M - 1) * R, kTw = kTw2 + (R - 1) * G;
 
@@ -176,7 +184,7 @@ struct Plan {
   template <int S>
   static __device__ __forceinline__ void last(const float2* b, float2* v, const float2* tw, int t) {
 #pragma unroll
-    for (int q = 0; q < R; ++q) v[q] = b[sw(t + G * q)];
+    for (int q = 0; q < R; ++q) v[q] = b[pt(t, q)];
 #pragma unroll
     for (int q = 1; q < R; ++q) {
       float2 w = tw[kTw2 + (q - 1) * G + t];
