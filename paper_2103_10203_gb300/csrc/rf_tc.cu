@@ -389,6 +389,242 @@ __global__ __launch_bounds__(128) void k_tc_row(TcRowArgs a) {
                  "r"(a.tmem_cols));
 }
 
+// ------------------------------------------------------------------------------------------
+// The row kernel with its twiddles held (BF16 parts, one j' tile): a persistent CTA per SM loads the
+// 128 KB of its x slice's tiles once, and four groups of 128 threads take tiles of R rows in turn,
+// each with a buffer and an accumulator pair of its own, so that one group's staging, law or stores
+// run beside another's products.
+//
+// k_tc_row fetches the same 128 KB for every tile of R rows (268 MB through L2 per update of a 128^3
+// cell) and runs its stages one after the other with eight warps per SM. Here a tile costs its
+// lines in and out only. The polarization takes the place of the staged lines, which the first
+// product has read by then: without that only two groups would fit beside the twiddles. Core
+// matrices lie with 16 bytes between neighbours along K, so that the law's two-byte stores of a warp
+// (four core matrices) hit different banks. 128^3, K = 2 %: row pass 106 -> 54 us.
+constexpr int kHeldGroups = 4;
+constexpr int kHeldBytes = 8 * kTileBytes;   // inverse and forward twiddles: two chunks, hi and lo
+constexpr int kHeldMaxJ = kTile / 2;         // kx columns of the one j' tile
+
+__host__ __device__ constexpr int held_k_pitch(int Qp) { return Qp / 8 * 128 + 16; }
+// one operand part of a group: Qp rows of 256 bytes, 16 core matrices along K
+__host__ __device__ constexpr int held_part(int Qp) { return 16 * held_k_pitch(Qp); }
+__host__ __device__ constexpr size_t held_smem(int Qp) {
+  return kHeldBytes + kHeldGroups * 2 * (size_t)held_part(Qp) + sizeof(float) * kHeldMaxJ + 128;
+}
+
+// Barrier of a group's 128 threads; true if any of them brings true.
+__device__ __forceinline__ bool group_any(int grp, bool x) {
+  int r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %1, 0;\n\t"
+      "barrier.cta.red.or.pred q, %2, 128, p;\n\tselp.b32 %0, 1, 0, q;\n\t}\n"
+      : "=r"(r)
+      : "r"((int)x), "r"(1 + grp)
+      : "memory");
+  return r != 0;
+}
+
+template <int NC, bool PLASTIC>
+__global__ __launch_bounds__(128 * kHeldGroups, 1) void k_tc_row_held(const __grid_constant__ TcRowArgs a) {
+  if (a.done && *a.done) return;
+  using E = EBf16;
+  extern __shared__ __align__(1024) unsigned char smem[];
+  const int part = held_part(a.Qp), kp = held_k_pitch(a.Qp);
+  unsigned char* ops = smem + kHeldBytes;
+  float* fac = reinterpret_cast<float*>(ops + kHeldGroups * 2 * part);
+  // twiddles, a barrier per group, and one that nothing completes (the stall test)
+  uint64_t* bars = reinterpret_cast<uint64_t*>(fac + kHeldMaxJ);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 + kHeldGroups);
+
+  const int tid = threadIdx.x, warp = tid >> 5, grp = tid >> 7, gt = tid & 127;
+  const int xs = blockIdx.x, x = xs * kTile + gt;
+  const int Q = a.R * NC, lines = a.rows * NC;
+  unsigned char* hi = ops + grp * 2 * part;   // the group's operand parts
+  unsigned char* lo = hi + part;
+  uint64_t* mbar = bars + 1 + grp;
+
+  if (tid == 0) {
+    mbar_init(&bars[0], 4);
+    for (int i = 1; i < 2 + kHeldGroups; ++i) mbar_init(&bars[i], 1);
+    asm volatile("fence.mbarrier_init.release.cluster;");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(
+        smem_u32(tmem_slot)));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  if (tid < kHeldMaxJ) fac[tid] = tid < a.Kx ? a.fac[tid] : 0.f;
+  asm volatile("tcgen05.fence::before_thread_sync;");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;");
+  const uint32_t tmem = *tmem_slot;
+  const uint32_t d1 = tmem + (uint32_t)(2 * a.Qp * grp), d2 = d1 + (uint32_t)a.Qp;
+  const uint32_t lanes = (uint32_t)(32 * (warp & 3)) << 16;
+  const uint32_t id_mma = idesc<E>(kTile, a.Qp);
+
+  bool bad = false;
+  if (a.stall) bad = __syncthreads_or(tid == 0 && !mbar_wait(&bars[1 + kHeldGroups], 0, a.wait_limit));
+  bool loads = false;
+  if (!bad) {
+    loads = true;
+    if (tid == 0) {
+      const unsigned char* pi = a.phiI + (long long)xs * 4 * kTileBytes;
+      const unsigned char* pf = a.phiF + (long long)xs * 4 * kTileBytes;
+      for (int i = 0; i < 2; ++i) {
+        bulk_load(smem + 2 * i * kTileBytes, pi + 2 * i * kTileBytes, 2 * kTileBytes, &bars[0]);
+        bulk_load(smem + (4 + 2 * i) * kTileBytes, pf + 2 * i * kTileBytes, 2 * kTileBytes, &bars[0]);
+      }
+    }
+  }
+
+  // the 24 products of one transform: chunks of 64 along K, hi hi + hi lo + lo hi
+  auto products = [&](uint32_t d, const unsigned char* tw) {
+    const uint32_t a0 = smem_u32(tw), b_hi = smem_u32(hi), b_lo = smem_u32(lo);
+    for (int s = 0; s < 8; ++s) {
+      const uint32_t oa = (uint32_t)((s >> 2) * 2 * kTileBytes + (s & 3) * 256);
+      const uint32_t ob = (uint32_t)(2 * s * kp), sbo_a = (kChunkBytes / 16) * 128;
+      const uint64_t ah = make_desc(a0 + oa, 128, sbo_a);
+      const uint64_t al = make_desc(a0 + oa + kTileBytes, 128, sbo_a);
+      const uint64_t bh = make_desc(b_hi + ob, (uint32_t)kp, 128);
+      const uint64_t bl = make_desc(b_lo + ob, (uint32_t)kp, 128);
+      mma<E>(d, ah, bh, id_mma, s == 0 ? 0u : 1u);
+      mma<E>(d, ah, bl, id_mma, 1u);
+      mma<E>(d, al, bh, id_mma, 1u);
+    }
+    mma_commit(mbar);
+  };
+
+  int issued = 0;   // product phases of this group
+  const int tiles = (a.rows + a.R - 1) / a.R;
+  bool first = true;
+  // A wait that gives up is agreed on at the group's next barrier: no thread leaves the loop before
+  // the others of its group know.
+  for (int tile = bad ? tiles : blockIdx.y + gridDim.y * grp; tile < tiles;
+       tile += gridDim.y * kHeldGroups) {
+    const int row0 = tile * a.R, line0 = row0 * NC;
+    // the tile's lines, scaled and split: item (line q, 16-byte segment sg of four kx) with the
+    // low three bits of q fastest (a warp's stores fill whole core matrices); zeros beyond
+    const float2* tp = a.T + (long long)line0 * a.Kx;
+    const int items = a.Qp * 16;
+    for (int i0 = gt; i0 < items; i0 += 2 * 128) {
+      float2 t[2][4];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int i = i0 + u * 128, q = ((i >> 7) << 3) | (i & 7), j0 = ((i >> 3) & 15) * 4;
+        const bool live = i < items && q < Q && line0 + q < lines;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          t[u][k] = make_float2(0.f, 0.f);
+          if (live && j0 + k < a.Kx) t[u][k] = tp[(long long)q * a.Kx + j0 + k];
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int i = i0 + u * 128, q = ((i >> 7) << 3) | (i & 7), sg = (i >> 3) & 15;
+        if (i >= items) continue;
+        float v[8];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float f = fac[sg * 4 + k];
+          v[2 * k] = f * t[u][k].x;
+          v[2 * k + 1] = f * t[u][k].y;
+        }
+        uint4 h, l;
+        split_seg<E>(v, h, l);
+        const int off = sg * kp + (q >> 3) * 128 + (q & 7) * 16;
+        *reinterpret_cast<uint4*>(hi + off) = h;
+        *reinterpret_cast<uint4*>(lo + off) = l;
+      }
+    }
+    if (first && !mbar_wait(&bars[0], 0, a.wait_limit)) bad = true;
+    first = false;
+    asm volatile("fence.proxy.async.shared::cta;");
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    bad = group_any(grp, bad);
+    if (bad) break;
+    if (gt == 0) {
+      asm volatile("tcgen05.fence::after_thread_sync;");
+      products(d1, smem);
+    }
+    ++issued;
+    // phase ids while the products run
+    uint8_t pid[kMaxQ / NC];
+#pragma unroll
+    for (int r = 0; r < kMaxQ / NC; ++r) {
+      pid[r] = 0;
+      if (r < a.R && row0 + r < a.rows && x < a.Nx) pid[r] = a.phase[(long long)(row0 + r) * a.Nx + x];
+    }
+    // law: eps for x = this thread's lane
+    bad = !__all_sync(0xffffffffu, mbar_wait(mbar, (issued - 1) & 1, a.wait_limit));
+    if (!bad) {
+      asm volatile("tcgen05.fence::after_thread_sync;");
+      float ev[kMaxQ];
+#pragma unroll
+      for (int c0 = 0; c0 < kMaxQ; c0 += 16)
+        if (c0 < a.Qp) tmem_ld16(d1 + lanes + c0, ev + c0);
+#pragma unroll
+      for (int r = 0; r < kMaxQ / NC; ++r) {
+        if (r >= a.R) break;
+        const int row = row0 + r;
+        float tv[6] = {0, 0, 0, 0, 0, 0};
+        if (row < a.rows && x < a.Nx) {
+          float e6[6], ep[6] = {0, 0, 0, 0, 0, 0}, alpha = 0.f;
+          comp_to6<NC>(ev + r * NC, e6);
+          if (PLASTIC) load_state<NC>(a.state, a.N, (long long)row * a.Nx + x, ep, alpha);
+          LawOut o;
+          stress6<PLASTIC>(e6, a.law.ph[pid[r]], ep, alpha, o);
+          const float tr = e6[0] + e6[1] + e6[2];
+#pragma unroll
+          for (int i = 0; i < 3; ++i) tv[i] = o.s[i] - (a.law.lam0 * tr + 2.f * a.law.mu0 * e6[i]);
+#pragma unroll
+          for (int i = 3; i < 6; ++i) tv[i] = o.s[i] - 2.f * a.law.mu0 * e6[i];
+        }
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+          const int q = r * NC + c;   // (rows Q .. Qp keep the zeros of the staging)
+          put_split<E>(hi, lo, (uint32_t)((gt >> 3) * kp + (q >> 3) * 128 + (q & 7) * 16 + (gt & 7) * 2),
+                       tv[comp6<NC>(c)]);
+        }
+      }
+    }
+    asm volatile("fence.proxy.async.shared::cta;");
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    bad = group_any(grp, bad);
+    if (bad) break;
+    if (gt == 0) {
+      asm volatile("tcgen05.fence::after_thread_sync;");
+      products(d2, smem + 4 * kTileBytes);
+    }
+    ++issued;
+    bad = !__all_sync(0xffffffffu, mbar_wait(mbar, (issued - 1) & 1, a.wait_limit));
+    if (!bad) {
+      asm volatile("tcgen05.fence::after_thread_sync;");
+      float ov[kMaxQ];
+#pragma unroll
+      for (int c0 = 0; c0 < kMaxQ; c0 += 16)
+        if (c0 < a.Qp) tmem_ld16(d2 + lanes + c0, ov + c0);
+      if (gt < 2 * a.Kx) {
+        float* to = a.Tout + ((long long)xs * lines + line0) * (2LL * a.Kx) + gt;
+#pragma unroll
+        for (int q = 0; q < kMaxQ; ++q) {
+          if (q >= Q || line0 + q >= lines) break;
+          to[(long long)q * 2 * a.Kx] = ov[q];
+        }
+      }
+    }
+  }
+  if (__syncthreads_or(bad)) {
+    // a wait gave up: report it, then let the copies and products in flight finish (each barrier's
+    // last issued phase, with the default limit) before tensor memory is released
+    if (tid == 0) atomicExch(a.err, 1);
+    if (loads) mbar_wait(&bars[0], 0);
+    if (issued > 0) mbar_wait(mbar, (issued - 1) & 1);
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;");
+  __syncthreads();
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
+}
+
 }  // namespace tc
 
 // ------------------------------------------------------------------------------------------
@@ -459,12 +695,36 @@ void init_attributes_tc() {
   cudaFuncSetAttribute(k_tc_row<ETf32, 3, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, s);
   cudaFuncSetAttribute(k_tc_row<ETf32, 6, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, s);
   cudaFuncSetAttribute(k_tc_row<ETf32, 6, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, s);
+  const int h = (int)held_smem(kMaxQ);
+  static_assert(held_smem(kMaxQ) <= 227 * 1024, "shared memory of a block");
+  cudaFuncSetAttribute(k_tc_row_held<3, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, h);
+  cudaFuncSetAttribute(k_tc_row_held<3, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, h);
+  cudaFuncSetAttribute(k_tc_row_held<6, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, h);
+  cudaFuncSetAttribute(k_tc_row_held<6, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, h);
 }
 
 template <class E, int NC, bool PL>
 static int tc_row_launch(rf_ctx* c, const tc::TcRowArgs& a) {
   dim3 grid(c->tc_nXS, (c->rows + c->tc_R - 1) / c->tc_R);
   tc::k_tc_row<E, NC, PL><<<grid, 128, c->tc_smem, c->stream>>>(a);
+  c->launches += 1;
+  cudaError_t e = cudaGetLastError();
+  return e == cudaSuccess ? RF_OK : cuda_fail(e, "tc row");
+}
+
+// BF16 parts of a pattern with at most 64 kx: the held twiddles fit beside four groups (128^3 33
+// updates 4954 us with staged twiddles, so 3355; TF32 parts and wider patterns take 256 KB and more
+// and stay with k_tc_row). At most R rows per tile, as many as give every group the same number of
+// tiles.
+template <int NC, bool PL>
+static int tc_row_held_launch(rf_ctx* c, tc::TcRowArgs a) {
+  using namespace tc;
+  int sms = 152;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->dev);
+  const int gy = std::max(1, std::min(sms / a.nXS, (a.rows + a.R - 1) / a.R));
+  const int groups = gy * kHeldGroups, rounds = (a.rows + groups * a.R - 1) / (groups * a.R);
+  a.R = std::min(a.R, (a.rows + groups * rounds - 1) / (groups * rounds));
+  k_tc_row_held<NC, PL><<<dim3(a.nXS, gy), 128 * kHeldGroups, held_smem(a.Qp), c->stream>>>(a);
   c->launches += 1;
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? RF_OK : cuda_fail(e, "tc row");
@@ -497,6 +757,10 @@ int launch_tc_row(rf_ctx* c, const int* done) {
   a.stall = c->opt.stall_test;
   const bool bf = c->opt.precision == RF_PREC_SPLIT_BF16;
   const bool pl = c->has_plastic;
+  if (bf && c->tc_nJT == 1) {
+    if (c->nc == 3) return pl ? tc_row_held_launch<3, true>(c, a) : tc_row_held_launch<3, false>(c, a);
+    return pl ? tc_row_held_launch<6, true>(c, a) : tc_row_held_launch<6, false>(c, a);
+  }
   if (c->nc == 3) {
     if (bf) return pl ? tc_row_launch<tc::EBf16, 3, true>(c, a) : tc_row_launch<tc::EBf16, 3, false>(c, a);
     return pl ? tc_row_launch<tc::ETf32, 3, true>(c, a) : tc_row_launch<tc::ETf32, 3, false>(c, a);
