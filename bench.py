@@ -497,7 +497,8 @@ def run_learned(args, rf, torch):
 def _tc_mma_flops(nx, rows, nc, Kx):
     """Tensor-core FLOPs one k_tc_row launch issues (split operands: 3 products per GEMM), from
     the kernel's tiling: 128-wide x slices, R rows per block (tensor-memory limit), Qp = R nc
-    padded to 16, the j' = 2 Kx range padded to 128."""
+    padded to 16, the j' = 2 Kx range padded to 128. (k_tc_row_held issues the same products per
+    tile and may take fewer rows per tile.)"""
     jt = (2 * Kx + 127) // 128
     R = 16 if nc == 3 else 8
     qp = lambda r: ((r * nc + 15) // 16) * 16
@@ -582,7 +583,9 @@ def run_3d(args, rf, torch):
             "iterations_per_solve": its / args.steps, "gpu_launches": int(launches),
             "roofline": {"bound": "tensor", "achieved": achieved, "peak": peak,
                          "unit": "TFLOP/s", "frac": achieved / peak, "traffic": None,
-                         "kernel": "k_tc_row", "launch_ms": row_ms,
+                         "kernel": "k_tc_row_held" if prec == "split_bf16" and info["Kx"] <= 64
+                                   else "k_tc_row",
+                         "launch_ms": row_ms,
                          "mma_flops_per_launch": mma,
                          "peak_source": "MEASURED_PEAKS.json bf16_tflops (cuBLAS bf16 burst)"
                                         + ("" if prec == "split_bf16" else " / 2 (TF32 nominal ratio)")},
@@ -832,10 +835,11 @@ def main():
     props = torch.cuda.get_device_properties(local)
     kernel_names = {("fft", "row"): "k_fft_row", ("fft", "column_phase"): "k_fft_colphase",
                     ("fft", "inverse_y"): "k_fft_cols",
-                    ("fft", "forward_y"): "k_fft_cols", ("dft", "row"): "k_row",
-                    ("dft", "inverse_y"): "k_dft_axis", ("dft", "forward_y"): "k_dft_axis"}
+                    ("fft", "forward_y"): "k_fft_cols", ("dft", "row"): "k_row_dft",
+                    ("dft", "inverse_y"): "k_axis_dft", ("dft", "forward_y"): "k_axis_dft"}
     if args.precision != "fp32" and dom == "row":
-        kernel_names[("dft", "row")] = "k_tc_row"
+        held = args.precision == "split_bf16" and info["Kx"] <= 64
+        kernel_names[("dft", "row")] = "k_tc_row_held" if held else "k_tc_row"
     if tile_info and tile_info.get("fft_row_warps"):
         kernel_names[("fft", "row")] = "k_fft_row_w"
     if tile_info and tile_info.get("fft_fused") == 4:
@@ -846,10 +850,12 @@ def main():
         kernel_names[("fft", "row")] = "k_persist_w (row phase)"
         kernel_names[("fft", "column_phase")] = "k_persist_w (column phase)"
     if tile_info and tile_info.get("fft_fused") == 3:
-        # the persistent solve: one kernel; its stages are the row and the column phase, each
-        # timed up to its grid barrier by global-timer stamps of block 0
-        kernel_names[("fft", "row")] = "k_persist2d (row phase)"
-        kernel_names[("fft", "column_phase")] = "k_persist2d (column phase)"
+        # the persistent solve: one kernel (on team FFTs up to 1024 voxels a side); its stages are
+        # the row and the column phase, each timed up to its grid barrier by global-timer stamps of
+        # block 0
+        kp = "k_team2d" if max(pm.shape) <= 1024 else "k_persist2d"
+        kernel_names[("fft", "row")] = kp + " (row phase)"
+        kernel_names[("fft", "column_phase")] = kp + " (column phase)"
     if args.transform == "fft" and dom in ("row", "inverse_y", "forward_y", "column_phase"):
         hbm = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))["hbm_gbs"] \
             if os.path.exists(os.path.join(ROOT, "MEASURED_PEAKS.json")) else 6800.0
