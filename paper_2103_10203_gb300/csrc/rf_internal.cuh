@@ -209,6 +209,8 @@ struct rf_ctx {
   int dft_U = 0;
   int2* d_zrange = nullptr;             // 3D on team FFTs: entries of each (ky, kx) ...
   short* d_ymap = nullptr;              // ... and the rectangle row of each position along y
+  // barrier words of the persistent solves (arrivals, generation), and the finished blocks of the
+  // team solve's final pass, which only that pass writes and leaves zero
   unsigned* d_bar = nullptr;
   unsigned long long* d_ptrace = nullptr;
   int* d_jptr = nullptr;                // [Kx + 1] offsets of each kx's entries in d_jlist

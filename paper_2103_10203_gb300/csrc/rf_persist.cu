@@ -636,10 +636,10 @@ bool persist_geometry(rf_ctx* c, int threads, int per_sm) {
 // Barrier words and a first geometry (the autotuner may choose another); RF_ERR_INVALID if
 // no geometry fits co-resident.
 int persist_setup(rf_ctx* c) {
-  if (int e = palloc(c, &c->d_bar, 2, "persistent solve")) return e;
+  if (int e = palloc(c, &c->d_bar, 3, "persistent solve")) return e;
   const size_t fin = 8 * (size_t)std::max(1, c->ny / 2);
   if (int e = palloc(c, &c->d_fin, fin, "persistent solve")) return e;
-  const cudaError_t e = cudaMemsetAsync(c->d_bar, 0, 2 * sizeof(unsigned), c->stream);
+  const cudaError_t e = cudaMemsetAsync(c->d_bar, 0, 3 * sizeof(unsigned), c->stream);
   if (e != cudaSuccess) return cuda_fail(e, "persistent solve");
   const int cand[4][2] = {{512, 2}, {256, 2}, {512, 1}, {256, 1}};
   for (const auto& cd : cand)

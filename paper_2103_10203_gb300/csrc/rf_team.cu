@@ -180,7 +180,7 @@ Args make_args(rf_ctx* c) {
   a.st = c->d_status;
   a.part = c->d_part;
   a.fin_part = c->d_fin;
-  a.fin_count = c->d_bar + 1;
+  a.fin_count = c->d_bar + 2;   // (the other persistent solves leave a generation in the second word)
   a.sbar_dev = c->d_sbar;
   a.sbar_host = c->h_sbar;
   a.st_host = c->h_status;
