@@ -107,7 +107,7 @@ int launch_fft3_row(rf_ctx* c, const int* done, bool final_pass, int commit, int
   a.table = c->d_twx;
   a.Kx = c->Kx;
   a.rows = c->rows;
-  a.teams = 256 / s.lanes;
+  a.teams = row_teams(s.lanes);
   a.groups = (c->rows + a.teams - 1) / a.teams;
   a.N = c->N;
   a.invN = (float)(1.0 / (double)c->N);
@@ -123,7 +123,7 @@ int launch_fft3_row(rf_ctx* c, const int* done, bool final_pass, int commit, int
   }
   RowKernel k = c->has_plastic ? row_kernel_plastic(c->nx, final_pass)
                                : row_kernel_elastic(c->nx, final_pass);
-  const int threads = a.teams * s.lanes;
+  const int threads = row_threads(s.lanes);
   const size_t smem = sizeof(float2) * (((s.tw + 1) & ~1) + (size_t)a.teams * 3 * even_span(c->nx)) +
                       sizeof(int) * c->Kx + sizeof(short) * (c->nx / 2 + 1) + 16;
   const int grid = fill(c, (const void*)k, threads, smem, a.groups);

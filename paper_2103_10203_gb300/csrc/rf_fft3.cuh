@@ -28,6 +28,14 @@ using fftc::sw;
 
 extern __shared__ __align__(16) unsigned char z_smem[];
 
+// Row pass: teams of `lanes` threads per block, and the block's threads. Whole warps (252 and 240
+// threads of teams of 12, 24 and 48 make 256): the final pass sums its stresses with shuffles of
+// all 32 lanes, and a lane that does not exist hands over no defined value.
+__host__ __device__ constexpr int row_teams(int lanes) { return 256 / lanes; }
+__host__ __device__ constexpr int row_threads(int lanes) {
+  return (row_teams(lanes) * lanes + 31) / 32 * 32;
+}
+
 struct RowArgs3 {
   const float2* T;      // [rows][6][Kx]
   float2* Tout;
@@ -58,6 +66,7 @@ __global__ __launch_bounds__(256, 2) void k_row3(const __grid_constant__ RowArgs
   using P = Plan<R, M>;
   constexpr int L = P::L, G = P::G;
   constexpr int span = (L + L / 16 + 2) & ~1;
+  static_assert(row_threads(G) % 32 == 0 && row_threads(G) <= 256, "whole warps");
   __shared__ DevPhase phs[kMaxPhases];
   __shared__ double red[32];
   float2* tw = reinterpret_cast<float2*>(z_smem);
@@ -79,12 +88,13 @@ __global__ __launch_bounds__(256, 2) void k_row3(const __grid_constant__ RowArgs
   grid_dep_wait();
   if (!FINAL && a.done && __ldcg(a.done)) return;   // the same flag value for every thread
   __syncthreads();
-  float2* b = bufs + team * 3 * span;
+  // (threads beyond the last team only take part in the block's barriers and sums)
+  float2* b = bufs + min(team, a.teams - 1) * 3 * span;
   const float lam0 = a.law.lam0, mu0 = a.law.mu0;
   double sb[6] = {0, 0, 0, 0, 0, 0}, vmax = 0.0;
   for (int g = blockIdx.x; g < a.groups; g += gridDim.x) {
     const int row = g * a.teams + team;
-    const bool on = row < a.rows;
+    const bool on = team < a.teams && row < a.rows;
     float2 v[3][R];
     uint8_t pid[R];
     if (on) {

@@ -9,7 +9,7 @@ import pytest
 
 import oracle as O
 from synth import random_discs
-from synth.configs import j2_phases, k_target
+from synth.configs import elastic_phases, j2_phases, k_target
 
 pytestmark = pytest.mark.gpu
 
@@ -34,4 +34,21 @@ def test_first_solve_after_the_tuner_timed_every_persistent_form(lib):
         assert off_average(s, s.rf_solve(macro)["sigma_bar"]) <= TOL
     out = s.rf_solve_path(macro * np.array([0.5, 1.0])[:, None])
     assert off_average(s, out["sigma_bar"][-1]) <= TOL
+    s.close()
+
+
+@pytest.mark.parametrize("nx", [48, 64, 96, 192, 384])
+@pytest.mark.parametrize("plastic", [False, True])
+def test_3d_final_pass(lib, nx, plastic):
+    """Rows whose teams do not fill their last warp (48, 96, 192, 384), and one that does."""
+    shape = (64, 64, nx)
+    pm = np.zeros(shape, np.uint8)
+    pm[10:40, 5:50, 3:nx // 2] = 1
+    pat = O.pattern_adapted(pm, 1, k_target(0.02, pm.size))
+    s = lib.Solver(pm, j2_phases() if plastic else elastic_phases(), pattern=pat, tol=0.0,
+                   max_iter=3, transform="fft")
+    s.rf_set_tracing(True)
+    out = s.rf_solve(np.array([0.015, -0.004, 0.002, 0.001, 0.003, -0.002]))
+    assert s.rf_get_stage_times()["column_phase"][1] == 3   # the updates on team FFTs ran
+    assert off_average(s, out["sigma_bar"]) <= TOL
     s.close()
