@@ -657,7 +657,7 @@ int rf_create(rf_ctx** out, const rf_grid* grid, int32_t n_phases, const rf_phas
     d.lam = (float)phases[p].lambda;
     d.mu = (float)phases[p].mu;
     d.plastic = phases[p].plastic ? 1 : 0;
-    d.sy = d.plastic ? (float)phases[p].sigma_y0 : 3.0e38f;   // no yield
+    d.sy = d.plastic ? (float)phases[p].sigma_y0 : INFINITY;   // no yield
     d.H = d.plastic ? (float)phases[p].hardening : 0.f;
     d.r3muH = d.plastic ? (float)(1.0 / (3.0 * phases[p].mu + phases[p].hardening)) : 0.f;
     any_plastic = any_plastic || d.plastic;

@@ -27,7 +27,7 @@ namespace rfk {
 constexpr int kMaxPhases = 16;
 constexpr int kGammaBlock = 128;   // threads per Green-operator block (one frequency each)
 
-// sy: initial yield stress; beyond any stress for an elastic phase
+// sy: initial yield stress; infinite for an elastic phase
 struct DevPhase {
   float lam, mu, sy, H;
   int plastic;

@@ -1,0 +1,40 @@
+"""The J2 law at the ends of FP32's range, in every kernel that evaluates it."""
+
+import numpy as np
+import pytest
+
+from synth.configs import j2_phases
+
+pytestmark = pytest.mark.gpu
+
+# grid, transform options: one per row kernel
+KERNELS = [((32, 32), dict(transform="fft")), ((32, 32), dict(transform="fft", fft_fuse=3)),
+           ((32, 32), dict(transform="fft", fft_fuse=-1)), ((40, 40), dict(transform="dft")),
+           ((1024, 1024), dict(transform="fft", fft_fuse=3)),
+           ((64, 64, 64), dict(transform="fft")), ((32, 32, 40), dict(transform="dft")),
+           ((40, 40), dict(transform="dft", precision="split_bf16")),
+           ((40, 40), dict(transform="dft", precision="split_tf32"))]
+
+
+def indices():
+    ph = j2_phases()
+    pl = [i for i, p in enumerate(ph) if p["plastic"]][0]
+    el = [i for i, p in enumerate(ph) if not p["plastic"]][0]
+    return ph, pl, el
+
+
+def waves(dim):
+    return np.array([[-1, 0, 0], [0, 0, 0], [1, 0, 0]], np.int32)
+
+
+@pytest.mark.parametrize("shape,opts", KERNELS)
+def test_overflowing_invariant_of_a_yielding_phase_is_an_error(lib, shape, opts):
+    """mu eps = 1e19: the squared invariant overflows, the trial stress itself does not. A J2 phase
+    must not hand that trial stress back as if it had not yielded."""
+    ph, pl, _ = indices()
+    pm = np.full(shape, pl, np.uint8)
+    s = lib.Solver(pm, ph, pattern=waves(len(shape)), tol=1e-3, max_iter=20, **opts)
+    with pytest.raises(lib.RFError) as e:
+        s.rf_solve(np.array([1e18, 0, 0, 0, 0, 0]))
+    assert e.value.code == -3
+    s.close()
