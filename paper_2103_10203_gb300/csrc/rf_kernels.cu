@@ -824,7 +824,10 @@ int launch_gamma_finalize(rf_ctx* c, const int* done) {
   g.cond = c->while_cond;
   g.use_cond = c->capturing_while ? 1 : 0;
   const unsigned gb = (unsigned)((c->Kh + kGammaBlock - 1) / kGammaBlock);
-  g.early = gb <= 76 ? 1 : 0;
+  // the inverse transform's blocks take their places on the SMs beside this kernel's, where they stay:
+  // a few blocks hide the launch (97 x 50: 21.5 -> 19.9 us per update), 20 and more leave the next
+  // kernel unevenly spread (600 x 400, 50 blocks: 125 -> 142 us; 4096 x 64, 58: 45 -> 49 us)
+  g.early = gb <= 16 ? 1 : 0;
   trace_stage(c, 5);
   const cudaError_t le =
       c->nc == 3 ? launch_pdl(k_gamma<3>, dim3(gb), dim3(kGammaBlock), 0, c->stream, g, (double)c->N)
