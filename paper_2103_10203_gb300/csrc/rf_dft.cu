@@ -292,8 +292,6 @@ struct AxisDftArgs {
   const float2* in;
   float2* out;
   long long in_bstride, out_bstride;
-  int splits;           // dense input: partial sums to add up (row passes over slices of x), ...
-  long long split_stride;
   int L, N, S;          // length, columns, sparse rows
   const int* vals;      // [S] frequency (mod L) of each sparse row
   const float2* table;  // exp(+2 pi i t / L)
@@ -306,6 +304,25 @@ struct AxisDftArgs {
 // otherwise sparse -> dense (exp(+)). A block takes 32 columns; each of its four warps MP dense
 // pairs (y, L - y) or MP sparse rows, over chunks of kC rows staged in shared memory.
 constexpr int kC = 64;
+
+// Sum of `splits` arrays of n values, `stride` apart (the row passes over slices of x): every block
+// of a transform reads all its lines, so adding them up on the way in read each slice once per
+// block of rows (1024^2 with every kx, split BF16, eight slices: 3550 us per update, so 907).
+__global__ __launch_bounds__(256) void k_sum_slices(const float2* in, int splits, long long stride,
+                                                    long long n, float2* out, const int* done) {
+  grid_dep_wait();
+  if (done && __ldcg(done)) return;
+  for (long long i = blockIdx.x * 256LL + threadIdx.x; i < n; i += gridDim.x * 256LL) {
+    float2 v = __ldcg(in + i);
+#pragma unroll 4
+    for (int s = 1; s < splits; ++s) {
+      const float2 u = __ldcg(in + s * stride + i);
+      v.x += u.x;
+      v.y += u.y;
+    }
+    out[i] = v;
+  }
+}
 
 template <int MP, bool FWD>
 __global__ __launch_bounds__(128) void k_axis_dft(const __grid_constant__ AxisDftArgs a) {
@@ -353,23 +370,6 @@ __global__ __launch_bounds__(128) void k_axis_dft(const __grid_constant__ AxisDf
           if (FWD && y > 0 && 2 * y != L) q[u] = __ldcg(in + (long long)(L - y) * a.N + n);
         }
       }
-      if (FWD && n < a.N)
-        for (int s = 1; s < a.splits; ++s) {
-          const float2* is = in + s * a.split_stride + n;
-#pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            const int r = r0 + 4 * u, y = k0 + r;
-            if (r >= kn) break;
-            const float2 e = __ldcg(is + (long long)y * a.N);
-            p[u].x += e.x;
-            p[u].y += e.y;
-            if (y > 0 && 2 * y != L) {
-              const float2 f = __ldcg(is + (long long)(L - y) * a.N);
-              q[u].x += f.x;
-              q[u].y += f.y;
-            }
-          }
-        }
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         const int r = r0 + 4 * u, y = k0 + r;
@@ -519,13 +519,20 @@ int launch_row_dft(rf_ctx* c, const int* done, bool final_pass, int commit, int*
   return pl ? row_dft<6, true, false>(c, a, nb, smem) : row_dft<6, false, false>(c, a, nb, smem);
 }
 
-// sign +1: S sparse rows -> L dense ones, -1: the reverse; N columns, `batch` arrays
+// sign +1: S sparse rows -> L dense ones, -1: the reverse (of `splits` partial sums); N columns,
+// `batch` arrays
 int launch_axis_dft(rf_ctx* c, const float2* in, int splits, long long split_stride,
                     long long in_bs, float2* out, long long out_bs, int L, int N, int S, int batch,
                     const int* vals, const float2* table, int sign, const int* done) {
+  if (splits > 1) {   // partial sums of the row pass, which leaves its other output free
+    const long long n = split_stride;
+    const int grid = (int)std::min<long long>((n + 255) / 256, 8LL * sm_count(c));
+    const cudaError_t e = launch_pdl(k_sum_slices, dim3(grid), dim3(256), 0, c->stream, in, splits,
+                                     split_stride, n, c->d_T1p, done);
+    if (int r = dft_check(c, e, "sum of slices")) return r;
+    in = c->d_T1p;
+  }
   AxisDftArgs a{};
-  a.splits = splits;
-  a.split_stride = split_stride;
   a.in = in;
   a.out = out;
   a.in_bstride = in_bs;
