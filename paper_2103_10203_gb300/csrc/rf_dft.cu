@@ -298,11 +298,14 @@ struct AxisDftArgs {
   FastDiv dL;
   const int* done;
   int early;
+  int ranks;            // blocks of one cluster (along the grid's z) that share a transform's sum
 };
 
 // Transform along one axis of [batch][rows][N]: FWD dense rows -> the S sparse ones (exp(-)),
 // otherwise sparse -> dense (exp(+)). A block takes 32 columns; each of its four warps MP dense
-// pairs (y, L - y) or MP sparse rows, over chunks of kC rows staged in shared memory.
+// pairs (y, L - y) or MP sparse rows, over chunks of kC rows staged in shared memory. Where a long
+// sum meets few results (2000 x 7, one frequency: 1001 pairs on one block; update 37 -> 17 us), the
+// blocks of a cluster take a share of the chunks each and add up their sums in rank order.
 constexpr int kC = 64;
 
 // Sum of `splits` arrays of n values, `stride` apart (the row passes over slices of x): every block
@@ -331,17 +334,20 @@ __global__ __launch_bounds__(128) void k_axis_dft(const __grid_constant__ AxisDf
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n0 = blockIdx.x * 32, m0 = blockIdx.y * 4 * MP, L = a.L, np = L / 2 + 1;
   const int n = n0 + lane;
-  const float2* in = a.in + (long long)blockIdx.z * a.in_bstride;
-  float2* out = a.out + (long long)blockIdx.z * a.out_bstride;
+  const int bz = blockIdx.z / a.ranks, rank = blockIdx.z - bz * a.ranks;
+  const float2* in = a.in + (long long)bz * a.in_bstride;
+  float2* out = a.out + (long long)bz * a.out_bstride;
   float2* xs2 = reinterpret_cast<float2*>(xs4);
-  const int K = FWD ? np : a.S, M = FWD ? a.S : np;
+  const int K = FWD ? np : a.S, M = FWD ? a.S : np, chunks = (K + kC - 1) / kC;
+  // this block's rows of the sum
+  const int kbeg = chunks * rank / a.ranks * kC, kend = min(K, chunks * (rank + 1) / a.ranks * kC);
   float ar[MP], ai[MP], br[MP], bi[MP];
 #pragma unroll
   for (int i = 0; i < MP; ++i) ar[i] = ai[i] = br[i] = bi[i] = 0.f;
   if (a.early) grid_dep_launch();
   // twiddles of a chunk: pair y (dense) and frequency v (sparse) meet at t = y v mod L
   auto twiddles = [&](int k0) {
-    const int kn = min(kC, K - k0);
+    const int kn = min(kC, kend - k0);
     for (int i = tid; i < kn * 4 * MP; i += 128) {
       const int kk = i / (4 * MP), mm = i - kk * 4 * MP, m = m0 + mm;
       float2 w = make_float2(0.f, 0.f);
@@ -353,12 +359,12 @@ __global__ __launch_bounds__(128) void k_axis_dft(const __grid_constant__ AxisDf
       ws[kk][mm] = w;
     }
   };
-  twiddles(0);   // the pattern's alone
+  twiddles(kbeg);   // the pattern's alone
   grid_dep_wait();
-  if (a.done && __ldcg(a.done)) return;
-  for (int k0 = 0; k0 < K; k0 += kC) {
-    const int kn = min(kC, K - k0);
-    if (k0 > 0) twiddles(k0);
+  if (a.done && __ldcg(a.done)) return;   // the same flag value for every thread
+  for (int k0 = kbeg; k0 < kend; k0 += kC) {
+    const int kn = min(kC, kend - k0);
+    if (k0 > kbeg) twiddles(k0);
     for (int r0 = warp; r0 < kn; r0 += 4 * 8) {
       float2 p[8], q[8];
 #pragma unroll
@@ -411,21 +417,44 @@ __global__ __launch_bounds__(128) void k_axis_dft(const __grid_constant__ AxisDf
     }
     __syncthreads();
   }
-  if (n >= a.N) return;
-#pragma unroll
-  for (int i = 0; i < MP; ++i) {
-    const int m = m0 + warp * MP + i;
-    if (m >= M) break;
+  auto put = [&](int m, int col, float vr, float vi, float wr, float wi) {
+    if (m >= M || col >= a.N) return;
     if (FWD) {
       // (s.x c + d.y s, s.y c - d.x s)
-      out[(long long)m * a.N + n] = make_float2(ar[i] + br[i], ai[i] - bi[i]);
+      out[(long long)m * a.N + col] = make_float2(vr + wr, vi - wi);
     } else {
       // x c - y s, y c + x s at m; the conjugate twiddle at L - m
-      out[(long long)m * a.N + n] = make_float2(ar[i] - br[i], ai[i] + bi[i]);
+      out[(long long)m * a.N + col] = make_float2(vr - wr, vi + wi);
       if (m > 0 && 2 * m != L)
-        out[(long long)(L - m) * a.N + n] = make_float2(ar[i] + br[i], ai[i] - bi[i]);
+        out[(long long)(L - m) * a.N + col] = make_float2(vr + wr, vi - wi);
     }
+  };
+  if (a.ranks == 1) {
+#pragma unroll
+    for (int i = 0; i < MP; ++i) put(m0 + warp * MP + i, n, ar[i], ai[i], br[i], bi[i]);
+    return;
   }
+  // [4 MP][128 threads] partial sums in place of the staged rows, which every warp has read
+  float* part = reinterpret_cast<float*>(xs4);
+#pragma unroll
+  for (int i = 0; i < MP; ++i) {
+    part[(4 * i) * 128 + tid] = ar[i];
+    part[(4 * i + 1) * 128 + tid] = ai[i];
+    part[(4 * i + 2) * 128 + tid] = br[i];
+    part[(4 * i + 3) * 128 + tid] = bi[i];
+  }
+  cluster_sync();
+  const int per = 128 / a.ranks;   // this block adds up the sums of that many threads
+  for (int q = tid; q < per * MP; q += 128) {
+    const int i = q / per, t = rank * per + q - i * per;
+    float v[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int r = 0; r < a.ranks; ++r)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) v[k] += ld_cluster(part + (4 * i + k) * 128 + t, r);
+    put(m0 + (t >> 5) * MP + i, n0 + (t & 31), v[0], v[1], v[2], v[3]);
+  }
+  __syncwarp();
+  cluster_sync();   // no block leaves while another still reads its sums
 }
 
 }  // namespace dftk
@@ -550,15 +579,17 @@ int launch_axis_dft(rf_ctx* c, const float2* in, int splits, long long split_str
   // every SM several blocks
   const long long b4 = (long long)((N + 31) / 32) * ((M + 15) / 16) * batch;
   const bool wide = b4 >= 4LL * sms;
-  const dim3 grid((N + 31) / 32, wide ? (M + 15) / 16 : (M + 7) / 8, batch);
-  a.early = (long long)grid.x * grid.y * grid.z <= 64;
-  cudaError_t e;
-  if (wide)
-    e = sign < 0 ? launch_pdl(k_axis_dft<4, true>, grid, dim3(128), 0, c->stream, a)
-                 : launch_pdl(k_axis_dft<4, false>, grid, dim3(128), 0, c->stream, a);
-  else
-    e = sign < 0 ? launch_pdl(k_axis_dft<2, true>, grid, dim3(128), 0, c->stream, a)
-                 : launch_pdl(k_axis_dft<2, false>, grid, dim3(128), 0, c->stream, a);
+  dim3 grid((N + 31) / 32, wide ? (M + 15) / 16 : (M + 7) / 8, batch);
+  const long long blocks = (long long)grid.x * grid.y * batch;
+  const int chunks = ((sign < 0 ? L / 2 + 1 : S) + kC - 1) / kC;
+  a.ranks = 1;
+  while (a.ranks < 8 && blocks * 2 * a.ranks <= sms && 2 * a.ranks <= chunks) a.ranks *= 2;
+  grid.z *= a.ranks;
+  a.early = blocks * a.ranks <= 64;
+  const auto kern = wide ? (sign < 0 ? k_axis_dft<4, true> : k_axis_dft<4, false>)
+                         : (sign < 0 ? k_axis_dft<2, true> : k_axis_dft<2, false>);
+  const cudaError_t e =
+      launch_pdl_cluster(kern, grid, dim3(128), dim3(1, 1, a.ranks), 0, c->stream, a);
   return dft_check(c, e, "dft axis");
 }
 

@@ -173,11 +173,6 @@ __device__ __forceinline__ void put_out(const GemmArgs& g, int m, int n, float x
   g.C[(long long)m * g.ldc + n] = x;
 }
 
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
 // TN = kTN: one CTA per tile. TN = kTNs: gridDim.z CTAs of one cluster share a tile's K chunks.
 template <class E, bool AK, bool BK, int EPI, int TN>
 __global__ __launch_bounds__(128) void k_gemm(GemmArgs g) {
@@ -274,15 +269,7 @@ __global__ __launch_bounds__(128) void k_gemm(GemmArgs g) {
     const int m = m0 + tid;
     for (int c = TN * rank / S; c < TN * (rank + 1) / S; ++c) {
       float x = 0.f;
-      for (int q = 0; q < S; ++q) {
-        uint32_t src;
-        asm("mapa.shared::cluster.u32 %0, %1, %2;"
-            : "=r"(src)
-            : "r"(smem_u32(part + c * kTM + tid)), "r"(q));
-        float y;
-        asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(y) : "r"(src) : "memory");
-        x += y;
-      }
+      for (int q = 0; q < S; ++q) x += ld_cluster(part + c * kTM + tid, q);
       if (m < g.M && n0 + c < g.N) put_out<EPI>(g, m, n0 + c, x);
     }
     __syncwarp();

@@ -121,10 +121,6 @@ __device__ __forceinline__ void st_remote(unsigned addr, float2 v) {
   asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(v.x), "f"(v.y)
                : "memory");
 }
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 
 __device__ __forceinline__ void workers_sync(int W) {
   asm volatile("bar.sync 1, %0;" ::"r"(W) : "memory");

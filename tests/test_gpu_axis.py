@@ -1,8 +1,10 @@
 """Transforms along y and z of the pruned DFT: lines that come as partial sums over slices of x (the
-split modes on rows of more than 128 voxels).
+split modes on rows of more than 128 voxels), and long sums for few results (blocks of a cluster
+share them).
 
-Tolerance of the split modes as in test_gpu_parity.py (3e-5: two-term operands and FP32
-accumulation along x, amplified by the fixed-point map).
+Tolerances as in test_gpu_parity.py: FP32 1e-5 for the strain field and 1e-6 for the homogenised
+stress, split modes 3e-5 (two-term operands and FP32 accumulation along x, amplified by the
+fixed-point map).
 """
 
 import numpy as np
@@ -42,3 +44,12 @@ def check(lib, shape, phases, K, eps_tol, sbar_tol, **opts):
 def test_slices_of_x(lib, prec, shape, K):
     """Two to nine slices, few and many rows of the pattern, 2D and 3D."""
     check(lib, shape, j2_phases(), K, SPLIT_TOL, SPLIT_TOL, precision=prec)
+
+
+@pytest.mark.parametrize("shape,K", [((2000, 7), 1), ((2000, 7), 30), ((1025, 5), 11), ((255, 40), 3),
+                                     ((130, 5), 650), ((131, 3), 393), ((700, 3, 4), 25),
+                                     ((3, 520, 2), 9)])
+def test_long_sums_for_few_results(lib, shape, K):
+    """Two to eight blocks per cluster, shares of unequal length, both directions (the full sets
+    make the inverse's sum the long one)."""
+    check(lib, shape, elastic_phases(), K, EPS_TOL, SBAR_TOL)
