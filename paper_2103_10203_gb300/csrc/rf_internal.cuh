@@ -137,8 +137,9 @@ struct rf_ctx {
   long long K = 0, Kh = 0;
   int Kx = 0, Ky = 0, Kz = 0;
   std::vector<int32_t> pat;       // [K][3] as given
-  int32_t* d_pmap = nullptr;      // per pattern entry: half index h, or ~h for the conjugate of h
-  float2* d_red = nullptr;        // [K][6] coefficients in the pattern's order (on demand)
+  // per pattern entry: half index h, or ~h for the conjugate of h
+  std::vector<int32_t> h_pmap;
+  int32_t* d_pmap = nullptr;
   std::vector<long long> h_src;   // per half entry: a pattern entry equal to it
   int* d_kx = nullptr;   // kx values (>= 0)
   int* d_kym = nullptr;  // ky values mod Ny
@@ -441,7 +442,7 @@ int launch_reset_er(rf_ctx* c, const double* ebar6, double scale_old);
 int launch_warm_project(rf_ctx* c, const float2* d_warm6, const double* ebar6);
 int launch_phase_hist(rf_ctx* c, unsigned long long* d_hist);
 int launch_scatter_full(rf_ctx* c, rf_ctx* full);
-int launch_gather_pattern(rf_ctx* c);
+int launch_gather_pattern(rf_ctx* c, long long p0, long long n, float2* out);
 int launch_law_sweep(rf_ctx* c, const float* eps, float* tau, float* sig);
 constexpr int kErrBlocks = 304;
 int launch_stress_errors(rf_ctx* c, const float* sig_ref, const double* sbar,

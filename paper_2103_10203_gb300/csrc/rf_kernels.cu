@@ -501,9 +501,10 @@ __global__ void k_gather_pattern(const float2* ER, const HIdx* hidx, const int32
   out[t] = v;
 }
 
-int launch_gather_pattern(rf_ctx* c) {
-  k_gather_pattern<<<(unsigned)((6 * c->K + 255) / 256), 256, 0, c->stream>>>(
-      c->d_ER, c->d_hidx, c->d_pmap, c->K, c->nc, c->Kx, c->Ky, c->d_red);
+// n entries of the pattern from entry p0 on
+int launch_gather_pattern(rf_ctx* c, long long p0, long long n, float2* out) {
+  k_gather_pattern<<<(unsigned)((6 * n + 255) / 256), 256, 0, c->stream>>>(
+      c->d_ER, c->d_hidx, c->d_pmap + p0, n, c->nc, c->Kx, c->Ky, out);
   return launch_check(c, "gather pattern");
 }
 
