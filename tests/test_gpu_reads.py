@@ -64,3 +64,40 @@ def test_reading_coefficients_between_solves(lib, shape, full, opts):
     want = np.stack([r.eps_hat[:, i, j] for (i, j) in O.rf_oracle.VOIGT], axis=1)
     tol = 3e-5 if "precision" in opts else 1e-5   # as in test_gpu_parity.py
     assert np.linalg.norm(co[..., 0] + 1j * co[..., 1] - want) <= tol * np.linalg.norm(want)
+
+
+def test_network_reads_need_no_device_memory_and_share_nothing(lib):
+    """Parameters and gradients of 1024 hidden units (5.4 MB), read by two threads at once."""
+    import threading
+
+    import torch
+    net = lib.WarmStartNet(1024, 8)
+    flat = np.random.default_rng(1).standard_normal(net.dims["n_params"]).astype(np.float32)
+    net.rf_mlp_set_params(flat)
+    before = torch.cuda.mem_get_info()[0]
+    assert np.array_equal(net.rf_mlp_get_params(), flat)
+    assert before - torch.cuda.mem_get_info()[0] < 2 << 20
+    bad = []
+
+    def read(f, want):
+        for _ in range(20):
+            if not np.array_equal(f(), want):
+                bad.append(f.__name__)
+
+    ts = [threading.Thread(target=read, args=(net.rf_mlp_get_params, flat)),
+          threading.Thread(target=read, args=(net.rf_mlp_get_grads, np.zeros_like(flat)))]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    net.close()
+    assert not bad
+
+
+@pytest.mark.parametrize("H", [16, 48, 512])
+def test_network_parameters_round_trip(lib, H):
+    net = lib.WarmStartNet(H, 8)
+    flat = np.arange(net.dims["n_params"], dtype=np.float32)
+    net.rf_mlp_set_params(flat)
+    assert np.array_equal(net.rf_mlp_get_params(), flat)
+    net.close()
