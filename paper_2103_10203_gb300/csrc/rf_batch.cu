@@ -2271,10 +2271,13 @@ int autotune(rf_batch* b, const double* macro) {
   // three-update solve each way (the sweeps without their final pass, the resident kernel with)
   b->resident = 0;
   b->cell = 0;
-  if (!err && b->res_ok && b->opt.batch_resident > 0) b->resident = 1;
-  // the cell-resident solve (pruned DFTs) against the sweeps in the same way, unless -1
-  const bool try_res = b->res_ok && b->opt.batch_resident == 0;
-  if (!err && (try_res || b->cell_smem > 0)) {
+  if (!err && b->opt.batch_resident > 0) {
+    b->resident = b->res_ok ? 1 : 0;
+    b->cell = b->cell_smem > 0 ? 1 : 0;
+  }
+  // (no batch qualifies for both: kb_resident takes FFT sides, kb_cell pruned DFTs)
+  const bool try_res = b->res_ok;
+  if (!err && b->opt.batch_resident == 0 && (try_res || b->cell_smem > 0)) {
     auto time_solve = [&](bool res, float* ms) -> int {
       *ms = 1e30f;
       for (int rep = 0; rep < 2; ++rep) {
