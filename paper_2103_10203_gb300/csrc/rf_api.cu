@@ -911,12 +911,9 @@ int rf_set_pattern(rf_ctx* c, const int32_t* freqs, int64_t K) {
     if (!err) err = palloc(c, &c->d_jent, jlist.size(), "pattern");
     if (!err) err = palloc(c, &c->d_jn, jlist.size(), "pattern");
     if (!err)
-      err = ck(cudaMemcpy(c->d_jptr, jptr.data(), sizeof(int) * jptr.size(), cudaMemcpyHostToDevice),
-               "up");
+      err = ck(upload(c->d_jptr, jptr.data(), sizeof(int) * jptr.size(), c->stream), "up");
     if (!err)
-      err = ck(cudaMemcpy(c->d_jlist, jlist.data(), sizeof(int) * jlist.size(),
-                          cudaMemcpyHostToDevice),
-               "up");
+      err = ck(upload(c->d_jlist, jlist.data(), sizeof(int) * jlist.size(), c->stream), "up");
   }
   if (!err) err = palloc(c, &c->d_counter, 1, "counter");
   if (!err) err = ck(cudaMemsetAsync(c->d_counter, 0, sizeof(unsigned), c->stream), "memset");

@@ -1906,8 +1906,8 @@ int build_col_items(rf_batch* b) {
       return e;
     b->n_items[st] = (int)lists[q]->size();
     if (!lists[q]->empty()) {
-      cudaError_t e = cudaMemcpy(b->d_items[st], lists[q]->data(),
-                                 sizeof(int2) * lists[q]->size(), cudaMemcpyHostToDevice);
+      cudaError_t e = upload(b->d_items[st], lists[q]->data(), sizeof(int2) * lists[q]->size(),
+                             b->stream);
       if (e != cudaSuccess) return bfail(e, "batch upload");
     }
   }
@@ -1984,13 +1984,12 @@ int build_row_items(rf_batch* b) {
   }
   b->row_smem = smem;
   cudaError_t e = items.empty() ? cudaSuccess
-                                : cudaMemcpy(b->d_items[1], items.data(),
-                                             sizeof(int2) * items.size(), cudaMemcpyHostToDevice);
+                                : upload(b->d_items[1], items.data(), sizeof(int2) * items.size(),
+                                         b->stream);
   if (e == cudaSuccess && !witems.empty())
-    e = cudaMemcpy(b->d_items[4], witems.data(), sizeof(int2) * witems.size(),
-                   cudaMemcpyHostToDevice);
+    e = upload(b->d_items[4], witems.data(), sizeof(int2) * witems.size(), b->stream);
   if (e == cudaSuccess)
-    e = cudaMemcpy(b->d_desc, b->desc.data(), sizeof(BDesc) * b->n, cudaMemcpyHostToDevice);
+    e = upload(b->d_desc, b->desc.data(), sizeof(BDesc) * b->n, b->stream);
   return e == cudaSuccess ? RF_OK : bfail(e, "batch upload");
 }
 
@@ -2588,13 +2587,13 @@ int rf_batch_create(rf_batch** out, int32_t n_rve, const rf_grid* grids,
   if (!err) err = balloc(&b->d_part, off_part, "batch partials");
   if (!err) err = balloc(&b->d_ndone, 1, "batch");
   if (!err) err = balloc(&b->d_counter, 1, "batch");
-  if (!err && cudaMemset(b->d_counter, 0, sizeof(unsigned)) != cudaSuccess)
+  if (!err && cudaMemsetAsync(b->d_counter, 0, sizeof(unsigned), b->stream) != cudaSuccess)
     err = bfail(cudaGetLastError(), "batch");
   if (!err) err = balloc(&b->d_warm_off, n_rve, "batch");
   b->n_slots = off_h;
   auto up = [&](void* dst, const void* src, size_t bytes) {
     if (err) return;
-    cudaError_t e = cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice);
+    cudaError_t e = upload(dst, src, bytes, b->stream);
     if (e != cudaSuccess) err = bfail(e, "batch upload");
   };
   up(b->d_phase, all_phase.data(), all_phase.size());
@@ -2756,10 +2755,9 @@ int rf_batch_solve(rf_batch* b, const double* macro, const float* const* warm,
               make_float2(warm[r][(p * 6 + i) * 2], warm[r][(p * 6 + i) * 2 + 1]);
       }
     }
-    cudaError_t e = cudaMemcpy(b->d_warm, w6.data(), sizeof(float2) * std::max(total, 1LL),
-                               cudaMemcpyHostToDevice);
+    cudaError_t e = upload(b->d_warm, w6.data(), sizeof(float2) * std::max(total, 1LL), b->stream);
     if (e == cudaSuccess)
-      e = cudaMemcpy(b->d_warm_off, off.data(), sizeof(long long) * b->n, cudaMemcpyHostToDevice);
+      e = upload(b->d_warm_off, off.data(), sizeof(long long) * b->n, b->stream);
     if (e != cudaSuccess) return bfail(e, "batch warm upload");
     use_warm = true;
   }

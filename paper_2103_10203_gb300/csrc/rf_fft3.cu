@@ -75,10 +75,8 @@ int fft3_setup(rf_ctx* c, const int* kym) {
   for (int i = 0; i < c->Ky; ++i) ymap[kym[i]] = (short)i;
   if (int e = palloc(c, &c->d_zrange, range.size(), "pattern")) return e;
   if (int e = palloc(c, &c->d_ymap, ymap.size(), "pattern")) return e;
-  cudaError_t e = cudaMemcpy(c->d_zrange, range.data(), sizeof(int2) * range.size(),
-                             cudaMemcpyHostToDevice);
-  if (e == cudaSuccess)
-    e = cudaMemcpy(c->d_ymap, ymap.data(), sizeof(short) * ymap.size(), cudaMemcpyHostToDevice);
+  cudaError_t e = upload(c->d_zrange, range.data(), sizeof(int2) * range.size(), c->stream);
+  if (e == cudaSuccess) e = upload(c->d_ymap, ymap.data(), sizeof(short) * ymap.size(), c->stream);
   return e == cudaSuccess ? RF_OK : cuda_fail(e, "pattern");
 }
 

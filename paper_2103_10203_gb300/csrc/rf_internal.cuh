@@ -433,6 +433,13 @@ inline int palloc(rf_ctx* c, T** p, size_t n, const char* what) {
   c->pcap[p] = bytes;
   return RF_OK;
 }
+// Copy of a set-up table to the device, there when it returns. On the stream of the kernels that
+// read it: a copy from pageable memory on the legacy stream may still be on its way when the call
+// returns, and a non-blocking stream does not wait for it.
+inline cudaError_t upload(void* dst, const void* src, size_t bytes, cudaStream_t s) {
+  const cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, s);
+  return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
+}
 int launch_iteration(rf_ctx* c);
 int launch_inverse(rf_ctx* c);
 int launch_final(rf_ctx* c, int commit);
