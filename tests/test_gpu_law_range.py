@@ -38,3 +38,38 @@ def test_overflowing_invariant_of_a_yielding_phase_is_an_error(lib, shape, opts)
         s.rf_solve(np.array([1e18, 0, 0, 0, 0, 0]))
     assert e.value.code == -3
     s.close()
+
+
+@pytest.mark.parametrize("shape,opts", KERNELS)
+def test_tiny_yield_stress_does_not_flow_at_rest(lib, shape, opts):
+    """A yield stress below the root of the smallest normal number (1.08e-19): an unstrained cell has
+    no stress, so nothing flows."""
+    ph, pl, _ = indices()
+    ph = ph.copy()
+    ph["sigma_y0"][pl] = 1e-22
+    s = lib.Solver(np.full(shape, pl, np.uint8), ph, pattern=waves(len(shape)), tol=1e-3, max_iter=5,
+                   **opts)
+    s.rf_solve_path(np.zeros((1, 6)))
+    _, sig, alpha = s.rf_get_fields()
+    s.close()
+    assert not alpha.any() and not sig.any()
+
+
+@pytest.mark.parametrize("shape,opts", KERNELS[:7])
+def test_flow_at_tiny_stresses(lib, shape, opts):
+    """A homogeneous cell in shear, its squared invariant near 1e-40 (subnormal, steps of 1.4e-45,
+    1.4e-5 of it at most after four roundings), yield stress half the trial stress: the accumulated
+    plastic strain is (seq - sy) / (3 mu + H), off by at most twice half that."""
+    ph, pl, _ = indices()
+    ph = ph.copy()
+    mu, H = float(ph["mu"][pl]), float(ph["hardening"][pl])
+    seq = 1.2e-20
+    ph["sigma_y0"][pl] = 0.5 * seq
+    e12 = seq / (np.sqrt(3.0) * 2.0 * mu)
+    s = lib.Solver(np.full(shape, pl, np.uint8), ph, pattern=waves(len(shape)), tol=1e-3, max_iter=5,
+                   **opts)
+    s.rf_solve_path(np.array([[0, 0, 0, 0, 0, e12]]))
+    alpha = s.rf_get_fields()[2]
+    s.close()
+    want = 0.5 * seq / (3.0 * mu + H)
+    assert np.abs(alpha - want).max() <= 1e-4 * want
