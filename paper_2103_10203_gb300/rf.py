@@ -236,7 +236,8 @@ def make_options(tol=1e-6, max_iter=1000, green="rotated", ref="minmax", precisi
 def rf_pattern_adapted(phase_map, inclusion_phase, k_target, stream=None):
     pm = np.ascontiguousarray(phase_map, dtype=np.uint8)
     g = make_grid(pm.shape)
-    cap = int(k_target) + 1
+    # (a target beyond the grid is the library's to refuse: no room for it here)
+    cap = min(int(k_target), pm.size) + 1
     out = _host_result((cap, 3), np.int32)
     K = C.c_int64(0)
     _check(lib.rf_pattern_adapted(C.byref(g), _ptr(pm), int(inclusion_phase), int(k_target),
