@@ -135,7 +135,10 @@ typedef struct rf_phase {
  *  fft_row_blocks  FFT mode: run the row kernel on this many blocks with the grid rows spread
  *             evenly (blocks differ by at most one row; clamped to the row count), instead of
  *             tiles of fft_rows; 0 = fft_rows or the autotuner (which also times such
- *             partitions over whole multiples of the SM count).
+ *             partitions over whole multiples of the SM count). With fft_fuse 3 and sides of 32 to
+ *             512, 768 or 1024 (2^b or 3 * 2^b) it asks for a form of the persistent solve: 8 or 16
+ *             = one thread-block cluster of that many blocks, any other number = a co-resident
+ *             grid, each where it fits.
  *  wait_limit  split-precision modes: polls of every bounded mbarrier wait in the tensor-core
  *             kernels before the wait gives up and the solve returns RF_ERR_TIMEOUT (0 = the
  *             library default, 2^26 polls); >= 0.

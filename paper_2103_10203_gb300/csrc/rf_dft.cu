@@ -538,6 +538,8 @@ int launch_row_dft(rf_ctx* c, const int* done, bool final_pass, int commit, int*
   const int nb = (units + a.U - 1) / a.U;
   if (blocks) *blocks = nb;
   const size_t smem = row_dft_smem(a.U, a.Kx, a.np);
+  // beside a grid of a few blocks the next kernel's prologue is free: up to 1 us per update (16 x 16,
+  // 50 x 97), and no cell of 5 to 2000 a side was slower
   a.early = nb <= 32;
   const bool pl = c->has_plastic;
   if (c->nc == 3) {
@@ -585,6 +587,7 @@ int launch_axis_dft(rf_ctx* c, const float2* in, int splits, long long split_str
   a.ranks = 1;
   while (a.ranks < 8 && blocks * 2 * a.ranks <= sms && 2 * a.ranks <= chunks) a.ranks *= 2;
   grid.z *= a.ranks;
+  // as in the row pass: 1 to 2 us per update of cells up to 200 x 190, none slower
   a.early = blocks * a.ranks <= 64;
   const auto kern = wide ? (sign < 0 ? k_axis_dft<4, true> : k_axis_dft<4, false>)
                          : (sign < 0 ? k_axis_dft<2, true> : k_axis_dft<2, false>);

@@ -1274,8 +1274,11 @@ int fft_autotune(rf_ctx* c) {
     // the team kernels where they take the sides (a co-resident grid, or one cluster of 8 or 16
     // blocks), the general persistent kernel otherwise
     int bestCl = -1;
+    // (fft_fuse 3 with fft_row_blocks asks for one of these forms)
+    const int blocks = c->opt.fft_fuse == 3 ? c->opt.fft_row_blocks : 0;
     c->team_on = true;
     for (int cl : {0, 8, 16}) {
+      if (blocks > 0 && cl != (blocks == 8 || blocks == 16 ? blocks : 0)) continue;
       if (err || !team_geometry(c, cl)) continue;
       float ms = 1e30f;
       const int e = time_it([&] {
