@@ -103,7 +103,7 @@ typedef struct rf_phase {
  *  precision  RF_PREC_FP32: FP32 SIMT transforms. RF_PREC_SPLIT_BF16 / RF_PREC_SPLIT_TF32:
  *             the transforms along x run on the tensor cores (tcgen05) with operands split into
  *             hi + lo parts of BF16 or TF32, three products (hi*hi + hi*lo + lo*hi) and FP32
- *             accumulation; the law stays FP32. The residual and the homogenised stress are
+ *             accumulation; those along y and z and the law stay FP32. The residual and the homogenised stress are
  *             accumulated in FP64 in every mode. Split modes need 2 Kx <= 1152.
  *  check_every  iterations launched between host checks of the device convergence flag
  *             (0 = library default). Work after convergence is skipped on the device, so
@@ -120,15 +120,17 @@ typedef struct rf_phase {
  *             (forward y, Green-operator update with the convergence decision, inverse y);
  *             1 one kernel per group of kx columns (steps b to d of Sec. 4 fused); 2 forward y,
  *             then the Green-operator update and decision inside the inverse y kernel; 3 the
- *             persistent solve: one cooperative launch per solve runs every update (row phase,
- *             grid barrier, column phase per kx, grid barrier, decision) with the grid
- *             co-resident (one or two blocks per SM); 4 (Ny = 1024) as 1 on the warp-FFT
+ *             persistent solve: one launch per solve runs every update (row phase, barrier,
+ *             column phase per kx, barrier, decision), a cooperative one with the grid
+ *             co-resident or, for small cells, one thread-block cluster; 4 (Ny = 1024) as 1 on the warp-FFT
  *             column kernel: a warp per line column, the 1024-point transforms along y in
  *             registers (four-step 32 x 32); 5 (1024 x 1024) the persistent solve on the
  *             passes of mode 4 (one cooperative launch per solve, grid barriers between the
  *             passes); 0 = chosen by timing when the pattern is set (the persistent solves only
  *             when fft_rows and fft_row_blocks are 0; modes 4 and 5 on 1024 x 1024 grids). Must
- *             be 0 or -1 in 3D. All give the same update up to the order of FP32 and FP64
+ *             be 0 or -1 in 3D: 0 = four kernels per update on team FFTs where all sides are 2^b or
+ *             3 * 2^b from 32 to 512 and no tile is set (fft_rows, fft_cols, fft_row_blocks), -1 =
+ *             the general kernels. All give the same update up to the order of FP32 and FP64
  *             summation.
  *  fft_fuse_kx  kx columns per block of the fused kernel (0 = chosen by timing; 1..16; 1 or 2
  *             in mode 4; mode 5 uses 2).
@@ -195,7 +197,8 @@ typedef struct rf_info {
   int32_t fft_row_threads;/* FFT mode: threads per row-kernel block, else 0 */
   int32_t fft_cols;       /* FFT mode: columns per column-kernel block, else 0 */
   int32_t fft_col_threads;/* FFT mode: threads per column-kernel block, else 0 */
-  int32_t fft_fused;      /* column-phase mode in use (see fft_fuse): 0 to 5 */
+  int32_t fft_fused;      /* 2D column-phase mode in use (see fft_fuse): 0 to 5; 0 in 3D, where the
+                           * stage times tell the updates on team FFTs (stage 6) */
   int32_t fft_fuse_kx;    /* kx columns per fused block, else 0 */
   int32_t fft_fuse_threads;/* threads per fused block, else 0 */
   int32_t fft_row_blocks; /* FFT mode: row-kernel blocks (fft_rows is the largest block's row
@@ -288,8 +291,8 @@ int rf_get_info(const rf_ctx* ctx, rf_info* info);
  * Stages: 0 inverse transform along z, 1 inverse along y, 2 row kernel (transforms along x,
  * constitutive law, polarization), 3 forward along y, 4 forward along z, 5 Green-operator
  * update with the convergence decision (with fft_fuse 2 it includes the inverse along y),
- * 6 fused column phase (fft_fuse 1: stages 3, 5 and 1 in one kernel), 7 final pass (fields,
- * homogenised stress, commit).
+ * 6 fused column phase (fft_fuse 1: stages 3, 5 and 1 in one kernel; 3D on team FFTs: stages 4, 5
+ * and 0 in one kernel), 7 final pass (fields, homogenised stress, commit).
  * rf_get_stage_times fills ms_total[8] (milliseconds) and counts[8] (launches timed). */
 int rf_set_tracing(rf_ctx* ctx, int on);
 int rf_get_stage_times(const rf_ctx* ctx, double ms_total[8], int64_t counts[8]);
