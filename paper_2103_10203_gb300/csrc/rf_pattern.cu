@@ -6,10 +6,10 @@
 // round(|g^| / |g^(0)| * 2^30) descending, |k|^2 ascending, signed linear index ascending.
 // Pairs are taken whole until at least k_target frequencies are held; the selection threshold
 // is found by radix passes over weighted histograms of the key, each decided on the device by its
-// last block, so the host waits once per pattern.
+// last block, so the host waits twice per pattern: for its size and for its entries.
 // g is real: two rows share a complex transform along x, and only kx = 0 .. Nx / 2 goes on, half
 // the work of transforms that the FP64 rate bounds (96 and 100 us for 1024^2 before). A 1024^2
-// pattern took 1374 us (some 530 us of kernels, 13 host reads, 16 allocations) and takes 562 us.
+// pattern took 1374 us (some 530 us of kernels, 13 host reads, 16 allocations) and takes 540 us.
 // Radial pattern (Sec. 4.1): L equiangular rasterised lines; the same selection machinery
 // ranks pairs by (not on a line, |k|^2, index).
 #include <algorithm>
@@ -611,8 +611,8 @@ int select_and_compact(const Grid3& g, const SelectScratch& ss, long long k_targ
   };
   const Digit digits[] = {{0, 53, 11}, {0, 42, 11}, {0, 33, 9}, {0, 22, 11}, {0, 11, 11},
                           {0, 0, 11},  {1, 20, 11}, {1, 10, 10}, {1, 0, 10}};
-  // a digit above every entry's |k|^2 or lin is zero throughout (two of the nine passes for 1024^2,
-  // 556 us a call with them, 525 without; 64^2 302 and 279)
+  // a digit above every entry's |k|^2 or lin is zero throughout (two of the nine passes for 1024^2:
+  // 31 us less of a call in turn with the nine; 64^2 302 and 279 us)
   const unsigned long long k2max = (unsigned long long)(g.nx / 2) * (g.nx / 2) +
                                    (unsigned long long)(g.ny / 2) * (g.ny / 2) +
                                    (unsigned long long)(g.nz / 2) * (g.nz / 2);
