@@ -638,16 +638,21 @@ __global__ __launch_bounds__(256) void k_law_sweep(const float* __restrict__ eps
 int launch_law_sweep(rf_ctx* c, const float* eps, float* tau, float* sig) {
   int sms = 152;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->dev);
-  const long long n4 = c->N >> 2;
-  const int grid = (int)std::max(1LL, std::min<long long>(8LL * sms, (n4 + 255) / 256));
   const bool pl = c->has_plastic;
-  if (c->nc == 3) {
-    if (pl) k_law_sweep<3, true><<<grid, 256, 0, c->stream>>>(eps, c->d_phase, c->d_state, c->N, c->law, tau, sig);
-    else k_law_sweep<3, false><<<grid, 256, 0, c->stream>>>(eps, c->d_phase, c->d_state, c->N, c->law, tau, sig);
-  } else {
-    if (pl) k_law_sweep<6, true><<<grid, 256, 0, c->stream>>>(eps, c->d_phase, c->d_state, c->N, c->law, tau, sig);
-    else k_law_sweep<6, false><<<grid, 256, 0, c->stream>>>(eps, c->d_phase, c->d_state, c->N, c->law, tau, sig);
-  }
+  const auto k = c->nc == 3 ? (pl ? k_law_sweep<3, true> : k_law_sweep<3, false>)
+                            : (pl ? k_law_sweep<6, true> : k_law_sweep<6, false>);
+  // Eight blocks per SM. Where that is many turns of each, whole waves of what is resident: the J2
+  // kernel's 48 registers hold five blocks per SM, and eight left the second wave 60 % full (4096^2
+  // 107 us, 103 with the four blocks of its 54 registers before; three waves 102). Below ten million
+  // voxels the turns themselves divide unevenly and eight measured better (2048^2 26 and 29 us).
+  const long long want = ((c->N >> 2) + 255) / 256;
+  long long grid = std::min(want, 8LL * sms);
+  int occ = 0;
+  if (want > 64LL * sms &&
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, 256, 0) == cudaSuccess && occ > 0)
+    grid = 3LL * occ * sms;
+  k<<<(unsigned)std::max(1LL, grid), 256, 0, c->stream>>>(eps, c->d_phase, c->d_state, c->N, c->law,
+                                                          tau, sig);
   return launch_check(c, "law sweep");
 }
 
