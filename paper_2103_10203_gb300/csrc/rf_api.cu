@@ -911,7 +911,8 @@ int rf_set_pattern(rf_ctx* c, const int32_t* freqs, int64_t K) {
     if (!err) err = palloc(c, &c->d_jent, jlist.size(), "pattern");
     if (!err) err = palloc(c, &c->d_jn, jlist.size(), "pattern");
     if (!err)
-      err = ck(upload(c->d_jptr, jptr.data(), sizeof(int) * jptr.size(), c->stream), "up");
+      err = ck(cudaMemcpyAsync(c->d_jptr, jptr.data(), sizeof(int) * jptr.size(),
+                               cudaMemcpyHostToDevice, c->stream), "up");   // (the next waits)
     if (!err)
       err = ck(upload(c->d_jlist, jlist.data(), sizeof(int) * jlist.size(), c->stream), "up");
   }

@@ -75,7 +75,9 @@ int fft3_setup(rf_ctx* c, const int* kym) {
   for (int i = 0; i < c->Ky; ++i) ymap[kym[i]] = (short)i;
   if (int e = palloc(c, &c->d_zrange, range.size(), "pattern")) return e;
   if (int e = palloc(c, &c->d_ymap, ymap.size(), "pattern")) return e;
-  cudaError_t e = upload(c->d_zrange, range.data(), sizeof(int2) * range.size(), c->stream);
+  // (the second copy waits for both)
+  cudaError_t e = cudaMemcpyAsync(c->d_zrange, range.data(), sizeof(int2) * range.size(),
+                                  cudaMemcpyHostToDevice, c->stream);
   if (e == cudaSuccess) e = upload(c->d_ymap, ymap.data(), sizeof(short) * ymap.size(), c->stream);
   return e == cudaSuccess ? RF_OK : cuda_fail(e, "pattern");
 }
